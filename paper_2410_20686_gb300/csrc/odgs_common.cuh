@@ -353,6 +353,51 @@ __device__ __forceinline__ float slice_exponent(float4 con, float t, float rowt)
     return __fmaf_rn(__fmul_rn(con.x, t), t, rowt);
 }
 
+// ------------------------------------------------------------------ footprint on a warp's pixels
+// Lanes of a warp cover one rectangle of the tile: 4 PPT columns x 8 rows (four lanes a row, each with
+// PPT pixels four columns apart) where the tile's shape allows it, else whole tile rows. An 8 x 8
+// rectangle meets fewer footprints than a 16 x 4 strip of the same 64 pixels.
+__host__ __device__ __forceinline__ int region_width(int tile_w, int tile_h, int ppt) {
+    return tile_h % 8 == 0 && tile_w % (4 * ppt) == 0 ? 4 * ppt : tile_w;
+}
+
+// A blend warp walks only the list entries whose footprint {d^T conic d <= Qb}, the set the tiles are
+// listed by, meets the rectangle of pixel centres the warp owns. Within the rectangle's rows the
+// footprint spans columns from the slice edge at -ystar to the one at +ystar (each clamped to the
+// rows), as in band_columns, with the same margins (Qb inflated by 1e-4, the edges by 0.01 px): an
+// entry left out has alpha < 1/255 at every pixel of the warp. NaNs count as meeting.
+struct Region {
+    float x0, x1, y0, y1;  // first and last pixel column and row
+};
+__device__ __forceinline__ Region make_region(int x, int w, int y, int h) {
+    return {(float)x, (float)(x + w - 1), (float)y, (float)(y + h - 1)};
+}
+
+// Footprint of a staged entry: (k, ev, ystar, Qb) of make_footprint. An entry with two images in the
+// tile (split by the seam) takes every column.
+__device__ __forceinline__ float4 stage_extent(float4 ra, float4 rb, bool split) {
+    const Footprint f = make_footprint(ra, rb);
+    return make_float4(f.k, f.ev, f.ystar, split ? 1e30f : f.Qb);
+}
+
+// Columns the footprint spans within the region's rows, relative to its centre; false if it misses
+// the rows. gamma from the staged conic's base-2 scaling.
+__device__ __forceinline__ bool region_span(float4 pos, float4 con, float4 ext, const Region& r, float& xmin,
+                                            float& xmax) {
+    const float d0 = fmaxf(r.y0 - pos.y - pos.w, -ext.y), d1 = fminf(r.y1 - pos.y - pos.w, ext.y);
+    const float yr = fminf(fmaxf(ext.z, d0), d1), yl = fminf(fmaxf(-ext.z, d0), d1);
+    const float gk = con.z * (2.f / kLog2e);  // -gamma
+    const float qr = fmaxf(fmaf(yr * yr, gk, ext.w), 0.f), ql = fmaxf(fmaf(yl * yl, gk, ext.w), 0.f);
+    xmax = fmaf(con.y, yr, fmaf(ext.x, fp_sqrt(qr), 0.01f));
+    xmin = fmaf(con.y, yl, -fmaf(ext.x, fp_sqrt(ql), 0.01f));
+    return !(d0 > d1);
+}
+__device__ __forceinline__ bool meets_region(float4 pos, float4 con, float4 ext, const Region& r) {
+    float xmin, xmax;
+    const bool rows = region_span(pos, con, ext, r, xmin, xmax);
+    return rows && !(r.x0 - pos.x - pos.z > xmax) && !(r.x1 - pos.x - pos.z < xmin);
+}
+
 // ------------------------------------------------------------------ saturated-tile truncation
 // A tile's list needs only the entries up to the point where every pixel of the tile has stopped
 // (transmittance below 1e-4): later entries are never evaluated, by the forward or the backward
