@@ -274,16 +274,6 @@ __device__ __forceinline__ void footprint_rows(const Footprint& f, int H, int& j
     jhi = min(H - 1, f.r0 + (int)floorf(__fadd_rn(f.dv, ev)));
 }
 
-// The same rows from the records directly, without the rest of the footprint: the backward blend
-// skips an entry for a warp whose pixel rows all lie outside them (x = jlo, y = jhi). The
-// operations are footprint_rows(make_footprint(ra, rb), H)'s, so the rows are the same.
-__device__ __forceinline__ int2 footprint_row_range(float4 ra, float4 rb, int H) {
-    int c0, r0;
-    unpack_anchor(ra.z, c0, r0);
-    const float ev = fminf(fp_sqrt(fp_div(rb.w, rb.z)), 2.f * (float)H);
-    return make_int2(max(0, r0 + (int)ceilf(__fsub_rn(ra.y, ev))), min(H - 1, r0 + (int)floorf(__fadd_rn(ra.y, ev))));
-}
-
 // Horizontal offset of the slice boundary at vertical offset y (side = +1 right, -1 left).
 __device__ __forceinline__ float slice_edge(const Footprint& f, float y, float side) {
     const float q = fmaxf(__fsub_rn(f.Qb, __fmul_rn(__fmul_rn(y, y), f.iC)), 0.f);
@@ -339,6 +329,13 @@ __device__ __forceinline__ void pixel_offset(float fi, float fj, float fc, float
 __device__ __forceinline__ float alpha_exp2(float p) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(p));
+    return r;
+}
+
+// 1 / x by the hardware's approximate reciprocal (relative error below 2^-22), x a normal number.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 

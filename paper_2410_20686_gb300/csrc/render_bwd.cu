@@ -15,13 +15,18 @@
 // slice centre (the exponent's own variable), dp, dp t and dp t^2 and dL/drgb; with dy the same
 // for all of a thread's pixels, these and dy times the first two and dy^2 times the first are the
 // nine values (sum dp t gives the mean terms free of the cancellation an image-axis form suffers
-// for needle-like Gaussians). The warp sums them over its lanes with a transpose
-// reduction (12 shuffles for 9 values), the CTA over its warps in shared memory; then one thread
-// per entry forms dL/d(u, v, conic, opacity), which are linear in these sums, and adds them to the
-// per-(view, Gaussian) accumulator with three 16-byte vector atomics. A warp whose pixels all stopped before an entry skips it, and so does a warp
-// none of whose pixel rows lies within the entry's footprint rows (the rows the binning lists the
-// Gaussian in; outside them no pixel reaches alpha = 1/255); a warp with a single contributing
-// lane skips the reduction.
+// for needle-like Gaussians). The warp sums them over its lanes (warp_reduce_rows4 where four lanes hold
+// a pixel row, else a transpose reduction of the nine values), the CTA over its warps in shared memory;
+// then one thread per entry forms dL/d(u, v, conic, opacity), which are linear in these sums, and adds
+// them to the per-(view, Gaussian) accumulator with three 16-byte vector atomics.
+//
+// A warp walks only the entries whose footprint meets its pixels and that one of its pixels reached in
+// the forward pass: it tests 32 at a time, one per lane, and takes the ballot's bits from the last.
+// The kernel is bound by instruction issue. Measured with the walk, the row reduction and the
+// exponents formed before the pixels' tests, against a row test of every entry by every warp and the
+// reduction of nine values: 1M Gaussians, one 2048 x 1024 view 696 -> 517 us; 500K Gaussians, 16 views
+// 4369 -> 3265 us; 3M Gaussians, 8 views of 4096 x 2048 11438 -> 8920 us. The walk alone: 585, 3660 and
+// 9920 us; with a mask per pixel slot instead of per warp 597, 3632 and 10865 us.
 #include "odgs_common.cuh"
 #include "odgs_internal.h"
 
@@ -67,29 +72,67 @@ __device__ __forceinline__ float warp_reduce9(const float v[9], int lane, int* v
     return z;
 }
 
-template <int PPT>
+// The warp's nine sums when its lanes hold rows of four (lane = 4 row + column): the six per-lane sums
+// are added over the four lanes of a row first, the products with dy (one value per row) formed by
+// the lane that owns the sum, then the rows are added: 9 shuffles and 13 selects instead of 12 and 22.
+// Returns the lane's share: value index row4_index(lane), if not negative.
+__device__ __forceinline__ float warp_reduce_rows4(float S0, float S1, float S2, float V0, float V1, float V2, float dy,
+                                                   int lane) {
+    const unsigned full = 0xffffffffu;
+    bool up = lane & 1;
+    const float w0 = (up ? V0 : S0) + __shfl_xor_sync(full, up ? S0 : V0, 1);
+    const float w1 = (up ? V1 : S1) + __shfl_xor_sync(full, up ? S1 : V1, 1);
+    const float w2 = (up ? V2 : S2) + __shfl_xor_sync(full, up ? S2 : V2, 1);
+    up = lane & 2;
+    const float x0 = (up ? w1 : w0) + __shfl_xor_sync(full, up ? w0 : w1, 2);  // S0, V0, S1, V1
+    const float b = w2 + __shfl_xor_sync(full, w2, 2);                         // S2, V2, S2, V2
+    const float x1 = dy * x0;
+    const float x2 = (lane & 3) == 0 ? dy * x1 : b;
+    up = lane & 16;
+    const float y0 = (up ? x1 : x0) + __shfl_xor_sync(full, up ? x0 : x1, 16);
+    const float y1 = x2 + __shfl_xor_sync(full, x2, 16);
+    up = lane & 8;
+    float z = (up ? y1 : y0) + __shfl_xor_sync(full, up ? y0 : y1, 8);
+    z += __shfl_xor_sync(full, z, 4);
+    return z;
+}
+__device__ __forceinline__ int row4_index(int lane) {
+    const int q = lane & 3;
+    if (lane & 4) return -1;
+    if ((lane & 24) == 0) return q == 0 ? 0 : (q == 1 ? 6 : (q == 2 ? 1 : 7));  // S0, V0, S1, V1
+    if ((lane & 24) == 16) return q == 0 ? 4 : (q == 2 ? 3 : -1);               // dy S0, dy S1
+    if ((lane & 24) == 8) return q == 0 ? 5 : (q == 1 ? 8 : (q == 2 ? 2 : -1));  // dy^2 S0, V2, S2
+    return -1;
+}
+
+// A staged entry, 80 bytes apart (conflict-free 16-byte accesses of consecutive entries).
+struct StagedBwd {
+    float4 pos, con, col;  // Staged's
+    float4 ext;            // stage_extent's
+    float4 raw;            // a, gamma (slice-form conic), 1 / opacity, item (bits)
+};
+
+template <int PPT, bool ROWS4>
 __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
     extern __shared__ float4 smem[];
     const int B = a.batch;
     const int nwarps = blockDim.x >> 5;
-    float4* s_pos = smem;
-    float4* s_con = smem + B;
-    float4* s_col = smem + 2 * B;
-    float4* s_raw = smem + 3 * B;  // a, beta, gamma (slice-form conic), 1 / opacity
-    int2* s_rows = reinterpret_cast<int2*>(smem + 4 * B);  // pixel rows the footprint reaches
-    float* s_fc2 = reinterpret_cast<float*>(s_rows + B);
-    uint32_t* s_idx = reinterpret_cast<uint32_t*>(s_fc2 + B);
-    float* s_red = reinterpret_cast<float*>(s_idx + B);  // [B][nwarps][9]
+    StagedBwd* s_e = reinterpret_cast<StagedBwd*>(smem);
+    float* s_fc2 = reinterpret_cast<float*>(s_e + B);
+    float* s_red = s_fc2 + B;                                                      // [B][nwarps][9]
+    uint32_t* s_got = reinterpret_cast<uint32_t*>(s_red + (size_t)B * nwarps * 9);  // [nwarps][2]: entries a warp's sums are in s_red for
     __shared__ int s_item;
     __shared__ int s_maxn;
 
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int tw = a.tile_w;
-    const int tpr = tw / PPT;
+    const int rw = region_width(tw, a.tile_h, PPT);
+    const int tpr = rw / PPT;  // threads per pixel row of the warp's region
     // a thread's PPT pixels are tpr columns apart (interleaved), so a footprint a few pixels wide
     // falls in one of each lane's pixel slots rather than in several
-    const int lx0 = tid % tpr, ly = tid / tpr;
-    const int wy0 = (warp << 5) / tpr, wy1 = ((warp << 5) + 31) / tpr;  // the warp's tile rows
+    const int rx0 = (warp % (tw / rw)) * rw, ry0 = (warp / (tw / rw)) * (32 / tpr);
+    const int lx0 = rx0 + lane % tpr, ly = ry0 + lane / tpr;
+    const int slot4 = row4_index(lane);
     uint32_t evals = 0u;
 
     for (;;) {
@@ -117,7 +160,7 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
         // entries past the tile's range (possible only when the lists were rebuilt after a sort
         // that gave up, so that they differ from the forward's) stage as never-blending entries
         const uint32_t rlen = rg.y > rg.x ? rg.y - rg.x : 0u;
-        const int wr0 = ty * a.tile_h + wy0, wr1 = ty * a.tile_h + wy1;
+        const Region reg = make_region(x0 + rx0, rw, ty * a.tile_h + ry0, 32 / tpr);
 
         float T[PPT], Bg[PPT], g0[PPT], g1[PPT], g2[PPT];
         int nl[PPT];
@@ -158,40 +201,41 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
                 float4 ra, rb, rc;
                 gather_records(a.rec_a, a.rec_b, a.rec_c, idx, a.n_items, ra, rb, rc);
                 Staged s = stage_entry(ra, rb, rc, x0, tw, V.W, V.model == 0);
-                s_pos[j] = s.pos;
-                s_con[j] = s.con;
-                s_col[j] = s.col;
+                StagedBwd& e = s_e[j];
+                e.pos = s.pos;
+                e.con = s.con;
+                e.col = s.col;
+                e.ext = stage_extent(ra, rb, s.col.w <= 1e30f);
+                e.raw = make_float4(rb.x, rb.z, ra.w > 0.f ? 1.f / ra.w : 0.f,
+                                    __uint_as_float(idx < a.n_items ? idx : 0u));
                 s_fc2[j] = s.fc2;
-                s_raw[j] = make_float4(rb.x, rb.y, rb.z, ra.w > 0.f ? 1.f / ra.w : 0.f);
-                s_idx[j] = idx < a.n_items ? idx : 0u;
-                s_rows[j] = footprint_row_range(ra, rb, V.H);
                 split |= (s.col.w <= 1e30f);
             }
             const int any_split = __syncthreads_or(split);
-            for (int j = cnt - 1; j >= 0; --j) {
-                const int e = lo + j;
-                float* red = s_red + ((size_t)j * nwarps + warp) * 9;
-                const int2 rows = s_rows[j];
-                // no pixel of this warp reached entry e in the forward pass, or none of its rows is
-                // within the footprint's rows
-                if (e >= wmax || rows.y < wr0 || rows.x > wr1) {
-                    if (lane < 9) red[lane] = 0.f;
-                    continue;
-                }
-                // sums over this thread's pixels of dp, dp t and dp t^2 (dp = dL/d power) and of
-                // dL/drgb; the conic, opacity and mean terms are linear in these and in dy times them,
-                // so the warp reduces them and the CTA pass after the batch forms the terms
-                float S0 = 0.f, S1 = 0.f, S2 = 0.f, V0 = 0.f, V1 = 0.f, V2 = 0.f, dy = 0.f;
-                bool contrib = false;
-                if (e < tmax) {
-                    const float4 P = s_pos[j];
-                    const float4 K = s_con[j];
-                    dy = __fsub_rn(__fsub_rn(fj, P.y), P.w);
+            // back to front, 32 entries at a time: each lane tests one entry against the warp's pixels
+            // and the warp walks those that can reach them and that one of its pixels reached in the forward pass
+            for (int g = (cnt - 1) & ~31; g >= 0; g -= 32) {
+                const int jl = g + lane;
+                unsigned m = __ballot_sync(0xffffffffu, jl < cnt && lo + jl < wmax &&
+                                                            meets_region(s_e[jl].pos, s_e[jl].con, s_e[jl].ext, reg));
+                unsigned got = 0u;
+                while (m) {
+                    const int jb = 31 - __clz(m);
+                    const unsigned bit = 1u << jb;
+                    m ^= bit;
+                    const int j = g + jb, e = lo + j;
+                    // sums over this thread's pixels of dp, dp t and dp t^2 (dp = dL/d power) and of
+                    // dL/drgb; the conic, opacity and mean terms are linear in these and in dy times them,
+                    // so the warp reduces them and the CTA pass after the batch forms the terms
+                    float S0 = 0.f, S1 = 0.f, S2 = 0.f, V0 = 0.f, V1 = 0.f, V2 = 0.f;
+                    bool contrib = false;
+                    const float4 P = s_e[j].pos;
+                    const float4 K = s_e[j].con;
+                    const float4 c = s_e[j].col;
+                    const float dy = __fsub_rn(__fsub_rn(fj, P.y), P.w);
                     float centre, rowt;
                     row_terms(K, P.z, dy, centre, rowt);
-                    // exponents of all PPT pixels first (the forward kernel's exact sequence); t is
-                    // the pixel's offset from the slice centre, dx = t + (centre - du)
-                    float pk[PPT], tk[PPT];
+                    float tk[PPT], pk[PPT];
                     if (!any_split) {
 #pragma unroll
                         for (int k = 0; k < PPT; ++k) {
@@ -199,22 +243,21 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
                             pk[k] = slice_exponent(K, tk[k], rowt);
                         }
                     } else {
-                        const float fsplit = s_col[j].w, fc2 = s_fc2[j];
+                        const float fc2 = s_fc2[j];
 #pragma unroll
                         for (int k = 0; k < PPT; ++k) {
-                            tk[k] = __fsub_rn(__fsub_rn(fik[k], (fik[k] >= fsplit) ? fc2 : P.x), centre);
+                            tk[k] = __fsub_rn(__fsub_rn(fik[k], fik[k] >= c.w ? fc2 : P.x), centre);
                             pk[k] = slice_exponent(K, tk[k], rowt);
                         }
                     }
-                    const float4 c = s_col[j];
 #pragma unroll
                     for (int k = 0; k < PPT; ++k) {
-                        if (e >= nl[k] || pk[k] < kLog2AlphaMin) continue;
+                        if (e >= nl[k] || !(pk[k] >= kLog2AlphaMin)) continue;
+                        const float t = tk[k], p = pk[k];
                         contrib = true;
-                        const float t = tk[k];
-                        const float ar = alpha_exp2(pk[k]);
+                        const float ar = alpha_exp2(p);
                         const float alpha = fminf(kAlphaMax, ar);
-                        const float inv = __fdividef(1.f, __fsub_rn(1.f, alpha));
+                        const float inv = rcp_approx(__fsub_rn(1.f, alpha));
                         const float Tj = T[k] * inv;
                         const float w = alpha * Tj;
                         const float cg = c.x * g0[k] + c.y * g1[k] + c.z * g2[k];
@@ -232,26 +275,24 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
                             S2 = fmaf(dpt, t, S2);
                         }
                     }
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, contrib);
-                if (m == 0u) {
-                    if (lane < 9) red[lane] = 0.f;
-                    continue;
-                }
-                // sum dp, sum dp t, sum dp t^2, sum dp t dy, sum dp dy, sum dp dy^2, dL/drgb
-                const float dyS0 = dy * S0;
-                const float vals[9] = {S0, S1, S2, dy * S1, dyS0, dy * dyS0, V0, V1, V2};
-                if ((m & (m - 1u)) == 0u) {  // one contributing lane: no reduction needed
-                    if (contrib) {
-#pragma unroll
-                        for (int q = 0; q < 9; ++q) red[q] = vals[q];
+                    const unsigned lanes = __ballot_sync(0xffffffffu, contrib);
+                    if (lanes == 0u) continue;
+                    got |= bit;
+                    float* red = s_red + ((size_t)j * nwarps + warp) * 9;
+                    // sum dp, sum dp t, sum dp t^2, sum dp t dy, sum dp dy, sum dp dy^2, dL/drgb
+                    if (ROWS4) {
+                        const float sm = warp_reduce_rows4(S0, S1, S2, V0, V1, V2, dy, lane);
+                        if (slot4 >= 0) red[slot4] = sm;
+                    } else {
+                        const float dyS0 = dy * S0;
+                        const float vals[9] = {S0, S1, S2, dy * S1, dyS0, dy * dyS0, V0, V1, V2};
+                        int vi;
+                        bool ok;
+                        const float sm = warp_reduce9(vals, lane, &vi, &ok);
+                        if (ok) red[vi] = sm;
                     }
-                } else {
-                    int vi;
-                    bool ok;
-                    const float sm = warp_reduce9(vals, lane, &vi, &ok);
-                    if (ok) red[vi] = sm;
                 }
+                if (lane == 0) s_got[2 * warp + (g >> 5)] = got;
             }
             __syncthreads();
             // per entry: the warps' sums added, then the screen-space gradient terms. With (dx, dy) =
@@ -267,16 +308,20 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
                 float q[9];
 #pragma unroll
                 for (int k = 0; k < 9; ++k) q[k] = 0.f;
+                bool some = false;
                 for (int w = 0; w < nwarps; ++w) {
+                    if (!((s_got[2 * w + (jj >> 5)] >> (jj & 31)) & 1u)) continue;
+                    some = true;
                     const float* r = s_red + ((size_t)jj * nwarps + w) * 9;
 #pragma unroll
                     for (int k = 0; k < 9; ++k) q[k] += r[k];
                 }
-                const float4 R = s_raw[jj];  // a, beta, gamma, 1 / o
+                if (!some) continue;
+                const float4 R = s_e[jj].raw;  // a, gamma, 1 / o, item
                 const float du_ = R.x * q[1];
-                const float4 p0 = make_float4(du_, fmaf(R.z, q[4], -R.y * du_), -0.5f * q[2], R.x * q[3]);
-                const float4 p1 = make_float4(-0.5f * q[5], R.w * q[0], q[6], q[7]);
-                float4* dst = a.acc + 3 * (size_t)s_idx[jj];
+                const float4 p0 = make_float4(du_, fmaf(R.y, q[4], -s_e[jj].con.y * du_), -0.5f * q[2], R.x * q[3]);
+                const float4 p1 = make_float4(-0.5f * q[5], R.z * q[0], q[6], q[7]);
+                float4* dst = a.acc + 3 * (size_t)__float_as_uint(R.w);
                 if (p0.x != 0.f || p0.y != 0.f || p0.z != 0.f || p0.w != 0.f) red_add_v4(dst, p0);
                 if (p1.x != 0.f || p1.y != 0.f || p1.z != 0.f || p1.w != 0.f) red_add_v4(dst + 1, p1);
                 if (q[8] != 0.f) red_add_v4(dst + 2, make_float4(q[8], 0.f, 0.f, 0.f));
@@ -290,36 +335,42 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
 }
 
 size_t render_bwd_smem(int batch, int threads) {
-    return (size_t)batch * (4 * sizeof(float4) + sizeof(int2) + sizeof(float) + sizeof(uint32_t)) +
-           (size_t)batch * (threads / 32) * 9 * sizeof(float);
+    return (size_t)batch * (sizeof(StagedBwd) + sizeof(float)) + (size_t)batch * (threads / 32) * 9 * sizeof(float) +
+           (size_t)(threads / 32) * 2 * sizeof(uint32_t);
 }
 
-int render_bwd_occupancy(int tile_w, int tile_h, int batch, int ppt) {
-    if (ppt == 0) return 1;
-    const int threads = tile_w * tile_h / ppt;
-    const size_t sm = render_bwd_smem(batch, threads);
-    int nb = 0;
-    cudaError_t e;
+namespace {
+
+using BwdKernel = void (*)(BwdArgs);
+
+// The kernel for a tile and pixels per thread: four lanes per pixel row have their own reduction.
+BwdKernel bwd_kernel(int tile_w, int tile_h, int ppt) {
+    const bool rows4 = region_width(tile_w, tile_h, ppt) == 4 * ppt;
     switch (ppt) {
-        case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_render_bwd<8>, threads, sm); break;
-        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_render_bwd<4>, threads, sm); break;
-        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_render_bwd<2>, threads, sm); break;
-        default: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_render_bwd<1>, threads, sm); break;
+        case 8: return rows4 ? k_render_bwd<8, true> : k_render_bwd<8, false>;
+        case 4: return rows4 ? k_render_bwd<4, true> : k_render_bwd<4, false>;
+        case 2: return rows4 ? k_render_bwd<2, true> : k_render_bwd<2, false>;
+        case 1: return rows4 ? k_render_bwd<1, true> : k_render_bwd<1, false>;
     }
+    return nullptr;
+}
+
+}  // namespace
+
+int render_bwd_occupancy(int tile_w, int tile_h, int batch, int ppt) {
+    const BwdKernel k = bwd_kernel(tile_w, tile_h, ppt);
+    if (!k) return 1;
+    const int threads = tile_w * tile_h / ppt;
+    int nb = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads, render_bwd_smem(batch, threads));
     return (e == cudaSuccess && nb > 0) ? nb : 1;
 }
 
 cudaError_t launch_render_bwd(const BwdArgs& a, int grid, cudaStream_t st) {
-    const int ppt = a.ppt;
-    if (ppt != 1 && ppt != 2 && ppt != 4 && ppt != 8) return cudaErrorInvalidValue;
-    const int threads = a.tile_w * a.tile_h / ppt;
-    const size_t sm = render_bwd_smem(a.batch, threads);
-    switch (ppt) {
-        case 8: k_render_bwd<8><<<grid, threads, sm, st>>>(a); break;
-        case 4: k_render_bwd<4><<<grid, threads, sm, st>>>(a); break;
-        case 2: k_render_bwd<2><<<grid, threads, sm, st>>>(a); break;
-        default: k_render_bwd<1><<<grid, threads, sm, st>>>(a); break;
-    }
+    const BwdKernel k = bwd_kernel(a.tile_w, a.tile_h, a.ppt);
+    if (!k) return cudaErrorInvalidValue;
+    const int threads = a.tile_w * a.tile_h / a.ppt;
+    k<<<grid, threads, render_bwd_smem(a.batch, threads), st>>>(a);
     return cudaGetLastError();
 }
 
