@@ -122,6 +122,26 @@ odgs_status odgs::check_settings(const odgs_settings* s, odgs_settings* out) {
     return ODGS_OK;
 }
 
+void odgs::fit_pixels_per_thread(odgs_settings* st, const odgs_settings& asked, int total_tiles, int num_sms) {
+    // Fewer pixels per thread give a tile more warps and each of them fewer pixels to miss an entry
+    // with; more share an entry's loads and its reduction over more pixels. A frame of few tiles
+    // leaves SMs idle or waits for its longest lists, so it takes the first. Measured (us) with
+    // 1 / 2 pixels in the forward and 1 / 2 / 4 in the backward blend:
+    //    tiles   300K Gaussians, 20 % at the poles      30K uniform Gaussians
+    //      128   775 / 1600     982 / 1707 / 2494        44 / 58     81 / 105 / 153
+    //      512   420 / 511      690 / 826 / 1660         27 / 33     55 / 60 / 78
+    //     1152   351 / 404      528 / 627 / 1120         38 / 31     77 / 62 / 64
+    //     2048   272 / 366      439 / 558 / 840         52 / 39    107 / 77 / 74
+    //     4608   180 / 196      317 / 332 / 354         93 / 65    187 / 131 / 113
+    //     8192   209 / 199      398 / 361 / 414        146 / 99    294 / 202 / 166
+    // The lines lie at 4 and 24 tiles per SM (608 and 3648): below the first both scenes gain.
+    if (asked.pixels_per_thread == 0)
+        st->pixels_per_thread = pixels_per_thread(st->tile_w, st->tile_h, 0, total_tiles <= 4 * num_sms ? 1 : 2);
+    if (asked.pixels_per_thread_bwd == 0)
+        st->pixels_per_thread_bwd = pixels_per_thread(
+            st->tile_w, st->tile_h, 0, total_tiles <= 4 * num_sms ? 1 : (total_tiles <= 24 * num_sms ? 2 : 4));
+}
+
 odgs_status odgs::build_geometry(const odgs_view* views, int n_views, const odgs_settings& s, int n, Geometry* g,
                                  ViewTable* tab) {
     if (!views || n_views < 1 || n_views > kMaxViews || n < 0) return ODGS_ERR_INVALID_ARG;
@@ -306,6 +326,7 @@ odgs_status odgs_preprocess(odgs_ctx* c, const odgs_gaussians* g, const odgs_vie
     Geometry geo;
     r = build_geometry(views, n_views, st, g->n, &geo, &tab);
     if (r != ODGS_OK) return r;
+    fit_pixels_per_thread(&st, *s, geo.total_tiles, c->num_sms);
     Layout L = make_layout(geo.n_items, geo, truncates(st, geo));
     if (!workspace) return ODGS_ERR_INVALID_ARG;
     if (reinterpret_cast<uintptr_t>(workspace) % kAlign != 0) return ODGS_ERR_INVALID_ARG;

@@ -49,6 +49,8 @@ struct Geometry {
 // kernels load 16 bytes), and the views (sizes, finite poses, camera model) with the per-view
 // device constants and the frame's tile / pixel totals. ODGS_ERR_INVALID_ARG on any violation.
 odgs_status check_settings(const odgs_settings* s, odgs_settings* out);
+// Pixels per thread of a frame whose caller left them to the library (0 in `asked`), by its tiles.
+void fit_pixels_per_thread(odgs_settings* st, const odgs_settings& asked, int total_tiles, int num_sms);
 odgs_status check_gaussians(const odgs_gaussians* g, const odgs_settings& st);
 odgs_status build_geometry(const odgs_view* views, int n_views, const odgs_settings& s, int n, Geometry* g,
                            ViewTable* tab);
@@ -206,8 +208,8 @@ cudaError_t launch_tile_ranges(const uint32_t* keys, const Header* hdr, uint2* r
 
 size_t render_fwd_smem(int batch);
 size_t render_bwd_smem(int batch, int threads);
-// Pixels per thread of a blend kernel: want if valid (0 if not), or for want = 0 `prefer` if it
-// fits the tile, else the largest of 4, 2, 1 that does. The forward prefers 2, the backward 4.
+// Pixels per thread of a blend kernel: want if valid (0 if not), or for want = 0 the smallest of prefer
+// and its doubles that fits the tile, else the largest smaller one that does.
 int pixels_per_thread(int tile_w, int tile_h, int want, int prefer);
 int render_fwd_occupancy(int tile_w, int tile_h, int batch, int ppt);
 int render_bwd_occupancy(int tile_w, int tile_h, int batch, int ppt);

@@ -212,8 +212,9 @@ int pixels_per_thread(int tile_w, int tile_h, int want, int prefer) {
     const int area = tile_w * tile_h;
     auto fits = [&](int p) { return tile_w % p == 0 && (area / p) % 32 == 0 && area / p <= 256; };
     if (want != 0) return (want == 1 || want == 2 || want == 4 || want == 8) && fits(want) ? want : 0;
-    if (fits(prefer)) return prefer;
-    for (int p = 4; p >= 1; p >>= 1)
+    for (int p = prefer; p <= 8; p <<= 1)
+        if (fits(p)) return p;
+    for (int p = prefer >> 1; p >= 1; p >>= 1)
         if (fits(p)) return p;
     return 0;
 }

@@ -81,6 +81,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
         cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return ODGS_ERR_CUDA;
     const int tiles = geo.total_tiles;
+    fit_pixels_per_thread(&st, *s, tiles, num_sms);
     const int key_bits = geo.key_bits;
     const size_t n = (size_t)g->n, pixels = (size_t)W * H;
 

@@ -27,9 +27,9 @@ class RenderSettings:
     bg: tuple = (0.0, 0.0, 0.0)
     recompute_lists: bool = False
     grad_accumulate: bool = False
-    pixels_per_thread: int = 0      # forward blend (0: automatic, 2 where it fits)
+    pixels_per_thread: int = 0      # forward blend (0: chosen by the frame's tiles)
     raw_params: bool = False  # scales are log-scales and opacity logits (activated by the kernels)
-    pixels_per_thread_bwd: int = 0  # backward blend (0: automatic, 4 where it fits)
+    pixels_per_thread_bwd: int = 0  # backward blend (0: chosen by the frame's tiles)
     checked: bool = False  # flag (ODGS_DEV_NONFINITE) and cull non-finite parameters / gradients
     full_lists: bool = False  # keep whole tile lists (default: cut after the tile saturates; same results)
 
