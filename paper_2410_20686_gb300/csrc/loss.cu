@@ -6,16 +6,21 @@
 // 11-tap Gaussian). Because every moment is a correlation with g, which is symmetric,
 //   dSSIM_mean / dx_p = (g * A)_p + 2 x_p (g * B)_p + y_p (g * C)_p,
 //   A = c (ds/dmx - 2 mx ds/dsxx - my ds/dsxy),  B = c ds/dsxx,  C = c ds/dsxy.
-//   k_ssim_fwd    per 32 x 32 tile and channel: the image and target with a 5-pixel halo in shared
-//                 memory (cp.async, double-buffered: the next channel loads while this one computes), a horizontal then a vertical 11-tap pass for the five moments (each thread
-//                 computes 4 outputs from the 14 inputs it loads once), then s, the loss partial
-//                 and the maps A, B, C (scratch)
-//   k_ssim_bwd    the same tiling over A, B, C: two passes, then the gradient with the L1 term
+//   k_ssim_fwd    a warp streams down a strip of 64 columns (two per lane): per row the horizontal
+//                 11-tap sums of the five moments from a row buffer in shared memory (a ring of eight
+//                 rows filled by cp.async), then the vertical sums as a FIR filter in transposed form
+//                 in registers (ten pending sums per moment and column), so that each finished row
+//                 gives s, the loss partial and the maps A, B, C (scratch) with no second pass
+//                 over shared memory and no barrier but the warp's
+//   k_ssim_bwd    the same over A, B, C, then the gradient with the L1 term
+// Measured at 2048 x 1024 against 32 x 32 tiles with both passes in shared memory: 104 -> 56 us and
+// 121 -> 43 us. The rows in registers instead of the ring, one ahead: 74 and 82 us.
 //   k_l1          lambda = 0: the L1 term alone, one pass
 //   k_loss_reduce one CTA: the CTAs' partials in a fixed order (deterministic)
 // Rows outside the image are zero (zero padding); columns wrap around the seam or are zero.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -25,11 +30,10 @@ namespace {
 
 constexpr int kR = 5;
 constexpr int kWin = 2 * kR + 1;
-constexpr int kTX = 32, kTY = 32;
-constexpr int kInW = kTX + 2 * kR, kInH = kTY + 2 * kR;
-constexpr int kLd = kInW + 1;  // odd row stride of the input tiles: rows of a warp hit distinct banks
-constexpr int kHd = kTX + 1;   // row stride of the horizontal pass's output
-constexpr int kCB = 4;         // outputs per thread in each pass (register blocking)
+constexpr int kTaps = 2 * kR;   // pending vertical sums per moment and column
+constexpr int kCols = 64;       // columns of a warp's strip
+constexpr int kRow = kCols + 2 * kR + 2;  // row buffer, padded to whole 16-byte reads
+constexpr int kRing = 8;        // rows in flight per warp: a row takes an SM less time than a load
 constexpr int kThreads = 256;
 constexpr float kC1 = 0.01f * 0.01f, kC2 = 0.03f * 0.03f;
 
@@ -37,9 +41,12 @@ struct LossArgs {
     const float* x;
     const float* y;
     float* grad;
-    float* maps;     // [3 channels][3 maps A, B, C][H][W]
+    float2* ab;      // maps A, B: [3 channels][H][pitch]
+    float* c;        // map C: [3 channels][H][pitch]
     float* partial;  // [CTAs]
     int W, H, wrap, area;
+    int pitch;                // row stride of the maps: W rounded up to whole 16-byte groups
+    int strips, segs, rows;   // strips of kCols columns, segments of `rows` rows
     float lam, inv_wsum;
     float g[kWin];
 };
@@ -49,32 +56,85 @@ __device__ __forceinline__ float row_weight(const LossArgs& a, int j) {
     return a.area ? sinpif(((float)j + 0.5f) / (float)a.H) : 1.f;
 }
 
-// Copies rows [y0 - kR, y0 + kTY + kR) x columns [x0 - kR, x0 + kTX + kR) of src into dst with
-// asynchronous 4-byte copies (cp.async; zero-filled outside the image): the caller commits the
-// group and waits for it later, so the copy overlaps the previous channel's passes.
-__device__ __forceinline__ void load_halo_async(const LossArgs& a, const float* __restrict__ src, float (*dst)[kLd],
-                                                int x0, int y0) {
-    for (int i = threadIdx.x; i < kInH * kInW; i += kThreads) {
-        const int r = i / kInW, q = i - r * kInW;
-        const int gy = y0 + r - kR;
-        int gx = x0 + q - kR;
-        bool ok = gy >= 0 && gy < a.H;
-        if (a.wrap) {  // gx lies in [-5, W + 36]: one wrap unless the image is narrower than that
-            if (gx < 0) gx += a.W;
-            else if (gx >= a.W) gx -= a.W;
-            if (gx < 0 || gx >= a.W) gx = ((gx % a.W) + a.W) % a.W;
-        } else {
-            ok = ok && gx >= 0 && gx < a.W;
-        }
-        const float* g = ok ? src + (size_t)gy * a.W + gx : src;
-        const unsigned d = (unsigned)__cvta_generic_to_shared(&dst[r][q]);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(g), "r"(ok ? 4 : 0) : "memory");
-    }
+// Two single-precision operations in one instruction, each half rounded as the scalar one. The window
+// sums of (x, y), of (x^2, y^2) and of the maps (A, B) run in pairs.
+__device__ __forceinline__ unsigned long long pack2(float2 v) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
 }
 
-__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Asynchronous copies into shared memory, zero-filled where !ok.
+__device__ __forceinline__ void copy4(float* dst, const float* src, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void copy8(float2* dst, const float2* src, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
-__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// One row's horizontal sum h enters the vertical filter; returns the finished sum, of the row kR rows
+// earlier (transposed form: each pending sum takes its tap of h and moves down by one).
+__device__ __forceinline__ float2 fir_step(float2 (&acc)[kTaps], float2 h, const float* g) {
+    const float2 out = fma2(make_float2(g[0], g[0]), h, acc[0]);
+#pragma unroll
+    for (int i = 0; i < kTaps - 1; ++i) acc[i] = fma2(make_float2(g[i + 1], g[i + 1]), h, acc[i + 1]);
+    acc[kTaps - 1] = mul2(make_float2(g[kTaps], g[kTaps]), h);
+    return out;
+}
+__device__ __forceinline__ float fir_step(float (&acc)[kTaps], float h, const float* g) {
+    const float out = fmaf(g[0], h, acc[0]);
+#pragma unroll
+    for (int i = 0; i < kTaps - 1; ++i) acc[i] = fmaf(g[i + 1], h, acc[i + 1]);
+    acc[kTaps - 1] = g[kTaps] * h;
+    return out;
+}
+
+// The strip, segment and channel of a warp (one per CTA), and the columns its lanes load: lane + 32 q
+// from the strip's first less kR, wrapped or -1 (zero) outside the image.
+struct Strip {
+    int x0, y0, y1, ch;
+    int col[3];
+};
+__device__ __forceinline__ Strip make_strip(const LossArgs& a, int lane) {
+    Strip s;
+    int k = blockIdx.x;
+    s.x0 = (k % a.strips) * kCols;
+    k /= a.strips;
+    s.y0 = (k % a.segs) * a.rows;
+    s.ch = k / a.segs;
+    s.y1 = min(s.y0 + a.rows, a.H);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        int x = s.x0 - kR + lane + 32 * q;
+        if (a.wrap) {
+            x = ((x % a.W) + a.W) % a.W;
+        } else if (x < 0 || x >= a.W) {
+            x = -1;
+        }
+        s.col[q] = lane + 32 * q < kCols + 2 * kR ? x : -1;
+    }
+    return s;
+}
 
 __device__ __forceinline__ float block_sum(float v, float* s_red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -86,199 +146,219 @@ __device__ __forceinline__ float block_sum(float v, float* s_red) {
     return t;
 }
 
-// Forward: per channel, the 11-tap passes with register blocking (a thread computes kCB outputs
-// from the kCB + 10 inputs it loads once), then SSIM, the loss partial and the maps A, B, C.
-__global__ void __launch_bounds__(kThreads) k_ssim_fwd(LossArgs a) {
-    // dynamic shared memory (above the 48 KB static limit): input tiles double-buffered over the
-    // channels, then the horizontal pass's five moments
-    extern __shared__ float s_dyn[];
-    float (*s_xb)[kInH][kLd] = reinterpret_cast<float (*)[kInH][kLd]>(s_dyn);
-    float (*s_yb)[kInH][kLd] = s_xb + 2;
-    float (*s_h)[kInH][kHd] = reinterpret_cast<float (*)[kInH][kHd]>(s_yb + 2);
-    __shared__ float s_red[kThreads / 32];
-    const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY;
+// Forward: loss partials and the maps A, B, C. 11 taps x 5 moments x 2 passes per value; a lane's two
+// columns share the row buffer's reads and the products.
+__global__ void __launch_bounds__(32) k_ssim_fwd(LossArgs a) {
+    __shared__ __align__(16) float2 s_row[kRing][kRow];
+    const int lane = threadIdx.x;
+    const Strip st = make_strip(a, lane);
     const size_t HW = (size_t)a.W * a.H;
-    float part = 0.f;
-    load_halo_async(a, a.x, s_xb[0], x0, y0);
-    load_halo_async(a, a.y, s_yb[0], x0, y0);
-    async_commit();
-    for (int c = 0; c < 3; ++c) {
-        if (c < 2) {  // the next channel's tiles load while this one computes
-            load_halo_async(a, a.x + (c + 1) * HW, s_xb[(c + 1) & 1], x0, y0);
-            load_halo_async(a, a.y + (c + 1) * HW, s_yb[(c + 1) & 1], x0, y0);
-            async_commit();
-            async_wait<1>();
-        } else {
-            async_wait<0>();
+    const float* __restrict__ px = a.x + st.ch * HW;
+    const float* __restrict__ py = a.y + st.ch * HW;
+    float2 m1[2][kTaps], m2[2][kTaps];  // pending sums of (x, y) and (x^2, y^2)
+    float m3[2][kTaps];                 // of xy
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < kTaps; ++i) {
+            m1[j][i] = m2[j][i] = make_float2(0.f, 0.f);
+            m3[j][i] = 0.f;
         }
-        __syncthreads();
-        float (*s_x)[kLd] = s_xb[c & 1];
-        float (*s_y)[kLd] = s_yb[c & 1];
-        // horizontal: rows [0, kInH) x output columns [0, kTX); lanes take consecutive rows
-        for (int it = threadIdx.x; it < kInH * (kTX / kCB); it += kThreads) {
-            const int r = it % kInH, q0 = (it / kInH) * kCB;
-            float o[5][kCB];
+    const int gx = st.x0 + 2 * lane;
+    const int r0 = max(st.y0 - kR, 0), rend = st.y1 + kR;
+    auto fetch = [&](int r) {  // row r, interleaved (x, y)
+        float2* row = s_row[r % kRing];
 #pragma unroll
-            for (int m = 0; m < 5; ++m)
+        for (int q = 0; q < 3; ++q) {
+            if (32 * q + lane >= kRow) continue;
+            const bool ok = st.col[q] >= 0 && r < a.H && r < rend;
+            const size_t o = ok ? (size_t)r * a.W + st.col[q] : 0;
+            copy4(&row[32 * q + lane].x, px + o, ok);
+            copy4(&row[32 * q + lane].y, py + o, ok);
+        }
+        copy_commit();
+    };
+    for (int k = 0; k < kRing - 1; ++k) fetch(r0 + k);
+    float part = 0.f, wv = 0.f, wo = 0.f;  // row weights of 32 loaded and of 32 finished rows
+    for (int r = r0; r < rend; ++r) {
+        const float2* row = s_row[r % kRing];
+        copy_wait<kRing - 2>();
+        __syncwarp();  // row r is in place, and every lane is done with the row the next copy replaces
+        fetch(r + kRing - 1);
+        // horizontal sums of columns gx and gx + 1: 12 inputs
+        float2 h1[2], h2[2];
+        float h3[2];
 #pragma unroll
-                for (int j = 0; j < kCB; ++j) o[m][j] = 0.f;
+        for (int j = 0; j < 2; ++j) {
+            h1[j] = h2[j] = make_float2(0.f, 0.f);
+            h3[j] = 0.f;
+        }
+        float2 centre[2];
 #pragma unroll
-            for (int i = 0; i < kCB + 2 * kR; ++i) {
-                const float xv = s_x[r][q0 + i], yv = s_y[r][q0 + i];
-                const float xx = xv * xv, yy = yv * yv, xy = xv * yv;
+        for (int i = 0; i < kWin + 1; i += 2) {
+            const float4 v4 = *reinterpret_cast<const float4*>(row + 2 * lane + i);
 #pragma unroll
-                for (int j = 0; j < kCB; ++j) {
-                    const int k = i - j;
+            for (int e = 0; e < 2; ++e) {
+                const float2 v = e ? make_float2(v4.z, v4.w) : make_float2(v4.x, v4.y);
+                const float2 vv = mul2(v, v);
+                const float xy = v.x * v.y;
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int k = i + e - j;
                     if (k < 0 || k >= kWin) continue;
-                    const float gk = a.g[k];
-                    o[0][j] = fmaf(gk, xv, o[0][j]);
-                    o[1][j] = fmaf(gk, yv, o[1][j]);
-                    o[2][j] = fmaf(gk, xx, o[2][j]);
-                    o[3][j] = fmaf(gk, yy, o[3][j]);
-                    o[4][j] = fmaf(gk, xy, o[4][j]);
+                    const float2 gk = make_float2(a.g[k], a.g[k]);
+                    h1[j] = fma2(gk, v, h1[j]);
+                    h2[j] = fma2(gk, vv, h2[j]);
+                    h3[j] = fmaf(a.g[k], xy, h3[j]);
+                    if (k == kR) centre[j] = v;
                 }
             }
-#pragma unroll
-            for (int m = 0; m < 5; ++m)
-#pragma unroll
-                for (int j = 0; j < kCB; ++j) s_h[m][r][q0 + j] = o[m][j];
         }
-        __syncthreads();
-        // vertical: output rows [r0, r0 + kCB) of column q; lanes take consecutive columns
-        for (int it = threadIdx.x; it < kTX * (kTY / kCB); it += kThreads) {
-            const int q = it % kTX, r0 = (it / kTX) * kCB;
-            float o[5][kCB];
+        if (r >= st.y0 && r < st.y1) {  // the L1 term of this row
+            if (((r - st.y0) & 31) == 0) wv = row_weight(a, r + lane);
+            const float w = __shfl_sync(0xffffffffu, wv, (r - st.y0) & 31);
+            float d = 0.f;
 #pragma unroll
-            for (int m = 0; m < 5; ++m)
-#pragma unroll
-                for (int j = 0; j < kCB; ++j) o[m][j] = 0.f;
-#pragma unroll
-            for (int i = 0; i < kCB + 2 * kR; ++i) {
-                float h[5];
-#pragma unroll
-                for (int m = 0; m < 5; ++m) h[m] = s_h[m][r0 + i][q];
-#pragma unroll
-                for (int j = 0; j < kCB; ++j) {
-                    const int k = i - j;
-                    if (k < 0 || k >= kWin) continue;
-                    const float gk = a.g[k];
-#pragma unroll
-                    for (int m = 0; m < 5; ++m) o[m][j] = fmaf(gk, h[m], o[m][j]);
-                }
-            }
-            const int gx = x0 + q;
-#pragma unroll
-            for (int j = 0; j < kCB; ++j) {
-                const int gy = y0 + r0 + j;
-                if (gy >= a.H || gx >= a.W) continue;
-                const float mx = o[0][j], my = o[1][j];
-                const float sxx = o[2][j] - mx * mx, syy = o[3][j] - my * my, sxy = o[4][j] - mx * my;
-                const float A1 = 2.f * mx * my + kC1, A2 = 2.f * sxy + kC2;
-                const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
-                const float iB1 = 1.f / B1, iB2 = 1.f / B2;
-                const float sv = A1 * A2 * iB1 * iB2;
-                const float ds_dmx = 2.f * A2 * (my * B1 - mx * A1) * iB1 * iB1 * iB2;
-                const float ds_dsxx = -sv * iB2;
-                const float ds_dsxy = 2.f * A1 * iB1 * iB2;
-                const float xv = s_x[r0 + j + kR][q + kR], yv = s_y[r0 + j + kR][q + kR];
-                const float w = row_weight(a, gy) * a.inv_wsum;
-                part = fmaf(w, (1.f - a.lam) * fabsf(xv - yv) + a.lam * (1.f - sv), part);
-                float* mp = a.maps + (size_t)(3 * c) * HW + (size_t)gy * a.W + gx;
-                mp[0] = w * (ds_dmx - 2.f * mx * ds_dsxx - my * ds_dsxy);
-                mp[HW] = w * ds_dsxx;
-                mp[2 * HW] = w * ds_dsxy;
-            }
+            for (int j = 0; j < 2; ++j) d += gx + j < a.W ? fabsf(centre[j].x - centre[j].y) : 0.f;
+            part = fmaf(w * a.inv_wsum * (1.f - a.lam), d, part);
         }
-        __syncthreads();  // the next channel overwrites the tiles
+        const int y = r - kR;
+        const bool done = y >= st.y0;  // warp-uniform
+        if (done && ((y - st.y0) & 31) == 0) wo = row_weight(a, y + lane);
+        const float w = __shfl_sync(0xffffffffu, wo, (y - st.y0) & 31) * a.inv_wsum;
+        float oa[2], ob[2], oc[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 m = fir_step(m1[j], h1[j], a.g), s = fir_step(m2[j], h2[j], a.g);
+            const float e = fir_step(m3[j], h3[j], a.g);
+            const float mx = m.x, my = m.y;
+            const float sxx = s.x - mx * mx, syy = s.y - my * my, sxy = e - mx * my;
+            const float A1 = 2.f * mx * my + kC1, A2 = 2.f * sxy + kC2;
+            const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
+            const float iB = 1.f / (B1 * B2), iB1 = B2 * iB, iB2 = B1 * iB;
+            const float sv = A1 * A2 * iB;
+            const float ds_dmx = 2.f * A2 * (my * B1 - mx * A1) * iB1 * iB;
+            const float ds_dsxx = -sv * iB2;
+            const float ds_dsxy = 2.f * A1 * iB;
+            if (done && gx + j < a.W) part = fmaf(w * a.lam, 1.f - sv, part);
+            oa[j] = w * (ds_dmx - 2.f * mx * ds_dsxx - my * ds_dsxy);
+            ob[j] = w * ds_dsxx;
+            oc[j] = w * ds_dsxy;
+        }
+        if (done && gx < a.W) {  // the pitch leaves room for a last odd column's pair
+            const size_t o = ((size_t)st.ch * a.H + y) * a.pitch + gx;
+            *reinterpret_cast<float4*>(a.ab + o) = make_float4(oa[0], ob[0], oa[1], ob[1]);
+            *reinterpret_cast<float2*>(a.c + o) = make_float2(oc[0], oc[1]);
+        }
     }
-    const float t = block_sum(part, s_red);
-    if (threadIdx.x == 0) a.partial[blockIdx.y * gridDim.x + blockIdx.x] = t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (lane == 0) a.partial[blockIdx.x] = part;
 }
 
-// Backward: the same blocked passes over the maps A, B, C, then the gradient with the L1 term.
-__global__ void __launch_bounds__(kThreads) k_ssim_bwd(LossArgs a) {
-    // dynamic shared memory: the three maps' tiles double-buffered over the channels, then the
-    // horizontal pass's outputs
-    extern __shared__ float s_dyn[];
-    float (*s_mb)[3][kInH][kLd] = reinterpret_cast<float (*)[3][kInH][kLd]>(s_dyn);
-    float (*s_h)[kInH][kHd] = reinterpret_cast<float (*)[kInH][kHd]>(s_mb + 2);
-    const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY;
+// Backward: the same streaming sums over the maps A, B, C, then the gradient with the L1 term.
+__global__ void __launch_bounds__(32) k_ssim_bwd(LossArgs a) {
+    __shared__ __align__(16) float2 s_row[kRing][kRow];
+    __shared__ __align__(16) float s_c[kRing][kRow];
+    __shared__ __align__(16) float s_x[kRing][kCols], s_y[kRing][kCols];  // the image rows being finished
+    const int lane = threadIdx.x;
+    const Strip st = make_strip(a, lane);
     const size_t HW = (size_t)a.W * a.H;
-    for (int k = 0; k < 3; ++k) load_halo_async(a, a.maps + (size_t)k * HW, s_mb[0][k], x0, y0);
-    async_commit();
-    for (int c = 0; c < 3; ++c) {
-        if (c < 2) {  // the next channel's maps load while this one computes
-            for (int k = 0; k < 3; ++k)
-                load_halo_async(a, a.maps + (size_t)(3 * (c + 1) + k) * HW, s_mb[(c + 1) & 1][k], x0, y0);
-            async_commit();
-            async_wait<1>();
-        } else {
-            async_wait<0>();
+    const float2* __restrict__ pab = a.ab + (size_t)st.ch * a.H * a.pitch;
+    const float* __restrict__ pc = a.c + (size_t)st.ch * a.H * a.pitch;
+    const float* __restrict__ px = a.x + st.ch * HW;
+    const float* __restrict__ py = a.y + st.ch * HW;
+    float2 m1[2][kTaps];
+    float m3[2][kTaps];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int i = 0; i < kTaps; ++i) {
+            m1[j][i] = make_float2(0.f, 0.f);
+            m3[j][i] = 0.f;
         }
-        __syncthreads();
-        float (*s_m)[kInH][kLd] = s_mb[c & 1];
-        for (int it = threadIdx.x; it < kInH * (kTX / kCB); it += kThreads) {
-            const int r = it % kInH, q0 = (it / kInH) * kCB;
-            float o[3][kCB];
+    const int gx = st.x0 + 2 * lane;
+    const int r0 = max(st.y0 - kR, 0), rend = st.y1 + kR;
+    const bool in0 = gx < a.W, in1 = gx + 1 < a.W;
+    const bool pair = in1 && (a.W & 1) == 0 && (reinterpret_cast<uintptr_t>(a.grad) & 7u) == 0;
+    auto fetch = [&](int r) {  // row r of the maps, row r - kR of the images
+        float2* row = s_row[r % kRing];
+        float* rowc = s_c[r % kRing];
 #pragma unroll
-            for (int m = 0; m < 3; ++m)
+        for (int q = 0; q < 3; ++q) {
+            if (32 * q + lane >= kRow) continue;
+            const bool ok = st.col[q] >= 0 && r < a.H && r < rend;
+            const size_t o = ok ? (size_t)r * a.pitch + st.col[q] : 0;
+            copy8(row + 32 * q + lane, pab + o, ok);
+            copy4(rowc + 32 * q + lane, pc + o, ok);
+        }
+        const int y = r - kR;
 #pragma unroll
-                for (int j = 0; j < kCB; ++j) o[m][j] = 0.f;
+        for (int q = 0; q < 2; ++q) {
+            const int x = st.x0 + 32 * q + lane;
+            const bool ok = y >= st.y0 && y < st.y1 && x < a.W;
+            const size_t o = ok ? (size_t)y * a.W + x : 0;
+            copy4(&s_x[r % kRing][32 * q + lane], px + o, ok);
+            copy4(&s_y[r % kRing][32 * q + lane], py + o, ok);
+        }
+        copy_commit();
+    };
+    for (int k = 0; k < kRing - 1; ++k) fetch(r0 + k);
+    float wo = 0.f;
+    for (int r = r0; r < rend; ++r) {
+        const float2* row = s_row[r % kRing];
+        const float* rowc = s_c[r % kRing];
+        copy_wait<kRing - 2>();
+        __syncwarp();  // row r is in place, and every lane is done with the row the next copy replaces
+        fetch(r + kRing - 1);
+        const int y = r - kR;
+        const bool done = y >= st.y0;  // warp-uniform
+        const size_t pix = (size_t)st.ch * HW + (size_t)y * a.W + gx;
+        const float2 xv2 = *reinterpret_cast<const float2*>(&s_x[r % kRing][2 * lane]);
+        const float2 yv2 = *reinterpret_cast<const float2*>(&s_y[r % kRing][2 * lane]);
+        const float xv[2] = {xv2.x, xv2.y}, yv[2] = {yv2.x, yv2.y};
+        float2 h1[2];
+        float h3[2];
 #pragma unroll
-            for (int i = 0; i < kCB + 2 * kR; ++i) {
-                float v[3];
+        for (int j = 0; j < 2; ++j) {
+            h1[j] = make_float2(0.f, 0.f);
+            h3[j] = 0.f;
+        }
 #pragma unroll
-                for (int m = 0; m < 3; ++m) v[m] = s_m[m][r][q0 + i];
+        for (int i = 0; i < kWin + 1; i += 2) {
+            const float4 v4 = *reinterpret_cast<const float4*>(row + 2 * lane + i);
+            const float2 c2 = *reinterpret_cast<const float2*>(rowc + 2 * lane + i);
 #pragma unroll
-                for (int j = 0; j < kCB; ++j) {
-                    const int k = i - j;
+            for (int e = 0; e < 2; ++e) {
+                const float2 v = e ? make_float2(v4.z, v4.w) : make_float2(v4.x, v4.y);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int k = i + e - j;
                     if (k < 0 || k >= kWin) continue;
-                    const float gk = a.g[k];
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) o[m][j] = fmaf(gk, v[m], o[m][j]);
+                    h1[j] = fma2(make_float2(a.g[k], a.g[k]), v, h1[j]);
+                    h3[j] = fmaf(a.g[k], e ? c2.y : c2.x, h3[j]);
                 }
             }
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int j = 0; j < kCB; ++j) s_h[m][r][q0 + j] = o[m][j];
         }
-        __syncthreads();
-        for (int it = threadIdx.x; it < kTX * (kTY / kCB); it += kThreads) {
-            const int q = it % kTX, r0 = (it / kTX) * kCB;
-            float o[3][kCB];
+        if (done && ((y - st.y0) & 31) == 0) wo = row_weight(a, y + lane);
+        const float w = __shfl_sync(0xffffffffu, wo, (y - st.y0) & 31) * a.inv_wsum;
+        float gr[2];
 #pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int j = 0; j < kCB; ++j) o[m][j] = 0.f;
-#pragma unroll
-            for (int i = 0; i < kCB + 2 * kR; ++i) {
-                float h[3];
-#pragma unroll
-                for (int m = 0; m < 3; ++m) h[m] = s_h[m][r0 + i][q];
-#pragma unroll
-                for (int j = 0; j < kCB; ++j) {
-                    const int k = i - j;
-                    if (k < 0 || k >= kWin) continue;
-                    const float gk = a.g[k];
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) o[m][j] = fmaf(gk, h[m], o[m][j]);
-                }
-            }
-            const int gx = x0 + q;
-#pragma unroll
-            for (int j = 0; j < kCB; ++j) {
-                const int gy = y0 + r0 + j;
-                if (gy >= a.H || gx >= a.W) continue;
-                const size_t pix = c * HW + (size_t)gy * a.W + gx;
-                const float xv = a.x[pix], yv = a.y[pix];
-                const float d = xv - yv;
-                const float sgn = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-                const float w = row_weight(a, gy) * a.inv_wsum;
-                a.grad[pix] = (1.f - a.lam) * w * sgn - a.lam * (o[0][j] + 2.f * xv * o[1][j] + yv * o[2][j]);
+        for (int j = 0; j < 2; ++j) {
+            const float2 m = fir_step(m1[j], h1[j], a.g);
+            const float e = fir_step(m3[j], h3[j], a.g);
+            const float d = xv[j] - yv[j];
+            const float sgn = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+            gr[j] = (1.f - a.lam) * w * sgn - a.lam * (m.x + 2.f * xv[j] * m.y + yv[j] * e);
+        }
+        if (done) {
+            if (pair) {
+                *reinterpret_cast<float2*>(a.grad + pix) = make_float2(gr[0], gr[1]);
+            } else {
+                if (in0) a.grad[pix] = gr[0];
+                if (in1) a.grad[pix + 1] = gr[1];
             }
         }
-        __syncthreads();
     }
 }
 
@@ -329,11 +409,41 @@ __global__ void __launch_bounds__(kThreads) k_loss_reduce(const float* __restric
     if (threadIdx.x == 0) *loss = accumulate ? *loss + t : t;
 }
 
-int blocks_for(int W, int H) { return ((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY); }
+constexpr int kSms = 152;  // GB300
+// CTAs of the L1 pass alone
+int l1_blocks(int W, int H) { return min(((W + 31) / 32) * ((H + 31) / 32), 3 * H); }
 
+// Strips and segments of the streaming passes, one warp each. A segment reads 2 kR rows more than it
+// finishes, and an SM needs about kBusy warps to hide the latencies: the number of segments that
+// minimises the rows the fullest SM works through (at 2048 x 1024 with kBusy 8 / 12 / 16: 72 + 51,
+// 56 + 43, 62 + 44 us).
+struct Plan {
+    int strips, segs, rows, pitch;
+    int warps() const { return 3 * strips * segs; }
+};
+Plan make_plan(int W, int H) {
+    constexpr int kBusy = 12;
+    Plan p{};
+    p.strips = (W + kCols - 1) / kCols;
+    p.pitch = (W + 3) & ~3;
+    long long best = -1;
+    for (int segs = 1; segs <= (H + 7) / 8; ++segs) {
+        const int rows = (H + segs - 1) / segs;
+        const long long warps = 3ll * p.strips * ((H + rows - 1) / rows);
+        const long long cost = std::max<long long>((warps + kSms - 1) / kSms, kBusy) * (rows + 2 * kR);
+        if (best < 0 || cost < best) {
+            best = cost;
+            p.rows = rows;
+            p.segs = (H + rows - 1) / rows;
+        }
+    }
+    return p;
+}
+
+size_t maps_bytes(const Plan& p, int H) { return (9 * (size_t)p.pitch * H * sizeof(float) + 15) & ~(size_t)15; }
 size_t scratch_for(int W, int H) {
-    const size_t maps = 9 * (size_t)W * H * sizeof(float);
-    return ((maps + 15) & ~(size_t)15) + (size_t)blocks_for(W, H) * sizeof(float);
+    const Plan p = make_plan(W, H);
+    return maps_bytes(p, H) + (size_t)std::max(p.warps(), l1_blocks(W, H)) * sizeof(float);
 }
 
 }  // namespace
@@ -353,13 +463,16 @@ extern "C" odgs_status odgs_loss_l1_dssim(const float* image, const float* targe
         return ODGS_ERR_WORKSPACE;
     LossArgs a{};
     a.x = image; a.y = target; a.grad = grad;
-    a.maps = static_cast<float*>(scratch);
-    a.partial = reinterpret_cast<float*>(static_cast<char*>(scratch) + (scratch_for(width, height) -
-                                                                        (size_t)blocks_for(width, height) * sizeof(float)));
+    const Plan plan = make_plan(width, height);
+    a.ab = static_cast<float2*>(scratch);
+    a.c = reinterpret_cast<float*>(a.ab + 3 * (size_t)plan.pitch * height);
+    a.partial = reinterpret_cast<float*>(static_cast<char*>(scratch) + maps_bytes(plan, height));
     a.W = width; a.H = height; a.wrap = p->wrap_u ? 1 : 0; a.area = p->area_weight ? 1 : 0;
+    a.pitch = plan.pitch; a.strips = plan.strips; a.segs = plan.segs; a.rows = plan.rows;
     a.lam = p->lambda;
-    double wsum = 0.0, gsum = 0.0;
-    for (int j = 0; j < height; ++j) wsum += a.area ? std::sin(M_PI * (j + 0.5) / height) : 1.0;
+    // sum over j of sin(pi (j + 1/2) / H) = 1 / sin(pi / (2 H))
+    const double wsum = a.area ? 1.0 / std::sin(M_PI / (2.0 * height)) : (double)height;
+    double gsum = 0.0;
     a.inv_wsum = (float)(1.0 / (3.0 * width * wsum));
     double g[kWin];
     for (int k = 0; k < kWin; ++k) {
@@ -370,23 +483,13 @@ extern "C" odgs_status odgs_loss_l1_dssim(const float* image, const float* targe
     for (int k = 0; k < kWin; ++k) a.g[k] = (float)(g[k] / gsum);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (p->lambda == 0.f) {  // L1 alone: no SSIM window
-        const int blocks = min(blocks_for(width, height), 3 * height);
+        const int blocks = l1_blocks(width, height);
         k_l1<<<blocks, kThreads, 0, st>>>(a);
         k_loss_reduce<<<1, kThreads, 0, st>>>(a.partial, blocks, loss, p->accumulate ? 1 : 0);
         return cudaGetLastError() == cudaSuccess ? ODGS_OK : ODGS_ERR_CUDA;
     }
-    const dim3 grid((width + kTX - 1) / kTX, (height + kTY - 1) / kTY);
-    constexpr size_t kFwdSmem = sizeof(float) * (4 * kInH * kLd + 5 * kInH * kHd);
-    constexpr size_t kBwdSmem = sizeof(float) * (6 * kInH * kLd + 3 * kInH * kHd);
-    static bool smem_set = false;
-    if (!smem_set) {
-        if (cudaFuncSetAttribute(k_ssim_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(k_ssim_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem) != cudaSuccess)
-            return ODGS_ERR_CUDA;
-        smem_set = true;
-    }
-    k_ssim_fwd<<<grid, kThreads, kFwdSmem, st>>>(a);
-    k_loss_reduce<<<1, kThreads, 0, st>>>(a.partial, blocks_for(width, height), loss, p->accumulate ? 1 : 0);
-    if (grad) k_ssim_bwd<<<grid, kThreads, kBwdSmem, st>>>(a);
+    k_ssim_fwd<<<plan.warps(), 32, 0, st>>>(a);
+    k_loss_reduce<<<1, kThreads, 0, st>>>(a.partial, plan.warps(), loss, p->accumulate ? 1 : 0);
+    if (grad) k_ssim_bwd<<<plan.warps(), 32, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? ODGS_OK : ODGS_ERR_CUDA;
 }
