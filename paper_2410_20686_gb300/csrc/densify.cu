@@ -4,10 +4,9 @@
 //                        the statistics that the backward preprocess accumulated
 //   k_apply_count        per tile of 1024 Gaussians: how many are kept, cloned, split
 //   k_apply_scan         one CTA: exclusive offsets of the tiles and the totals
-//   k_apply_scatter      per tile again: each Gaussian's output slots (block scan + tile
-//                        offset), then its copies / children (all but the SH rows) and the
-//                        source index of every slot
-//   k_apply_sh           the SH rows, slot by slot in 16-byte chunks (coalesced)
+//   k_apply_place        per tile again: the source index of each Gaussian's output slots (block scan
+//                        + tile offset)
+//   k_apply_copy         the parameters slot by slot, coalesced, and the split children
 // Each step streams its arrays once; densification runs every few hundred iterations, so the
 // point is to keep the parameters on the device, not to reach the copy bandwidth.
 #include <cuda_runtime.h>
@@ -25,30 +24,51 @@ constexpr int kPerThread = 4;
 constexpr int kTile = kThreads * kPerThread;
 constexpr float kLog1p6 = 0.470003629245735553650937f;  // ln 1.6: log-scale of a split child
 
-__global__ void __launch_bounds__(kThreads) k_densify_select(const float* __restrict__ grad,
-                                                             const float* __restrict__ elev,
-                                                             const uint32_t* __restrict__ count,
-                                                             const float* __restrict__ scales,
-                                                             const float* __restrict__ opacity, int n,
-                                                             odgs_densify_params p, float big_thr, float op_thr,
-                                                             float max_thr, uint8_t* __restrict__ action) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t c = count[i];
+// The rule for one Gaussian; smax: its largest scale. big_thr, op_thr, max_thr: thresholds in the space of
+// the inputs (activated, or log-scale / logit), set by the host.
+__device__ __forceinline__ uint32_t decide(float grad, float elev, uint32_t c, float smax, float opacity,
+                                           const odgs_densify_params& p, float big_thr, float op_thr, float max_thr) {
     float gmean = 0.f, emean = 0.f;
     if (c > 0u) {
         const float fc = __uint2float_rn(c);
-        gmean = __fdiv_rn(grad[i], fc);
-        emean = __fdiv_rn(elev[i], fc);
+        gmean = __fdiv_rn(grad, fc);
+        emean = __fdiv_rn(elev, fc);
     }
     // Sec. 3.3: tau = tau_min + (1 - cos theta)(tau_max - tau_min), with the views' mean of 1 - cos theta
     const float tau = __fadd_rn(p.tau_min, __fmul_rn(emean, __fsub_rn(p.tau_max, p.tau_min)));
     const bool hot = c > 0u && gmean >= tau;
-    const float smax = fmaxf(fmaxf(scales[3 * i], scales[3 * i + 1]), scales[3 * i + 2]);
-    // thresholds in the space of the inputs (activated, or log-scale / logit), set by the host
-    const bool big = smax > big_thr;
-    const bool prune = opacity[i] < op_thr || smax > max_thr;
-    action[i] = (uint8_t)(prune ? ODGS_PRUNE : hot ? (big ? ODGS_SPLIT : ODGS_CLONE) : ODGS_KEEP);
+    const bool prune = opacity < op_thr || smax > max_thr;
+    return prune ? ODGS_PRUNE : hot ? (smax > big_thr ? ODGS_SPLIT : ODGS_CLONE) : ODGS_KEEP;
+}
+
+// Four Gaussians per thread, in 16-byte loads when every array is 16-byte aligned (vec): 29 bytes are
+// read and written per Gaussian, and one 4-byte load at a time kept too few of them in flight.
+__global__ void __launch_bounds__(kThreads) k_densify_select(const float* __restrict__ grad,
+                                                             const float* __restrict__ elev,
+                                                             const uint32_t* __restrict__ count,
+                                                             const float* __restrict__ scales,
+                                                             const float* __restrict__ opacity, int n, int vec,
+                                                             odgs_densify_params p, float big_thr, float op_thr,
+                                                             float max_thr, uint8_t* __restrict__ action) {
+    const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i0 >= n) return;
+    if (vec && i0 + 4 <= n) {
+        const float4 g = *reinterpret_cast<const float4*>(grad + i0), e = *reinterpret_cast<const float4*>(elev + i0);
+        const uint4 c = *reinterpret_cast<const uint4*>(count + i0);
+        const float4* s4 = reinterpret_cast<const float4*>(scales + 3 * (size_t)i0);
+        const float4 s0 = s4[0], s1 = s4[1], s2 = s4[2], o = *reinterpret_cast<const float4*>(opacity + i0);
+        uint32_t r = decide(g.x, e.x, c.x, fmaxf(fmaxf(s0.x, s0.y), s0.z), o.x, p, big_thr, op_thr, max_thr);
+        r |= decide(g.y, e.y, c.y, fmaxf(fmaxf(s0.w, s1.x), s1.y), o.y, p, big_thr, op_thr, max_thr) << 8;
+        r |= decide(g.z, e.z, c.z, fmaxf(fmaxf(s1.z, s1.w), s2.x), o.z, p, big_thr, op_thr, max_thr) << 16;
+        r |= decide(g.w, e.w, c.w, fmaxf(fmaxf(s2.y, s2.z), s2.w), o.w, p, big_thr, op_thr, max_thr) << 24;
+        *reinterpret_cast<uint32_t*>(action + i0) = r;
+        return;
+    }
+    for (int i = i0; i < min(i0 + 4, n); ++i) {
+        const float* s = scales + 3 * (size_t)i;
+        action[i] = (uint8_t)decide(grad[i], elev[i], count[i], fmaxf(fmaxf(s[0], s[1]), s[2]), opacity[i], p, big_thr,
+                                    op_thr, max_thr);
+    }
 }
 
 // (kept, cloned, split) indicator of one action
@@ -146,65 +166,8 @@ struct ApplyArgs {
     int raw;        // scales are log-scales
 };
 
-// Copies Gaussian i into slot d (d < cap); child >= 0 places it as that split child.
-__device__ __forceinline__ void write_gaussian(const ApplyArgs& a, int i, uint32_t d, int child) {
-    if (d >= a.cap) return;
-    const float4 q = *reinterpret_cast<const float4*>(a.quats + 4 * (size_t)i);
-    float m[3] = {a.means[3 * i], a.means[3 * i + 1], a.means[3 * i + 2]};
-    float s[3] = {a.scales[3 * i], a.scales[3 * i + 1], a.scales[3 * i + 2]};
-    if (child >= 0) {
-        if (a.raw) {  // the child's offset uses the activated scales
-#pragma unroll
-            for (int r = 0; r < 3; ++r) s[r] = expf(s[r]);
-        }
-        const float qn = sqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
-        float R[9];
-        quat_rot(q.x / qn, q.y / qn, q.z / qn, q.w / qn, R);
-        const float* z = a.noise + 6 * (size_t)i + 3 * child;
-        const float sz[3] = {s[0] * z[0], s[1] * z[1], s[2] * z[2]};
-#pragma unroll
-        for (int r = 0; r < 3; ++r) m[r] += R[3 * r] * sz[0] + R[3 * r + 1] * sz[1] + R[3 * r + 2] * sz[2];
-        if (a.raw) {
-#pragma unroll
-            for (int r = 0; r < 3; ++r) s[r] = __fsub_rn(a.scales[3 * i + r], kLog1p6);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 3; ++r) s[r] = __fdiv_rn(s[r], 1.6f);
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        a.o_means[3 * (size_t)d + r] = m[r];
-        a.o_scales[3 * (size_t)d + r] = s[r];
-    }
-    *reinterpret_cast<float4*>(a.o_quats + 4 * (size_t)d) = q;
-    a.o_opacity[d] = a.opacity[i];
-    a.src[d] = (uint32_t)i;
-}
-
-// SH rows of all output slots: thread t copies 16-byte chunk t % chunks of slot t / chunks (or
-// single floats when the rows are not 16-byte multiples).
-__global__ void __launch_bounds__(kThreads) k_apply_sh(const float* __restrict__ sh, float* __restrict__ o_sh,
-                                                       const uint32_t* __restrict__ src, const uint4* __restrict__ totals,
-                                                       uint32_t cap, int sh_coeffs) {
-    const uint32_t slots = min(totals->w, cap);
-    const int ns = 3 * sh_coeffs;
-    const bool vec = (ns % 4) == 0 && (reinterpret_cast<uintptr_t>(sh) % 16) == 0 &&
-                     (reinterpret_cast<uintptr_t>(o_sh) % 16) == 0;
-    const int chunks = vec ? ns / 4 : ns;
-    const size_t total = (size_t)slots * chunks;
-    for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const size_t d = t / chunks;
-        const int c = (int)(t - d * chunks);
-        const size_t i = src[d];
-        if (vec)
-            reinterpret_cast<float4*>(o_sh + d * ns)[c] = reinterpret_cast<const float4*>(sh + i * ns)[c];
-        else
-            o_sh[d * ns + c] = sh[i * ns + c];
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) k_apply_scatter(ApplyArgs a) {
+// Source Gaussian of every output slot.
+__global__ void __launch_bounds__(kThreads) k_apply_place(ApplyArgs a) {
     __shared__ uint3 s_warp[kThreads / 32];
     const int base = blockIdx.x * kTile + threadIdx.x * kPerThread;
     uint8_t act[kPerThread];
@@ -219,18 +182,86 @@ __global__ void __launch_bounds__(kThreads) k_apply_scatter(ApplyArgs a) {
     const uint4 to = a.tile_offsets[blockIdx.x];
     const uint4 T = *a.totals;
     off = add3(off, make_uint3(to.x, to.y, to.z));
+    auto put = [&](uint32_t d, int i) {
+        if (d < a.cap) a.src[d] = (uint32_t)i;
+    };
 #pragma unroll
     for (int k = 0; k < kPerThread; ++k) {
         const int i = base + k;
         if (i >= a.n) break;
         const uint3 cl = classes(act[k]);
-        if (cl.x) write_gaussian(a, i, off.x, -1);
-        if (cl.y) write_gaussian(a, i, T.x + off.y, -1);
+        if (cl.x) put(off.x, i);
+        if (cl.y) put(T.x + off.y, i);
         if (cl.z) {
-            write_gaussian(a, i, T.x + T.y + off.z, 0);
-            write_gaussian(a, i, T.x + T.y + T.z + off.z, 1);
+            put(T.x + T.y + off.z, i);
+            put(T.x + T.y + T.z + off.z, i);
         }
         off = add3(off, cl);
+    }
+}
+
+// The mean and scales of slot d, a split child of Gaussian i.
+__device__ __forceinline__ void write_child(const ApplyArgs& a, size_t i, uint32_t d, int child) {
+    const float4 q = *reinterpret_cast<const float4*>(a.quats + 4 * i);
+    float m[3] = {a.means[3 * i], a.means[3 * i + 1], a.means[3 * i + 2]};
+    float s[3] = {a.scales[3 * i], a.scales[3 * i + 1], a.scales[3 * i + 2]};
+    if (a.raw) {  // the child's offset uses the activated scales
+#pragma unroll
+        for (int r = 0; r < 3; ++r) s[r] = expf(s[r]);
+    }
+    const float qn = sqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
+    float R[9];
+    quat_rot(q.x / qn, q.y / qn, q.z / qn, q.w / qn, R);
+    const float* z = a.noise + 6 * i + 3 * child;
+    const float sz[3] = {s[0] * z[0], s[1] * z[1], s[2] * z[2]};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        m[r] += R[3 * r] * sz[0] + R[3 * r + 1] * sz[1] + R[3 * r + 2] * sz[2];
+        a.o_means[3 * (size_t)d + r] = m[r];
+        a.o_scales[3 * (size_t)d + r] = a.raw ? __fsub_rn(a.scales[3 * i + r], kLog1p6) : __fdiv_rn(s[r], 1.6f);
+    }
+}
+
+// The parameters of kThreads consecutive slots per CTA, array by array with consecutive threads on
+// consecutive elements: a run of slots has nearly consecutive sources, so the reads coalesce too.
+// Only the means and scales of split children (the last slots) are computed, a thread each.
+__global__ void __launch_bounds__(kThreads) k_apply_copy(ApplyArgs a) {
+    __shared__ uint32_t s_src[kThreads];
+    const uint4 T = *a.totals;
+    const uint32_t slots = min(T.w, a.cap), plain = min(T.x + T.y, slots);
+    const int ns = 3 * a.sh_coeffs;
+    const bool vec = (ns % 4) == 0 && (reinterpret_cast<uintptr_t>(a.sh) % 16) == 0 &&
+                     (reinterpret_cast<uintptr_t>(a.o_sh) % 16) == 0;
+    const int per = vec ? ns / 4 : ns;  // 16-byte chunks (or floats) of an SH row
+    const uint32_t groups = (slots + kThreads - 1) / kThreads;
+    for (uint32_t grp = blockIdx.x; grp < groups; grp += gridDim.x) {
+        const uint32_t d0 = grp * kThreads;
+        const int cnt = (int)min((uint32_t)kThreads, slots - d0);
+        __syncthreads();  // the previous group's reads of s_src
+        if ((int)threadIdx.x < cnt) s_src[threadIdx.x] = a.src[d0 + threadIdx.x];
+        __syncthreads();
+        for (int t = threadIdx.x; t < cnt * per; t += kThreads) {
+            const int j = t / per, c = t - j * per;
+            const size_t i = s_src[j], d = d0 + j;
+            if (vec)
+                reinterpret_cast<float4*>(a.o_sh + d * ns)[c] = __ldg(reinterpret_cast<const float4*>(a.sh + i * ns) + c);
+            else
+                a.o_sh[d * ns + c] = __ldg(a.sh + i * ns + c);
+        }
+        const int copied = d0 < plain ? (int)min((uint32_t)cnt, plain - d0) : 0;
+        for (int t = threadIdx.x; t < 3 * copied; t += kThreads) {
+            const int j = t / 3, r = t - 3 * j;
+            const size_t i = s_src[j];
+            a.o_means[3 * (size_t)d0 + t] = __ldg(a.means + 3 * i + r);
+            a.o_scales[3 * (size_t)d0 + t] = __ldg(a.scales + 3 * i + r);
+        }
+        if ((int)threadIdx.x < cnt) {
+            const uint32_t d = d0 + threadIdx.x;
+            const size_t i = s_src[threadIdx.x];
+            reinterpret_cast<float4*>(a.o_quats)[d] = __ldg(reinterpret_cast<const float4*>(a.quats) + i);
+            a.o_opacity[d] = __ldg(a.opacity + i);
+            if (d >= T.x + T.y) write_child(a, i, d, d >= T.x + T.y + T.z ? 1 : 0);
+        }
     }
 }
 
@@ -263,8 +294,12 @@ extern "C" odgs_status odgs_densify_select(const float* grad, const float* elev,
         op_thr = p->min_opacity;
         max_thr = p->max_scale > 0.f ? p->max_scale : inf;
     }
-    k_densify_select<<<(n + kThreads - 1) / kThreads, kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        grad, elev, count, scales, opacity, n, *p, big_thr, op_thr, max_thr, action);
+    const uintptr_t at = reinterpret_cast<uintptr_t>(grad) | reinterpret_cast<uintptr_t>(elev) |
+                         reinterpret_cast<uintptr_t>(count) | reinterpret_cast<uintptr_t>(scales) |
+                         reinterpret_cast<uintptr_t>(opacity);
+    const int vec = at % 16 == 0 && reinterpret_cast<uintptr_t>(action) % 4 == 0;
+    k_densify_select<<<(n + 4 * kThreads - 1) / (4 * kThreads), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
+        grad, elev, count, scales, opacity, n, vec, *p, big_thr, op_thr, max_thr, action);
     return cudaGetLastError() == cudaSuccess ? ODGS_OK : ODGS_ERR_CUDA;
 }
 
@@ -303,10 +338,10 @@ extern "C" odgs_status odgs_densify_apply(const odgs_gaussians* in, int sh_coeff
     a.o_means = out->means; a.o_scales = out->scales; a.o_quats = out->quats; a.o_opacity = out->opacity;
     a.o_sh = out->sh; a.cap = cap; a.tile_offsets = tile_offsets; a.totals = totals; a.src = src;
     a.raw = raw_params;
-    k_apply_scatter<<<tiles, kThreads, 0, st>>>(a);
+    k_apply_place<<<tiles, kThreads, 0, st>>>(a);
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return ODGS_ERR_CUDA;
-    k_apply_sh<<<sms * 8, kThreads, 0, st>>>(in->sh, out->sh, src, totals, cap, sh_coeffs);
+    k_apply_copy<<<sms * 8, kThreads, 0, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? ODGS_OK : ODGS_ERR_CUDA;
 }
