@@ -114,7 +114,8 @@ typedef struct {
                            of a convex exponent over the tile is at a corner pixel). Images,
                            final T and gradients are the same as with the whole lists; fewer
                            pairs are emitted and sorted. Frames of more than 2^19 tiles keep
-                           the whole lists. 1: the whole lists (every Gaussian whose footprint
+                           the whole lists, and so do frames whose pairs odgs_query_pairs has
+                           reported as at most 32768 when they all fit in the pair buffer. 1: the whole lists (every Gaussian whose footprint
                            meets the tile)                                                 */
 } odgs_settings;
 

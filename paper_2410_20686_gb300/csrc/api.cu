@@ -215,6 +215,10 @@ struct odgs_ctx {
     // workspace (they are computed from the depth keys by item, which the depth sort overwrites,
     // so a second odgs_bin_sort or a rebuild of the lists reuses them)
     bool cut_ready = false;
+    // the pairs of the current preprocess, once odgs_query_pairs has read them back
+    bool pairs_known = false;
+    size_t pairs = 0;
+    bool whole_lists = false;  // what the last binning that was no rebuild did
     // a second stream on which the binning computes the cuts while the depth sort runs (forked
     // from and joined back to the caller's stream by events)
     cudaStream_t side = nullptr;
@@ -282,7 +286,9 @@ static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
     ViewDev* vd = reinterpret_cast<ViewDev*>(w + c->L.views);
     float4* trig = reinterpret_cast<float4*>(w + c->L.trig);
     uint32_t* dhist = reinterpret_cast<uint32_t*>(w + c->L.sort_hist);
-    if (launch_setup(c->tab, vd, trig, hdr, c->geo.total_trig, dhist, st) != cudaSuccess) return ODGS_ERR_CUDA;
+    if (launch_setup(c->tab, vd, trig, hdr, c->geo.total_trig, dhist, reinterpret_cast<uint4*>(w + c->L.sort_ctr),
+                     sort_scratch_quads(c->geo.n_items, kDepthLbRegions), st) != cudaSuccess)
+        return ODGS_ERR_CUDA;
     c->launches += 1;
     PreArgs a{};
     a.means = c->g.means; a.scales = c->g.scales; a.quats = c->g.quats; a.opacity = c->g.opacity; a.sh = c->g.sh;
@@ -344,6 +350,7 @@ odgs_status odgs_preprocess(odgs_ctx* c, const odgs_gaussians* g, const odgs_vie
     c->stage = 0;
     c->launches = 0;
     c->cut_ready = false;
+    c->pairs_known = false;
     c->bwd_batch = std::min(st.batch, 64);
     const int bwd_threads = st.tile_w * st.tile_h / st.pixels_per_thread_bwd;
     while (c->bwd_batch > 8 && render_bwd_smem(c->bwd_batch, bwd_threads) > 48 * 1024) c->bwd_batch /= 2;
@@ -362,6 +369,8 @@ odgs_status odgs_query_pairs(odgs_ctx* c, size_t* pairs, void* stream) {
         return ODGS_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return ODGS_ERR_CUDA;
     *pairs = (size_t)h.pairs;
+    c->pairs = *pairs;
+    c->pairs_known = true;
     if (h.status & kStTimeout) return ODGS_ERR_TIMEOUT;
     if (h.status & kStCapacity) return ODGS_ERR_CAPACITY;
     if (h.status & kStNonfinite) return ODGS_ERR_NONFINITE;
@@ -387,8 +396,16 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     uint8_t* w = c->ws;
     Header* hdr = reinterpret_cast<Header*>(w + c->L.hdr);
     bool joined = true;  // no side-stream work to wait for
+    // A frame known to have few pairs, all of which fit, keeps its whole lists (the same images and
+    // gradients): a tile sort of kFewPairs keys takes one wave of its smallest tiles, so cutting them
+    // saves nothing, and the cuts are five launches and four event calls of a frame that is bound by
+    // its launches (1K Gaussians at 256 x 128, one view: 151 -> 134 us with this and the sorts'
+    // scratch cleared by kernels instead of memsets).
+    constexpr size_t kFewPairs = 32768;
+    if (!rebuild) c->whole_lists = !c->L.truncate || (c->pairs_known && c->pairs <= std::min(c->pb_cap, kFewPairs));
+    const bool truncate = !c->whole_lists;
     // 0. which tiles saturate, and from which depth on (before the depth sort reorders the keys)
-    if (c->L.truncate && !c->cut_ready) {
+    if (truncate && !c->cut_ready) {
         SatArgs sa{};
         sa.rect = reinterpret_cast<const uint4*>(w + c->L.rect);
         sa.rec_a = reinterpret_cast<const float4*>(w + c->L.rec_a);
@@ -423,7 +440,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         if (launch_radix_sort(dk, dv, &hdr->n_items, c->geo.n_items, 32, reinterpret_cast<uint32_t*>(w + c->L.sort_hist),
                               reinterpret_cast<uint32_t*>(w + c->L.sort_ctr), reinterpret_cast<uint32_t*>(w + c->L.sort_lb),
                               &hdr->status, c->num_sms, st, &rb, &c->launches, /*hist_ready=*/true,
-                              c->wait_limit, kDepthLbRegions) != cudaSuccess)
+                              c->wait_limit, kDepthLbRegions, /*cleared=*/true) != cudaSuccess)
             return ODGS_ERR_CUDA;
         c->depth_buf = rb;
     }
@@ -451,7 +468,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     b.num_sms = c->num_sms;
     b.key_hist = reinterpret_cast<uint32_t*>(p + c->P.hist);
     b.key_passes = radix_passes(c->geo.key_bits);
-    if (c->L.truncate && c->geo.n_items > 0) {
+    if (truncate && c->geo.n_items > 0) {
         b.cut = w + c->L.cut;
         b.G = reinterpret_cast<const uint32_t*>(w + c->L.cover);
         b.sorted_keys = dk[rb];
@@ -466,6 +483,17 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         b.ranges_zero = reinterpret_cast<uint2*>(w + c->L.ranges);
         b.n_ranges = (uint32_t)c->geo.total_tiles;
     }
+    // k_emit clears the tile sort's scratch, and the depth sort's for another odgs_bin_sort of this frame
+    // (the preprocess clears it for the first)
+    const bool emits = c->geo.n_items > 0 && c->pb_cap > 0;
+    if (emits) {
+        b.clear[0] = reinterpret_cast<uint4*>(p + c->P.ctr);
+        b.clear_quads[0] = sort_scratch_quads(c->pb_cap, kPairLbRegions);
+    }
+    if (!rebuild && c->geo.n_items > 0) {
+        b.clear[1] = reinterpret_cast<uint4*>(w + c->L.sort_ctr);
+        b.clear_quads[1] = sort_scratch_quads(c->geo.n_items, kDepthLbRegions);
+    }
     if (!joined && cudaStreamWaitEvent(st, c->ev_join, 0) != cudaSuccess) return ODGS_ERR_CUDA;
     if (launch_binning(b, st, &c->launches) != cudaSuccess) return ODGS_ERR_CUDA;
     // 3. stable sort of the pairs by tile id
@@ -473,7 +501,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     if (launch_radix_sort(pk, pv, &hdr->n_pairs_sort, c->pb_cap, c->geo.key_bits, reinterpret_cast<uint32_t*>(p + c->P.hist),
                           reinterpret_cast<uint32_t*>(p + c->P.ctr), reinterpret_cast<uint32_t*>(p + c->P.lb),
                           &hdr->status, c->num_sms, st, &rp, &c->launches, /*hist_ready=*/true,
-                          c->wait_limit, kPairLbRegions) != cudaSuccess)
+                          c->wait_limit, kPairLbRegions, /*cleared=*/emits) != cudaSuccess)
         return ODGS_ERR_CUDA;
     c->sorted_vals = pv[rp];
     c->pair_buf = rp;

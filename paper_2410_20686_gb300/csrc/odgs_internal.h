@@ -115,6 +115,8 @@ struct BinArgs {
     // the pair counts, their scan and the kept-pair words of this depth order are in place from an
     // earlier binning of the same frame: emit only (a rebuild of the lists for the backward pass)
     bool emit_only;
+    uint4* clear[2];  // cleared by k_emit: the tile sort's scratch, the depth sort's (or null)
+    size_t clear_quads[2];
 };
 
 struct EmitArgs {
@@ -135,6 +137,8 @@ struct EmitArgs {
     int key_passes;
     const uint32_t* kcount;  // by depth-order position, or null
     const uint8_t* cut;
+    uint4* clear[2];
+    size_t clear_quads[2];
 };
 
 struct SatArgs {
@@ -184,7 +188,7 @@ struct BwdArgs {
 };
 
 cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Header* hdr, int total_trig,
-                         uint32_t* dhist, cudaStream_t st);
+                         uint32_t* dhist, uint4* clear, size_t clear_quads, cudaStream_t st);
 cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st);
 cudaError_t launch_preprocess_bwd(const PreBwdArgs& a, int sh_degree, cudaStream_t st);
 
@@ -195,10 +199,14 @@ constexpr uint32_t kDefaultWaitLimit = 1u << 22;
 cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_ptr, size_t max_items, int bits,
                               uint32_t* hist, uint32_t* tile_ctrs, uint32_t* lookback, uint32_t* status, int num_sms,
                               cudaStream_t st, int* result_buf, int* launches, bool hist_ready, uint32_t wait_limit,
-                              int lb_regions = 1);  // look-back regions of radix_lookback_words each
+                              int lb_regions = 1,     // look-back regions of radix_lookback_words each
+                              bool cleared = false);  // counters and regions are already 0
 // A sort whose four tile counters lie kCtrBytes before its look-back regions (one per pass) clears
-// both with one memset.
+// both at once (sort_scratch_quads 16-byte groups).
 constexpr size_t kCtrBytes = 256;
+inline size_t sort_scratch_quads(size_t max_items, int lb_regions) {
+    return (kCtrBytes + sizeof(uint32_t) * radix_lookback_words(max_items) * (size_t)lb_regions) / sizeof(uint4);
+}
 
 int scan_blocks_for(uint32_t n_items);
 cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches);

@@ -15,11 +15,14 @@ namespace odgs {
 
 // ------------------------------------------------------------------ setup
 
-__global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr, int total_trig, uint32_t* dhist) {
+__global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr, int total_trig, uint32_t* dhist,
+                        uint4* clear, size_t clear_quads) {
     int gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid < tab.n_views) views[gid] = tab.v[gid];
     // the depth sort's digit histograms, counted by k_preprocess_geom
     for (int i = gid; i < 4 * 256; i += gridDim.x * blockDim.x) dhist[i] = 0u;
+    // and its scratch
+    for (size_t i = gid; i < clear_quads; i += gridDim.x * blockDim.x) clear[i] = make_uint4(0u, 0u, 0u, 0u);
     if (gid == 0) {
         hdr->pairs = 0ull;
         hdr->pairs_emitted = 0ull;
@@ -867,11 +870,12 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
 // ------------------------------------------------------------------ launchers
 
 cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Header* hdr, int total_trig,
-                         uint32_t* dhist, cudaStream_t st) {
+                         uint32_t* dhist, uint4* clear, size_t clear_quads, cudaStream_t st) {
     int threads = 256;
     int blocks = (max(total_trig, tab.n_views) + threads - 1) / threads;
+    blocks = max(blocks, (int)min(clear_quads / (4 * (size_t)threads), (size_t)1024));
     blocks = max(1, min(blocks, 1024));
-    k_setup<<<blocks, threads, 0, st>>>(tab, views, trig, hdr, total_trig, dhist);
+    k_setup<<<blocks, threads, 0, st>>>(tab, views, trig, hdr, total_trig, dhist, clear, clear_quads);
     return cudaGetLastError();
 }
 
