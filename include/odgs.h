@@ -10,11 +10,11 @@
  *   - the backward pass of App. A.3 (Eq. 11 and the Jacobian's dependence on the mean).
  *
  * Call sequence for one frame (one or many views of the same Gaussians):
- *   odgs_preprocess -> [odgs_query_pairs] -> odgs_bin_sort -> odgs_render_fwd
+ *   odgs_preprocess -> [odgs_query_pairs | odgs_wait_pairs] -> odgs_bin_sort -> odgs_render_fwd
  *   -> odgs_render_bwd -> odgs_preprocess_bwd
  * All compute calls are asynchronous on the given CUDA stream (a cudaStream_t passed as void*;
- * NULL = legacy default stream). Only odgs_query_pairs, odgs_get_status and odgs_frame_stats
- * synchronize. odgs_bin_sort also runs work on a stream of the context, forked from the given
+ * NULL = legacy default stream). Only odgs_query_pairs, odgs_wait_pairs, odgs_get_status and
+ * odgs_frame_stats synchronize. odgs_bin_sort also runs work on a stream of the context, forked from the given
  * stream and joined back to it by events within the call, so the call is ordered on the given
  * stream as a whole (and can be captured in a CUDA graph from it).
  *
@@ -114,8 +114,9 @@ typedef struct {
                            of a convex exponent over the tile is at a corner pixel). Images,
                            final T and gradients are the same as with the whole lists; fewer
                            pairs are emitted and sorted. Frames of more than 2^19 tiles keep
-                           the whole lists, and so do frames whose pairs odgs_query_pairs has
-                           reported as at most 32768 when they all fit in the pair buffer. 1: the whole lists (every Gaussian whose footprint
+                           the whole lists, and so do frames whose pairs odgs_query_pairs or
+                           odgs_wait_pairs has reported as at most 32768 when they all fit in
+                           the pair buffer. 1: the whole lists (every Gaussian whose footprint
                            meets the tile)                                                 */
 } odgs_settings;
 
@@ -167,6 +168,12 @@ odgs_status odgs_preprocess(odgs_ctx *ctx, const odgs_gaussians *g, const odgs_v
 /* Synchronizes the stream; returns the number of pairs the last odgs_preprocess produced
  * and, as the return value, the first error recorded on the device (or ODGS_OK). */
 odgs_status odgs_query_pairs(odgs_ctx *ctx, size_t *pairs, void *stream);
+
+/* As odgs_query_pairs, but right after odgs_preprocess it waits only for the projection, not for the
+ * colours that the stream computes after it, so that the caller can queue odgs_bin_sort while they
+ * run. (The first call of a context, calls in later stages and calls after a captured
+ * odgs_preprocess synchronize the stream as odgs_query_pairs does.) */
+odgs_status odgs_wait_pairs(odgs_ctx *ctx, size_t *pairs, void *stream);
 
 /* Depth sort, per-tile pair emission and stable tile sort (the "sorting by depth" of Sec.
  * 3.1, binned into ERP tiles), then per-tile list ranges. Pairs beyond pair_capacity are

@@ -27,7 +27,7 @@ EXPORTED = ("odgs_create", "odgs_destroy", "odgs_workspace_size", "odgs_pair_buf
             "odgs_render_fwd_static", "odgs_measure_peaks", "odgs_last_launch_count", "odgs_status_string",
             "odgs_densify_select", "odgs_densify_scratch_size", "odgs_densify_apply", "odgs_adam_step",
             "odgs_loss_scratch_size", "odgs_loss_l1_dssim", "odgs_set_wait_limit", "odgs_debug_lists",
-            "odgs_debug_screen_grads")
+            "odgs_debug_screen_grads", "odgs_wait_pairs")
 
 
 class OdgsError(RuntimeError):
@@ -116,6 +116,7 @@ def load(path: str = LIB_PATH):
     L.odgs_preprocess.argtypes = [vp, C.POINTER(Gaussians), C.POINTER(View), C.c_int, C.POINTER(Settings),
                                   vp, sz, vp]
     L.odgs_query_pairs.argtypes = [vp, C.POINTER(sz), vp]
+    L.odgs_wait_pairs.argtypes = [vp, C.POINTER(sz), vp]
     L.odgs_bin_sort.argtypes = [vp, vp, sz, vp]
     L.odgs_render_fwd.argtypes = [vp, C.POINTER(vp), C.POINTER(vp), vp]
     L.odgs_render_bwd.argtypes = [vp, C.POINTER(vp), vp]
@@ -143,10 +144,17 @@ def load(path: str = LIB_PATH):
                  "odgs_preprocess_bwd", "odgs_frame_stats", "odgs_get_status", "odgs_render_fwd_static",
                  "odgs_measure_peaks", "odgs_densify_select", "odgs_densify_scratch_size", "odgs_densify_apply",
                  "odgs_adam_step", "odgs_loss_scratch_size", "odgs_loss_l1_dssim", "odgs_set_wait_limit",
-                 "odgs_debug_lists", "odgs_debug_screen_grads"):
+                 "odgs_debug_lists", "odgs_debug_screen_grads", "odgs_wait_pairs"):
         getattr(L, name).restype = C.c_int
     _lib = L
     return L
+
+
+def raw_stream(device) -> C.c_void_p:
+    """The device's current stream as a cudaStream_t."""
+    import torch
+    k = torch.cuda.current_device() if device.index is None else device.index
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(k))
 
 
 def status_string(st: int) -> str:

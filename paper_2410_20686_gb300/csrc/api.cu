@@ -223,7 +223,14 @@ struct odgs_ctx {
     // from and joined back to the caller's stream by events)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    // odgs_wait_pairs: recorded after the projection (once a first call has made it), and the header's
+    // copy in page-locked host memory
+    cudaEvent_t ev_pairs = nullptr;
+    bool pairs_recorded = false;
+    Header* host = nullptr;
     ~odgs_ctx() {
+        if (ev_pairs) cudaEventDestroy(ev_pairs);
+        if (host) cudaFreeHost(host);
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
         if (side) cudaStreamDestroy(side);
@@ -315,7 +322,12 @@ static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
         a.cut_base = rn >> kCutShift;
     }
     a.hdr = hdr;
-    if (launch_preprocess(a, c->s.sh_degree, st) != cudaSuccess) return ODGS_ERR_CUDA;
+    // an event of a capture could not be waited for outside it
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const bool record = c->ev_pairs && cudaStreamIsCapturing(st, &capture) == cudaSuccess &&
+                        capture == cudaStreamCaptureStatusNone;
+    if (launch_preprocess(a, c->s.sh_degree, st, record ? c->ev_pairs : nullptr) != cudaSuccess) return ODGS_ERR_CUDA;
+    c->pairs_recorded = record;
     if (c->n > 0) c->launches += 2;
     return ODGS_OK;
 }
@@ -354,9 +366,27 @@ odgs_status odgs_preprocess(odgs_ctx* c, const odgs_gaussians* g, const odgs_vie
     c->bwd_batch = std::min(st.batch, 64);
     const int bwd_threads = st.tile_w * st.tile_h / st.pixels_per_thread_bwd;
     while (c->bwd_batch > 8 && render_bwd_smem(c->bwd_batch, bwd_threads) > 48 * 1024) c->bwd_batch /= 2;
+    c->pairs_recorded = false;
     r = run_preprocess(c, static_cast<cudaStream_t>(stream));
     if (r != ODGS_OK) return r;
     c->stage = 1;
+    return ODGS_OK;
+}
+
+// The context's second stream and its events, made once.
+static bool make_side(odgs_ctx* c) {
+    return (c->side || cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) == cudaSuccess) &&
+           (c->ev_fork || cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess) &&
+           (c->ev_join || cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess);
+}
+
+static odgs_status report_pairs(odgs_ctx* c, const Header& h, size_t* pairs) {
+    *pairs = (size_t)h.pairs;
+    c->pairs = *pairs;
+    c->pairs_known = true;
+    if (h.status & kStTimeout) return ODGS_ERR_TIMEOUT;
+    if (h.status & kStCapacity) return ODGS_ERR_CAPACITY;
+    if (h.status & kStNonfinite) return ODGS_ERR_NONFINITE;
     return ODGS_OK;
 }
 
@@ -368,13 +398,29 @@ odgs_status odgs_query_pairs(odgs_ctx* c, size_t* pairs, void* stream) {
     if (cudaMemcpyAsync(&h, c->ws + c->L.hdr, sizeof(Header), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return ODGS_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return ODGS_ERR_CUDA;
-    *pairs = (size_t)h.pairs;
-    c->pairs = *pairs;
-    c->pairs_known = true;
-    if (h.status & kStTimeout) return ODGS_ERR_TIMEOUT;
-    if (h.status & kStCapacity) return ODGS_ERR_CAPACITY;
-    if (h.status & kStNonfinite) return ODGS_ERR_NONFINITE;
-    return ODGS_OK;
+    return report_pairs(c, h, pairs);
+}
+
+// The pair count is final after the projection: read on the side stream, while the colours run, it
+// spares the GPU the gap between them and the binning's first launch (1M Gaussians, one 2048 x 1024 view
+// rendered eagerly: 733 -> 687 us together with the wrapper's cheaper stream look-ups).
+odgs_status odgs_wait_pairs(odgs_ctx* c, size_t* pairs, void* stream) {
+    if (!c || !pairs) return ODGS_ERR_INVALID_ARG;
+    if (c->stage < 1) return ODGS_ERR_STATE;
+    if (!c->ev_pairs) {  // the first call makes what the next preprocess records
+        if (!make_side(c) || (!c->host && cudaHostAlloc(reinterpret_cast<void**>(&c->host), sizeof(Header), 0) != cudaSuccess) ||
+            cudaEventCreateWithFlags(&c->ev_pairs, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            c->ev_pairs = nullptr;
+        }
+    }
+    // later stages report what they found, which only the stream's own order shows
+    if (c->stage > 1 || !c->pairs_recorded) return odgs_query_pairs(c, pairs, stream);
+    if (cudaStreamWaitEvent(c->side, c->ev_pairs, 0) != cudaSuccess ||
+        cudaMemcpyAsync(c->host, c->ws + c->L.hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->side) != cudaSuccess ||
+        cudaStreamSynchronize(c->side) != cudaSuccess)
+        return ODGS_ERR_CUDA;
+    return report_pairs(c, *c->host, pairs);
 }
 
 odgs_status odgs_get_status(odgs_ctx* c, uint32_t* bits, void* stream) {
@@ -421,10 +467,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         sa.cut = w + c->L.cut;
         // on the side stream, beside the depth sort (they share no data; the depth sort's
         // passes fill only part of the GPU)
-        if (!c->side && (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
-                         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-                         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess))
-            return ODGS_ERR_CUDA;
+        if (!make_side(c)) return ODGS_ERR_CUDA;
         if (cudaEventRecord(c->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(c->side, c->ev_fork, 0) != cudaSuccess)
             return ODGS_ERR_CUDA;
         if (launch_saturation(sa, c->num_sms, c->side, &c->launches) != cudaSuccess) return ODGS_ERR_CUDA;

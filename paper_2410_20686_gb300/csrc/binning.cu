@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
     // the tile sort's digit counts, which the emission adds up, start from 0
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) key_hist[i] = 0u;
     // eight consecutive totals per thread and step: a frame of 8M items has 15.6K of them, which took
-    // 34 us with one per thread and 9 us so
+    // 34 us with one per thread and 15 us so
     constexpr int kEach = 8;
     __shared__ unsigned long long s_warp[32];
     __shared__ unsigned long long s_carry;

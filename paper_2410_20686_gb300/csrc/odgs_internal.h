@@ -189,7 +189,8 @@ struct BwdArgs {
 
 cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Header* hdr, int total_trig,
                          uint32_t* dhist, uint4* clear, size_t clear_quads, cudaStream_t st);
-cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st);
+// projected: recorded once the projection (records, pairs, keys) is done, before the colours; or null
+cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, cudaEvent_t projected = nullptr);
 cudaError_t launch_preprocess_bwd(const PreBwdArgs& a, int sh_degree, cudaStream_t st);
 
 int radix_passes(int bits);

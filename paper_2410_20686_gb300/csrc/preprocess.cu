@@ -879,10 +879,14 @@ cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Hea
     return cudaGetLastError();
 }
 
-cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st) {
-    if (a.n == 0) return cudaSuccess;
+cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, cudaEvent_t projected) {
+    if (a.n == 0) return projected ? cudaEventRecord(projected, st) : cudaSuccess;
     const int threads = 256, blocks = (a.n + threads - 1) / threads;
     k_preprocess_geom<<<blocks, threads, 0, st>>>(a);
+    if (projected) {
+        const cudaError_t e = cudaEventRecord(projected, st);
+        if (e != cudaSuccess) return e;
+    }
     switch (sh_degree) {
         case 0: k_preprocess_color<0><<<blocks, threads, 0, st>>>(a); break;
         case 1: k_preprocess_color<1><<<blocks, threads, 0, st>>>(a); break;

@@ -23,10 +23,6 @@ def _ptr(t):
     return C.c_void_p(t.data_ptr()) if t is not None and t.numel() > 0 else C.c_void_p(0)
 
 
-def _stream(device):
-    return C.c_void_p(torch.cuda.current_stream(device).cuda_stream)
-
-
 @dataclass
 class DensifyParams:
     tau_min: float = 2e-5       # App. A.1
@@ -72,7 +68,7 @@ def select(stats: DensifyStats, scales: torch.Tensor, opacity: torch.Tensor,
     lib = L.load()
     prm = params.to_c()
     L.check(lib.odgs_densify_select(_ptr(stats.grad), _ptr(stats.elev), _ptr(stats.count), _ptr(scales),
-                                    _ptr(opacity), int(n), C.byref(prm), _ptr(action), _stream(dev)),
+                                    _ptr(opacity), int(n), C.byref(prm), _ptr(action), L.raw_stream(dev)),
             "odgs_densify_select")
     return action
 
@@ -99,12 +95,12 @@ def apply(means, scales, quats, opacity, sh, action, noise=None, generator=None,
     nbytes = C.c_size_t()
     L.check(lib.odgs_densify_scratch_size(int(n), C.byref(nbytes)), "odgs_densify_scratch_size")
     scratch = torch.empty(max(int(nbytes.value), 16), dtype=torch.uint8, device=dev)
-    n_out = torch.zeros(1, dtype=torch.int32, device=dev)
+    n_out = torch.empty(1, dtype=torch.int32, device=dev)  # always written
     g = L.Gaussians(_ptr(means), _ptr(scales), _ptr(quats), _ptr(opacity), _ptr(sh), int(n))
     o = L.ParamsOut(*[_ptr(t) for t in out])
     L.check(lib.odgs_densify_apply(C.byref(g), int(k), int(bool(raw_params)), _ptr(action), _ptr(noise), C.byref(o),
                                    int(cap),
-                                   _ptr(n_out), _ptr(scratch), C.c_size_t(scratch.numel()), _stream(dev)),
+                                   _ptr(n_out), _ptr(scratch), C.c_size_t(scratch.numel()), L.raw_stream(dev)),
             "odgs_densify_apply")
     m = int(n_out.item())
     if m > cap:  # cannot happen: every Gaussian yields at most two outputs

@@ -31,7 +31,7 @@ def l1_dssim(images, targets, lam: float = 0.2, area_weight: bool = True, wrap_u
     scratch = torch.empty(need, dtype=torch.uint8, device=dev)
     loss = torch.empty(1, dtype=torch.float32, device=dev)  # the first view writes it, the others add
     grads = []
-    stream = C.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
+    stream = L.raw_stream(dev)
     for k, (im, tg) in enumerate(zip(images, targets)):
         for t in (im, tg):
             if t.dtype != torch.float32 or not t.is_contiguous() or t.dim() != 3 or t.shape[0] != 3 or t.device != dev:

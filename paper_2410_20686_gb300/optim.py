@@ -52,5 +52,5 @@ class GaussianAdam:
             groups[k] = L.AdamGroup(_ptr(p).value, _ptr(gr).value, _ptr(m).value, _ptr(v).value, p.numel(),
                                     lr, lr_tail, row, head)
         prm = L.AdamParams(self.betas[0], self.betas[1], self.eps, self.t)
-        stream = C.c_void_p(torch.cuda.current_stream(self.params[0].device).cuda_stream)
+        stream = L.raw_stream(self.params[0].device)
         L.check(L.load().odgs_adam_step(groups, 5, C.byref(prm), stream), "odgs_adam_step")

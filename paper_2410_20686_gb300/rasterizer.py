@@ -145,7 +145,7 @@ class Rasterizer:
         nv = len(views)
         self._ensure_workspace(n, views_c, nv, st_c)
         g = L.Gaussians(_ptr(means), _ptr(scales), _ptr(quats), _ptr(opacity), _ptr(sh), int(n))
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_preprocess(self.ctx, C.byref(g), views_c, nv, C.byref(st_c), _ptr(self.ws),
                                          self.ws.numel(), stream), "odgs_preprocess")
         # the library keeps raw pointers until the backward pass
@@ -158,22 +158,24 @@ class Rasterizer:
         return self._keep
 
     def query_pairs(self) -> int:
+        return self._pairs(self.lib.odgs_query_pairs, "odgs_query_pairs")
+
+    def _pairs(self, call, where) -> int:
         p = C.c_size_t()
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
-        st = self.lib.odgs_query_pairs(self.ctx, C.byref(p), stream)
+        st = call(self.ctx, C.byref(p), L.raw_stream(self.device))
         # capacity and non-finite inputs are reported by status() and do not stop the frame
         if st not in (L.ODGS_OK, L.ODGS_ERR_CAPACITY, L.ODGS_ERR_NONFINITE):
-            L.check(st, "odgs_query_pairs")
+            L.check(st, where)
         return int(p.value)
 
     def bin_sort(self):
         if self.capacity_mode == "query":
-            p = self.query_pairs()
+            p = self._pairs(self.lib.odgs_wait_pairs, "odgs_wait_pairs")
             if p > self.capacity or self.pairs is None:
                 self.reserve_pairs(max(int(p * self.headroom) + 1024, 1024))
         elif self.pairs is None:
             raise RuntimeError("fixed capacity mode: call reserve_pairs() first")
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_bin_sort(self.ctx, _ptr(self.pairs), self.capacity, stream), "odgs_bin_sort")
 
     def render_fwd(self, images=None, want_T=True):
@@ -183,7 +185,7 @@ class Rasterizer:
         Ts = [torch.empty((v.height, v.width), dtype=torch.float32, device=self.device) for v in views] if want_T else None
         img_arr = (C.c_void_p * len(views))(*[im.data_ptr() for im in images])
         T_arr = (C.c_void_p * len(views))(*[t.data_ptr() for t in Ts]) if want_T else None
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_render_fwd(self.ctx, img_arr, T_arr, stream), "odgs_render_fwd")
         return images, Ts
 
@@ -191,7 +193,7 @@ class Rasterizer:
         """Reverse blend: per-(view, Gaussian) screen-space gradients into the workspace."""
         gi = [g.contiguous() for g in grad_images]
         arr = (C.c_void_p * len(gi))(*[g.data_ptr() for g in gi])
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_render_bwd(self.ctx, arr, stream), "odgs_render_bwd")
         self._gi_keep = gi
 
@@ -213,7 +215,7 @@ class Rasterizer:
                     raise ValueError(f"densify.{name} must be a contiguous {dt} tensor of {n} elements on {means.device}")
             gc.densify_grad, gc.densify_elev, gc.densify_count = (_ptr(densify.grad), _ptr(densify.elev),
                                                                   _ptr(densify.count))
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_preprocess_bwd(self.ctx, C.byref(gc), stream), "odgs_preprocess_bwd")
         return grads
 
@@ -223,7 +225,7 @@ class Rasterizer:
 
     def stats(self) -> dict:
         s = L.Stats()
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_frame_stats(self.ctx, C.byref(s), stream), "odgs_frame_stats")
         return dict(pairs=int(s.pairs), pairs_sorted=int(s.pairs_sorted), evals_fwd=int(s.evals_fwd),
                     evals_bwd=int(s.evals_bwd), blended=int(s.blended), entries_tile=int(s.entries_tile),
@@ -231,7 +233,7 @@ class Rasterizer:
 
     def status(self) -> int:
         bits = C.c_uint32()
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_get_status(self.ctx, C.byref(bits), stream), "odgs_get_status")
         return int(bits.value)
 
@@ -250,7 +252,7 @@ class Rasterizer:
         out = dict(depth_keys=torch.empty(n_items, **u32), depth_items=torch.empty(n_items, **u32),
                    pair_tiles=torch.empty(n_pairs, **u32), pair_items=torch.empty(n_pairs, **u32),
                    ranges=torch.empty((n_tiles, 2), **u32))
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_debug_lists(self.ctx, _ptr(out["depth_keys"]), _ptr(out["depth_items"]), n_items,
                                           _ptr(out["pair_tiles"]), _ptr(out["pair_items"]), n_pairs,
                                           _ptr(out["ranges"]), n_tiles, stream), "odgs_debug_lists")
@@ -262,7 +264,7 @@ class Rasterizer:
         float32 (dL/du, dL/dv, dL/da, dL/db, dL/dc, dL/do, dL/dr, dL/dg, dL/db)."""
         n_items = int(self._keep[0].shape[0]) * self.n_views
         out = torch.empty((n_items, 12), dtype=torch.float32, device=self.device)
-        stream = C.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        stream = L.raw_stream(self.device)
         L.check(self.lib.odgs_debug_screen_grads(self.ctx, _ptr(out), n_items, stream), "odgs_debug_screen_grads")
         return out[:, :9].cpu().numpy()
 
@@ -316,6 +318,6 @@ def measure_peaks(device=None) -> dict:
     lib = L.load()
     p = L.Peaks()
     with torch.cuda.device(dev):
-        stream = C.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
+        stream = L.raw_stream(dev)
         L.check(lib.odgs_measure_peaks(C.byref(p), stream), "odgs_measure_peaks")
     return {"ffma_tflops": float(p.ffma_tflops), "ex2_gops": float(p.ex2_gops), "sms": int(p.sms)}
