@@ -482,8 +482,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     if (!rebuild) {
         if (launch_radix_sort(dk, dv, &hdr->n_items, c->geo.n_items, 32, reinterpret_cast<uint32_t*>(w + c->L.sort_hist),
                               reinterpret_cast<uint32_t*>(w + c->L.sort_ctr), reinterpret_cast<uint32_t*>(w + c->L.sort_lb),
-                              &hdr->status, c->num_sms, st, &rb, &c->launches, /*hist_ready=*/true,
-                              c->wait_limit, kDepthLbRegions, /*cleared=*/true) != cudaSuccess)
+                              &hdr->status, c->num_sms, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions, /*cleared=*/true) != cudaSuccess)
             return ODGS_ERR_CUDA;
         c->depth_buf = rb;
     }
@@ -543,8 +542,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     int rp = 0;
     if (launch_radix_sort(pk, pv, &hdr->n_pairs_sort, c->pb_cap, c->geo.key_bits, reinterpret_cast<uint32_t*>(p + c->P.hist),
                           reinterpret_cast<uint32_t*>(p + c->P.ctr), reinterpret_cast<uint32_t*>(p + c->P.lb),
-                          &hdr->status, c->num_sms, st, &rp, &c->launches, /*hist_ready=*/true,
-                          c->wait_limit, kPairLbRegions, /*cleared=*/emits) != cudaSuccess)
+                          &hdr->status, c->num_sms, st, &rp, &c->launches, c->wait_limit, kPairLbRegions, /*cleared=*/emits) != cudaSuccess)
         return ODGS_ERR_CUDA;
     c->sorted_vals = pv[rp];
     c->pair_buf = rp;

@@ -5,10 +5,9 @@
 // Together they give every tile its Gaussians in (depth, index) order, the same order as one
 // stable sort of 64-bit (tile | depth) keys, with far fewer bytes moved.
 //
-// One histogram kernel counts the digits of all passes in a single read of the keys; each
-// pass is then one "onesweep" kernel (Adinets & Merrill 2022): a CTA ranks a 2048- or 4096-key
-// tile in shared memory (warp-level ranking by ballots or a match keeps it stable), publishes its per-digit counts,
-// obtains the exclusive prefix of all earlier tiles by decoupled look-back, and writes its keys
+// The kernels that write the keys count the digits of all passes; each pass is one "onesweep" kernel
+// (Adinets & Merrill 2022): a CTA ranks a 2048- or 4096-key tile in shared memory, publishes its
+// per-digit counts, obtains the exclusive prefix of all earlier tiles by decoupled look-back, and writes its keys
 // digit-run by digit-run (coalesced). The CTAs are persistent (as many as fit on the GPU, each
 // claiming tiles in order), so a sort sized for a capacity far above its keys launches no idle
 // CTAs. Look-back waits are bounded: a CTA that has read the
@@ -23,46 +22,11 @@ namespace odgs {
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItemsMax = 16;  // 4096 keys per CTA for sorts of at least kLargeSort keys, else 2048
-constexpr size_t kLargeSort = 1u << 19;  // measured: the 1M-item depth sort is faster with 4096-key tiles
+constexpr size_t kLargeSort = 1u << 20;  // 1M items by depth: 78 us with 2048-key tiles, 82 with 4096
 constexpr int kRadix = 256;
 constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagPrefix = 2u << 30;
 constexpr uint32_t kCountMask = (1u << 30) - 1u;
-
-__global__ void __launch_bounds__(256) k_radix_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_ptr,
-                                                    int begin_bit, int n_passes, uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[4][kRadix];
-    for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) (&h[0][0])[i] = 0u;
-    __syncthreads();
-    const uint32_t n = *n_ptr;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    // warp-uniform trip count so every lane takes part in the match
-    for (uint32_t base = gwarp * 32u; base < n; base += nwarps * 32u) {
-        const uint32_t idx = base + lane;
-        const bool valid = idx < n;
-        const uint32_t k = valid ? keys[idx] : 0u;
-        // the low digits of the keys (depths, tile ids) are spread over many bins: one shared
-        // atomic per key; the top digit takes few values (the exponent byte of a positive float
-        // depth), so equal digits of the warp are counted with one atomic
-        for (int p = 0; p + 1 < n_passes; ++p) {
-            const uint32_t d = (k >> (begin_bit + 8 * p)) & 0xFFu;
-            if (valid) atomicAdd(&h[p][d], 1u);
-        }
-        {
-            const int p = n_passes - 1;
-            const uint32_t d = (k >> (begin_bit + 8 * p)) & 0xFFu;
-            const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 0x100u);
-            if (valid && lane == (uint32_t)(__ffs(peers) - 1)) atomicAdd(&h[p][d], (uint32_t)__popc(peers));
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n_passes * kRadix; i += blockDim.x) {
-        uint32_t c = (&h[0][0])[i];
-        if (c) atomicAdd(hist + i, c);
-    }
-}
 
 // Block-wide exclusive scan of one value per thread (256 threads).
 __device__ __forceinline__ uint32_t block_excl_scan_256(uint32_t v, uint32_t* s_warp, uint32_t& total) {
@@ -91,15 +55,16 @@ template <int kSortItems>
 __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                                          uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                          const uint32_t* __restrict__ n_ptr, int shift,
-                                                         int bits, int use_match, const uint32_t* __restrict__ hist,
+                                                         int bits, const uint32_t* __restrict__ hist,
                                                          uint32_t* lookback, uint32_t* tile_ctr, uint32_t* status,
                                                          uint32_t wait_limit) {
+    extern __shared__ uint2 s_dyn[];
+    uint2 (*s_cell)[kRadix] = reinterpret_cast<uint2 (*)[kRadix]>(s_dyn);  // [warps] lanes, count
+    uint32_t* s_keys = reinterpret_cast<uint32_t*>(s_dyn + kSortWarps * kRadix);
+    uint32_t* s_vals = s_keys + kSortThreads * kSortItems;
     __shared__ uint32_t s_tile;
-    __shared__ uint32_t s_warp_hist[kSortWarps][kRadix];
     __shared__ uint32_t s_digit_excl[kRadix];
     __shared__ uint32_t s_base[kRadix];
-    __shared__ uint32_t s_keys[kSortThreads * kSortItems];
-    __shared__ uint32_t s_vals[kSortThreads * kSortItems];
     __shared__ uint32_t s_scan[kSortWarps];
     __shared__ uint32_t s_gex[kRadix];
 
@@ -120,7 +85,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
     const uint32_t per_cta = (uint32_t)(kSortThreads * kSortItems);
     for (;;) {
         if (tid == 0) s_tile = atomicAdd(tile_ctr, 1u);
-        for (int i = tid; i < kSortWarps * kRadix; i += kSortThreads) (&s_warp_hist[0][0])[i] = 0u;
+        for (int i = tid; i < kSortWarps * kRadix; i += kSortThreads) s_dyn[i] = make_uint2(0u, 0u);
         __syncthreads();
         const uint32_t tile = s_tile;
         const uint32_t base = tile * per_cta;
@@ -141,28 +106,18 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
             const uint32_t idx = wbase + (uint32_t)i * 32u + (uint32_t)lane;
             const bool valid = idx < n;
             const uint32_t d = (key[i] >> shift) & mask;
-            // lanes holding the same digit: a warp match costs more the more distinct digits the
-            // warp holds, so it ranks the last (most significant) pass, where they are few; the
-            // others take one ballot per digit bit (an invalid lane's peers are never used)
-            uint32_t peers;
-            if (use_match) {
-                peers = __match_any_sync(0xffffffffu, valid ? d : (0x100u | (uint32_t)lane));
-            } else {
-                peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    if (b < bits) {
-                        const bool bit = (d >> b) & 1u;
-                        const uint32_t bb = __ballot_sync(0xffffffffu, bit);
-                        peers &= bit ? bb : ~bb;
-                    }
-                }
-            }
-            const uint32_t before = valid ? s_warp_hist[warp][d] : 0u;
+            // lanes holding the same digit: each sets its bit in the digit's cell of the warp. A
+            // ballot per digit bit took three times the instructions: 23.3M pairs by tile and 6M items
+            // by depth, all passes of 8 views, 4293 -> 3520 us; 1M items and 2.3M pairs 138 -> 128 us
+            uint2* cell = &s_cell[warp][d];
+            if (valid) atomicOr(&cell->x, 1u << lane);
             __syncwarp();
-            if (valid && lane == (uint32_t)(__ffs(peers) - 1)) s_warp_hist[warp][d] = before + (uint32_t)__popc(peers);
+            const uint2 c = valid ? *cell : make_uint2(0u, 0u);
             __syncwarp();
-            rank[i] = before + (uint32_t)__popc(peers & lt);
+            const uint32_t below = c.x & lt;
+            if (valid && below == 0u) *cell = make_uint2(0u, c.y + (uint32_t)__popc(c.x));  // the first of them
+            __syncwarp();
+            rank[i] = c.y + (uint32_t)__popc(below);
         }
         __syncthreads();
         // per digit (one thread each): exclusive prefix over warps, CTA count
@@ -171,8 +126,8 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
             const int d = tid;
 #pragma unroll
             for (int w = 0; w < kSortWarps; ++w) {
-                uint32_t c = s_warp_hist[w][d];
-                s_warp_hist[w][d] = cnt;
+                uint32_t c = s_cell[w][d].y;
+                s_cell[w][d].y = cnt;
                 cnt += c;
             }
         }
@@ -215,7 +170,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
             const uint32_t idx = wbase + (uint32_t)i * 32u + (uint32_t)lane;
             if (idx < n) {
                 const uint32_t d = (key[i] >> shift) & mask;
-                const uint32_t pos = s_digit_excl[d] + s_warp_hist[warp][d] + rank[i];
+                const uint32_t pos = s_digit_excl[d] + s_cell[warp][d].y + rank[i];
                 s_keys[pos] = key[i];
                 s_vals[pos] = val[i];
             }
@@ -233,8 +188,12 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
         }
         if ((n + per_cta - 1) / per_cta <= gridDim.x) break;
         // the next tile's first barrier orders these reads of s_keys, s_vals and s_base before
-        // its writes; s_tile and s_warp_hist are not read here
+        // its writes; s_tile and s_cell are not read here
     }
+}
+
+constexpr size_t onesweep_smem(int items) {
+    return kSortWarps * kRadix * sizeof(uint2) + 2 * sizeof(uint32_t) * (size_t)kSortThreads * items;
 }
 
 int radix_passes(int bits) { return (bits + 7) / 8; }
@@ -247,12 +206,12 @@ size_t radix_lookback_words(size_t max_items) {
 }
 
 // Sorts (k[0], v[0]) by key bits [0, bits); returns the buffer index (0 or 1) that holds the
-// result. scratch: hist [4 * 256] + tile counters [4] + lookback [radix_lookback_words]. With
-// hist_ready the digit histograms of all passes are already in hist (counted by the producer).
+// result. hist: the digit counts of all passes, [passes][256], from the kernels that wrote the keys.
+// scratch: tile counters [4] + lookback [radix_lookback_words].
 cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_ptr, size_t max_items, int bits,
                               uint32_t* hist, uint32_t* tile_ctrs, uint32_t* lookback, uint32_t* status, int num_sms,
-                              cudaStream_t st, int* result_buf, int* launches, bool hist_ready, uint32_t wait_limit,
-                              int lb_regions, bool cleared) {
+                              cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit, int lb_regions,
+                              bool cleared) {
     const int passes = radix_passes(bits);
     *result_buf = 0;
     if (passes == 0 || max_items == 0) return cudaSuccess;
@@ -262,20 +221,14 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
     const bool ctr_with_lb = lb_regions >= passes &&
                              reinterpret_cast<uint8_t*>(lookback) == reinterpret_cast<uint8_t*>(tile_ctrs) + kCtrBytes;
     if (!ctr_with_lb && !cleared && (e = cudaMemsetAsync(tile_ctrs, 0, sizeof(uint32_t) * 4, st)) != cudaSuccess) return e;
-    if (!hist_ready) {
-        if ((e = cudaMemsetAsync(hist, 0, sizeof(uint32_t) * 4 * kRadix, st)) != cudaSuccess) return e;
-        int hblocks = (int)min((max_items + 255) / 256, (size_t)num_sms * 8);
-        hblocks = max(hblocks, 1);
-        k_radix_hist<<<hblocks, 256, 0, st>>>(k[0], n_ptr, 0, passes, hist);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        *launches += 1;
-    }
     static bool carveout_set = false;  // all of the SM's shared memory for the onesweep CTAs
     if (!carveout_set) {
         cudaFuncSetAttribute(k_onesweep<kSortItemsMax>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
         cudaFuncSetAttribute(k_onesweep<kSortItemsMax / 2>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(k_onesweep<kSortItemsMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)onesweep_smem(kSortItemsMax));
         carveout_set = true;
     }
     const bool large = max_items >= kLargeSort;
@@ -288,9 +241,9 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
     if (res == 0) {
         int per_sm = 0;
         if (large)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<kSortItemsMax>, kSortThreads, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<kSortItemsMax>, kSortThreads, onesweep_smem(kSortItemsMax));
         else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<kSortItemsMax / 2>, kSortThreads, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<kSortItemsMax / 2>, kSortThreads, onesweep_smem(kSortItemsMax / 2));
         res = max(per_sm, 1);
     }
     const int grid = max(min(tiles, res * num_sms), 1);
@@ -308,12 +261,12 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
         uint32_t* lb = regions ? lookback + (size_t)p * lb_words : lookback;
         if (!regions && (e = cudaMemsetAsync(lb, 0, sizeof(uint32_t) * lb_words, st)) != cudaSuccess) return e;
         if (large)
-            k_onesweep<kSortItemsMax><<<grid, kSortThreads, 0, st>>>(
-                k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits, p == passes - 1 ? 1 : 0,
+            k_onesweep<kSortItemsMax><<<grid, kSortThreads, onesweep_smem(kSortItemsMax), st>>>(
+                k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits,
                 hist + p * kRadix, lb, tile_ctrs + p, status, wait_limit);
         else
-            k_onesweep<kSortItemsMax / 2><<<grid, kSortThreads, 0, st>>>(
-                k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits, p == passes - 1 ? 1 : 0,
+            k_onesweep<kSortItemsMax / 2><<<grid, kSortThreads, onesweep_smem(kSortItemsMax / 2), st>>>(
+                k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits,
                 hist + p * kRadix, lb, tile_ctrs + p, status, wait_limit);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *launches += 1;

@@ -143,7 +143,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
     if (launch_preprocess(a, st.sh_degree, strm) != cudaSuccess) return ODGS_ERR_CUDA;
     int rb = 0;
     if (launch_radix_sort(dk, dv, &hdr->n_items, n, 32, d_hist, d_ctr, d_lb, &hdr->status, num_sms, strm, &rb,
-                          &launches, /*hist_ready=*/true, kDefaultWaitLimit) != cudaSuccess)
+                          &launches, kDefaultWaitLimit) != cudaSuccess)
         return ODGS_ERR_CUDA;
     BinArgs b{};
     b.sorted_idx = dv[rb]; b.rect = rect; b.rect2 = rect2; b.views = vd; b.n_per_view = g->n > 0 ? g->n : 1;
@@ -155,7 +155,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
     if (launch_binning(b, strm, &launches) != cudaSuccess) return ODGS_ERR_CUDA;
     int rp = 0;
     if (launch_radix_sort(pk, pv, &hdr->n_pairs_sort, cap, key_bits, p_hist, p_ctr, p_lb, &hdr->status, num_sms,
-                          strm, &rp, &launches, /*hist_ready=*/true, kDefaultWaitLimit) != cudaSuccess)
+                          strm, &rp, &launches, kDefaultWaitLimit) != cudaSuccess)
         return ODGS_ERR_CUDA;
     if (launch_tile_ranges(pk[rp], hdr, ranges, tiles, cap, num_sms, strm, &launches) != cudaSuccess)
         return ODGS_ERR_CUDA;
