@@ -223,14 +223,11 @@ struct odgs_ctx {
     // from and joined back to the caller's stream by events)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // odgs_wait_pairs: recorded after the projection (once a first call has made it), and the header's
-    // copy in page-locked host memory
+    // odgs_wait_pairs: recorded after the projection (once a first call has made it)
     cudaEvent_t ev_pairs = nullptr;
     bool pairs_recorded = false;
-    Header* host = nullptr;
     ~odgs_ctx() {
         if (ev_pairs) cudaEventDestroy(ev_pairs);
-        if (host) cudaFreeHost(host);
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
         if (side) cudaStreamDestroy(side);
@@ -408,19 +405,19 @@ odgs_status odgs_wait_pairs(odgs_ctx* c, size_t* pairs, void* stream) {
     if (!c || !pairs) return ODGS_ERR_INVALID_ARG;
     if (c->stage < 1) return ODGS_ERR_STATE;
     if (!c->ev_pairs) {  // the first call makes what the next preprocess records
-        if (!make_side(c) || (!c->host && cudaHostAlloc(reinterpret_cast<void**>(&c->host), sizeof(Header), 0) != cudaSuccess) ||
-            cudaEventCreateWithFlags(&c->ev_pairs, cudaEventDisableTiming) != cudaSuccess) {
+        if (!make_side(c) || cudaEventCreateWithFlags(&c->ev_pairs, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
             c->ev_pairs = nullptr;
         }
     }
     // later stages report what they found, which only the stream's own order shows
     if (c->stage > 1 || !c->pairs_recorded) return odgs_query_pairs(c, pairs, stream);
+    Header h;
     if (cudaStreamWaitEvent(c->side, c->ev_pairs, 0) != cudaSuccess ||
-        cudaMemcpyAsync(c->host, c->ws + c->L.hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->side) != cudaSuccess ||
+        cudaMemcpyAsync(&h, c->ws + c->L.hdr, sizeof(Header), cudaMemcpyDeviceToHost, c->side) != cudaSuccess ||
         cudaStreamSynchronize(c->side) != cudaSuccess)
         return ODGS_ERR_CUDA;
-    return report_pairs(c, *c->host, pairs);
+    return report_pairs(c, h, pairs);
 }
 
 odgs_status odgs_get_status(odgs_ctx* c, uint32_t* bits, void* stream) {
