@@ -312,6 +312,7 @@ static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
     a.dkey = reinterpret_cast<uint32_t*>(w + c->L.dkey0);
     a.dval = reinterpret_cast<uint32_t*>(w + c->L.dval0);
     a.dhist = dhist;
+    a.num_sms = c->num_sms;
     if (c->L.truncate) {
         a.dbucket = w + c->L.dbucket;
         uint32_t rn;

@@ -68,6 +68,7 @@ struct PreArgs {
     uint32_t* dhist;  // [4][256] digit histograms of dkey (zeroed by k_setup), for the depth sort
     uint8_t* dbucket;  // per item its depth bucket (saturation.cu), or null
     uint32_t cut_base;  // depth_bucket's origin
+    int num_sms;
     Header* hdr;
 };
 

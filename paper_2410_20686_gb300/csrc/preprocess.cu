@@ -458,6 +458,11 @@ __global__ void __launch_bounds__(256, 3) k_preprocess_geom(PreArgs a) {
 // View-dependent colour of every visible item: max(0, sum_k sh_k Y_k(d) + 0.5) with d the unit
 // vector from the camera centre to the mean in world space. A separate streaming kernel, so the
 // 48 SH coefficients do not weigh on the geometry kernel's registers.
+// A CTA takes many Gaussians: at its end it adds its digit counts to the 1024 global ones, and with a
+// CTA per 256 Gaussians those atomics, all to the same addresses, cost as much as the coefficients'
+// fetch. Three CTAs per SM (80 registers); measured (us) with a CTA per 256 Gaussians and so: 1M
+// Gaussians, one view 57 -> 50 (35 at the copy bandwidth); 1M, six views 107 -> 74; 500K, 16 views
+// 103 -> 77; 3M, 2 views 167 -> 136. Coefficient rows staged through shared memory: 48, 73, 84, 132.
 template <int DEG>
 __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
     constexpr int K = (DEG + 1) * (DEG + 1);
@@ -466,39 +471,41 @@ __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
     __shared__ uint32_t s_dh[4][256];
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) s_dh[i >> 8][i & 255] = 0u;
     __syncthreads();
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    for (int v = 0; v < a.n_views && g < a.n; ++v) {
-        const uint32_t key = a.dkey[(size_t)v * a.n + g];
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.n; g += gridDim.x * blockDim.x) {
+        bool seen = false;  // in some view
+        for (int v = 0; v < a.n_views; ++v) {
+            const uint32_t key = a.dkey[(size_t)v * a.n + g];
+            seen |= key != 0xFFFFFFFFu;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) atomicAdd(&s_dh[p][(key >> (8 * p)) & 0xFFu], 1u);
+            for (int p = 0; p < 4; ++p) atomicAdd(&s_dh[p][(key >> (8 * p)) & 0xFFu], 1u);
+        }
+        if (!seen) continue;
+        const float m0 = __ldg(a.means + 3 * g), m1 = __ldg(a.means + 3 * g + 1), m2 = __ldg(a.means + 3 * g + 2);
+        float shc[16][3];
+        load_sh<DEG>(a.sh, a.sh_coeffs, g, shc);
+        for (int v = 0; v < a.n_views; ++v) {
+            const size_t item = (size_t)v * a.n + g;
+            if (a.dkey[item] == 0xFFFFFFFFu) continue;  // culled in this view
+            const ViewDev& V = a.views[v];
+            const float dx = m0 - V.cam[0], dy = m1 - V.cam[1], dz = m2 - V.cam[2];
+            const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
+            float Y[16];
+            sh_basis<DEG>(dx * il, dy * il, dz * il, Y);
+            float rgb[3];
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) {
+                float acc = 0.5f;
+#pragma unroll
+                for (int k = 0; k < K; ++k) acc = fmaf(shc[k][ch], Y[k], acc);
+                rgb[ch] = fmaxf(acc, 0.f);
+            }
+            a.rec_c[item] = make_float4(rgb[0], rgb[1], rgb[2], 0.f);
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
         const uint32_t c = s_dh[i >> 8][i & 255];
         if (c) atomicAdd(a.dhist + i, c);
-    }
-    if (g >= a.n) return;
-    const float m0 = __ldg(a.means + 3 * g), m1 = __ldg(a.means + 3 * g + 1), m2 = __ldg(a.means + 3 * g + 2);
-    bool loaded = false;
-    float shc[16][3];
-    for (int v = 0; v < a.n_views; ++v) {
-        const size_t item = (size_t)v * a.n + g;
-        if (a.dkey[item] == 0xFFFFFFFFu) continue;  // culled in this view
-        if (!loaded) { load_sh<DEG>(a.sh, a.sh_coeffs, g, shc); loaded = true; }
-        const ViewDev& V = a.views[v];
-        const float dx = m0 - V.cam[0], dy = m1 - V.cam[1], dz = m2 - V.cam[2];
-        const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-        float Y[16];
-        sh_basis<DEG>(dx * il, dy * il, dz * il, Y);
-        float rgb[3];
-#pragma unroll
-        for (int ch = 0; ch < 3; ++ch) {
-            float acc = 0.5f;
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc = fmaf(shc[k][ch], Y[k], acc);
-            rgb[ch] = fmaxf(acc, 0.f);
-        }
-        a.rec_c[item] = make_float4(rgb[0], rgb[1], rgb[2], 0.f);
     }
 }
 
@@ -887,11 +894,12 @@ cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, 
         const cudaError_t e = cudaEventRecord(projected, st);
         if (e != cudaSuccess) return e;
     }
+    const int grid = min(blocks, 3 * a.num_sms);
     switch (sh_degree) {
-        case 0: k_preprocess_color<0><<<blocks, threads, 0, st>>>(a); break;
-        case 1: k_preprocess_color<1><<<blocks, threads, 0, st>>>(a); break;
-        case 2: k_preprocess_color<2><<<blocks, threads, 0, st>>>(a); break;
-        default: k_preprocess_color<3><<<blocks, threads, 0, st>>>(a); break;
+        case 0: k_preprocess_color<0><<<grid, threads, 0, st>>>(a); break;
+        case 1: k_preprocess_color<1><<<grid, threads, 0, st>>>(a); break;
+        case 2: k_preprocess_color<2><<<grid, threads, 0, st>>>(a); break;
+        default: k_preprocess_color<3><<<grid, threads, 0, st>>>(a); break;
     }
     return cudaGetLastError();
 }

@@ -139,6 +139,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
     a.st.checked = st.checked;
     a.rec_a = rec_a; a.rec_b = rec_b; a.rec_c = rec_c; a.rect = rect; a.rect2 = rect2; a.dkey = dk[0]; a.dval = dv[0];
     a.dhist = d_hist;
+    a.num_sms = num_sms;
     a.hdr = hdr;
     if (launch_preprocess(a, st.sh_degree, strm) != cudaSuccess) return ODGS_ERR_CUDA;
     int rb = 0;
