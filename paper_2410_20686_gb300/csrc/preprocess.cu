@@ -223,6 +223,47 @@ __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int stride
     }
 }
 
+// A warp's rows of SH coefficients (32 Gaussians) in shared memory. Rows of 16-byte chunks with no
+// coefficients beyond the degree's are copied with consecutive lanes on consecutive chunks, so a warp
+// instruction touches four 128-byte lines where a thread that reads its own row touches 32; the rows lie
+// an odd number of chunks apart, so that the lanes' reads of their own rows hit distinct banks.
+template <int DEG>
+struct ShRows {
+    static constexpr int K = (DEG + 1) * (DEG + 1);
+    static constexpr int kChunks = 3 * K / 4;      // 3 (degree 1) or 12 (degree 3)
+    static constexpr int kPitch = kChunks | 1;
+};
+template <int DEG>
+__device__ __forceinline__ void sh_rows_fetch(float4* rows, const float* __restrict__ sh, int g0, unsigned mask, int lane) {
+    using R = ShRows<DEG>;
+    const float4* src = reinterpret_cast<const float4*>(sh) + (size_t)g0 * R::kChunks;
+#pragma unroll
+    for (int i = 0; i < R::kChunks; ++i) {
+        const int t = lane + 32 * i, row = t / R::kChunks, c = t - row * R::kChunks;
+        if ((mask >> row) & 1u) {
+            const unsigned d = (unsigned)__cvta_generic_to_shared(rows + row * R::kPitch + c);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src + t) : "memory");
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void sh_rows_wait() {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+}
+// max(0, sum_k sh_k Y_k + 0.5) before the clamp, from a staged row.
+template <int DEG>
+__device__ __forceinline__ void sh_row_colour(const float4* row, const float Y[16], float col[3]) {
+    col[0] = col[1] = col[2] = 0.5f;
+#pragma unroll
+    for (int i = 0; i < ShRows<DEG>::kChunks; ++i) {
+        const float4 q4 = row[i];
+        const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) col[(4 * i + r) % 3] = fmaf(q[r], Y[(4 * i + r) / 3], col[(4 * i + r) % 3]);
+    }
+}
+
 // ------------------------------------------------------------------ forward projection
 
 // Footprints with at most this many row bands are counted by their own thread; larger ones (the
@@ -515,11 +556,26 @@ __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
 // the direction's gradient) and forms dL/dsh = m_c dL/drgb_c Y_k when it writes them (m_c = 0 for
 // a clamped channel), so neither the 48 coefficients nor 48 accumulators stay in registers.
 // Frames of several views accumulate dL/dsh over the views in registers.
-template <int DEG, bool ONE>
-__global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
+// STAGED: the coefficient rows and the rows of their gradients go through shared memory (ShRows), so that
+// the global accesses of a warp are consecutive; a thread per row reads and writes 192 bytes apart, which
+// bound the kernel by the L1 (76 % busy) at 45 % of the DRAM bandwidth. Four CTAs per SM (128 registers; the
+// kernel of several views spills 228 bytes, and with three CTAs takes 312, 218 and 1639 us below). Measured
+// (us), unstaged and staged: 1M Gaussians, one view 111 -> 83 (75 at the copy bandwidth); 500K, 16 views
+// 357 -> 319; 1M, six views 240 -> 229; 3M, eight views in four groups 1580 -> 1452.
+template <int DEG, bool ONE, bool STAGED>
+__global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
     constexpr int K = (DEG + 1) * (DEG + 1);
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= a.n) return;
+    using R = ShRows<DEG>;
+    extern __shared__ float4 s_rows[];
+    const int lane = threadIdx.x & 31;
+    float4* rows = s_rows + (threadIdx.x >> 5) * 32 * R::kPitch;
+    float4* row = rows + lane * R::kPitch;
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
+    // lanes past the end run along (as Gaussian 0) where the warp works together, and write nothing
+    const bool act = gt < a.n;
+    if (!STAGED && !act) return;
+    const int g = act ? gt : 0;
+    if (STAGED && !ONE) sh_rows_fetch<DEG>(rows, a.sh, gt - lane, __ballot_sync(0xffffffffu, act), lane);
     const float m0 = __ldg(a.means + 3 * g), m1 = __ldg(a.means + 3 * g + 1), m2 = __ldg(a.means + 3 * g + 2);
     float s[3] = {__ldg(a.scales + 3 * g), __ldg(a.scales + 3 * g + 1), __ldg(a.scales + 3 * g + 2)};
     if (a.raw) {
@@ -553,9 +609,19 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
         st_count = a.d_count[g];
     }
     const uint32_t st_count0 = st_count;
+    // the next view's accumulators load while this view's are used: most items of a frame of many
+    // views have none, and their views would be one load's latency each
+    float4 n0 = a.acc[3 * (size_t)g], n1 = a.acc[3 * (size_t)g + 1], n2 = a.acc[3 * (size_t)g + 2];
+    if (STAGED && ONE)
+        sh_rows_fetch<DEG>(rows, a.sh, gt - lane,
+                           __ballot_sync(0xffffffffu, act && (n1.z != 0.f || n1.w != 0.f || n2.x != 0.f)), lane);
     for (int v = 0; v < a.n_views; ++v) {
         const size_t item = (size_t)v * a.n + g;
-        const float4 g0 = a.acc[3 * item], g1 = a.acc[3 * item + 1], g2 = a.acc[3 * item + 2];
+        const float4 g0 = n0, g1 = n1, g2 = n2;
+        if (!ONE && v + 1 < a.n_views) {
+            const float4* nx = a.acc + 3 * (item + (size_t)a.n);
+            n0 = nx[0]; n1 = nx[1]; n2 = nx[2];
+        }
         if (a.d_count && a.rect[item].y > 0u) {
             // visible in view v: ERP-mean gradient in [-1, 1] image units, and 1 - cos(theta)
             // as t_y^2 / (r (r + rho)), free of the cancellation of 1 - rho / r
@@ -678,7 +744,7 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
 
     }
 
-    if (a.d_count && st_count != st_count0) {  // this thread owns Gaussian g
+    if (a.d_count && act && st_count != st_count0) {  // this thread owns Gaussian g
         a.d_grad[g] = st_grad;
         a.d_elev[g] = st_elev;
         a.d_count[g] = st_count;
@@ -716,6 +782,7 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
     float ysh[ONE ? 16 : 1], msh[3] = {0.f, 0.f, 0.f};  // one view: dL/dsh[k][c] = msh[c] ysh[k]
 #pragma unroll
     for (int k = 0; k < (ONE ? 16 : 1); ++k) ysh[k] = 0.f;
+    if (STAGED) sh_rows_wait();
     if (ONE && any) {
         const float4 g1 = a.acc[1 + 3 * (size_t)g], g2 = a.acc[2 + 3 * (size_t)g];
         if (g1.z != 0.f || g1.w != 0.f || g2.x != 0.f) {
@@ -735,8 +802,8 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
 #pragma unroll
             for (int i = 0; i < (K * 3 + 3) / 4; ++i) {
                 float q[4];
-                if (vec) {
-                    const float4 t4 = __ldg(reinterpret_cast<const float4*>(shg) + i);
+                if (STAGED || vec) {
+                    const float4 t4 = STAGED ? row[i] : __ldg(reinterpret_cast<const float4*>(shg) + i);
                     q[0] = t4.x; q[1] = t4.y; q[2] = t4.z; q[3] = t4.w;
                 } else {
 #pragma unroll
@@ -757,8 +824,8 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
 #pragma unroll
                 for (int i = 0; i < (K * 3 + 3) / 4; ++i) {
                     float q[4];
-                    if (vec) {
-                        const float4 t4 = __ldg(reinterpret_cast<const float4*>(shg) + i);
+                    if (STAGED || vec) {
+                        const float4 t4 = STAGED ? row[i] : __ldg(reinterpret_cast<const float4*>(shg) + i);
                         q[0] = t4.x; q[1] = t4.y; q[2] = t4.z; q[3] = t4.w;
                     } else {
 #pragma unroll
@@ -782,11 +849,16 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
         }
     }
     if (!ONE && any) {
-        float shc[16][3];
-        load_sh<DEG>(a.sh, a.sh_coeffs, g, shc);
+        float shc[STAGED ? 1 : 16][3];
+        if (!STAGED) load_sh<DEG>(a.sh, a.sh_coeffs, g, reinterpret_cast<float(*)[3]>(shc));
+        n1 = a.acc[3 * (size_t)g + 1], n2 = a.acc[3 * (size_t)g + 2];
         for (int v = 0; v < a.n_views; ++v) {
             const size_t item = (size_t)v * a.n + g;
-            const float4 g1 = a.acc[3 * item + 1], g2 = a.acc[3 * item + 2];
+            const float4 g1 = n1, g2 = n2;
+            if (v + 1 < a.n_views) {
+                const float4* nx = a.acc + 3 * (item + (size_t)a.n);
+                n1 = nx[1]; n2 = nx[2];
+            }
             if (g1.z == 0.f && g1.w == 0.f && g2.x == 0.f) continue;
             const ViewDev& V = a.views[v];
             const float vx = m0 - V.cam[0], vy = m1 - V.cam[1], vz = m2 - V.cam[2];
@@ -798,16 +870,34 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
             float wsum[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) wsum[k] = 0.f;
+            if (STAGED) {
+                float col[3], mc[3];
+                sh_row_colour<DEG>(row, Y, col);
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) {
-                float acc = 0.5f;
+                for (int ch = 0; ch < 3; ++ch) mc[ch] = col[ch] < 0.f ? 0.f : drgb[ch];  // clamped channels
 #pragma unroll
-                for (int k = 0; k < K; ++k) acc = fmaf(shc[k][ch], Y[k], acc);
-                if (acc < 0.f) continue;  // clamped channel
+                for (int i = 0; i < R::kChunks; ++i) {
+                    const float4 q4 = row[i];
+                    const float q[4] = {q4.x, q4.y, q4.z, q4.w};
 #pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    gsh[ONE ? 0 : k][ch] += drgb[ch] * Y[k];
-                    wsum[k] += drgb[ch] * shc[k][ch];
+                    for (int r = 0; r < 4; ++r) {
+                        const int e = 4 * i + r;
+                        wsum[e / 3] = fmaf(mc[e % 3], q[r], wsum[e / 3]);
+                        gsh[ONE ? 0 : e / 3][e % 3] = fmaf(mc[e % 3], Y[e / 3], gsh[ONE ? 0 : e / 3][e % 3]);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch) {
+                    float acc = 0.5f;
+#pragma unroll
+                    for (int k = 0; k < K; ++k) acc = fmaf(shc[STAGED ? 0 : k][ch], Y[k], acc);
+                    if (acc < 0.f) continue;  // clamped channel
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        gsh[ONE ? 0 : k][ch] += drgb[ch] * Y[k];
+                        wsum[k] += drgb[ch] * shc[STAGED ? 0 : k][ch];
+                    }
                 }
             }
             if (DEG > 0) {
@@ -829,6 +919,35 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
         const float o = sigmoid_act(__ldg(a.opacity + g));
         gop *= o * (1.f - o);
     }
+    if (STAGED) {
+        // the SH gradients: each lane its row into shared memory, then the warp all rows in order
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < R::kChunks; ++i) {
+            float q[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int kk = (4 * i + r) / 3, ch = (4 * i + r) % 3;
+                q[r] = ONE ? msh[ch] * ysh[ONE ? kk : 0] : gsh[ONE ? 0 : kk][ch];
+            }
+            row[i] = make_float4(q[0], q[1], q[2], q[3]);
+        }
+        const unsigned valid = __ballot_sync(0xffffffffu, act && (any || !a.accumulate));  // rows to write
+        __syncwarp();
+        float4* dst = reinterpret_cast<float4*>(a.g_sh) + (size_t)(gt - lane) * R::kChunks;
+#pragma unroll
+        for (int i = 0; i < R::kChunks; ++i) {
+            const int t = lane + 32 * i, rr = t / R::kChunks;
+            if (!((valid >> rr) & 1u)) continue;
+            float4 q = rows[rr * R::kPitch + (t - rr * R::kChunks)];
+            if (a.accumulate) {
+                const float4 o = dst[t];
+                q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w;
+            }
+            dst[t] = q;
+        }
+        if (!act) return;
+    }
     // write (or accumulate) the parameter gradients
     float* pm = a.g_means + 3 * g;
     float* ps = a.g_scales + 3 * g;
@@ -841,6 +960,7 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) pq[i] += gq[i];
         a.g_opacity[g] += gop;
+        if (STAGED) return;
 #pragma unroll
         for (int k = 0; k < K; ++k)
 #pragma unroll
@@ -850,6 +970,7 @@ __global__ void __launch_bounds__(128) k_preprocess_bwd(PreBwdArgs a) {
         for (int i = 0; i < 3; ++i) { pm[i] = gm[i]; ps[i] = gs[i]; }
         reinterpret_cast<float4*>(pq)[0] = make_float4(gq[0], gq[1], gq[2], gq[3]);
         a.g_opacity[g] = gop;
+        if (STAGED) return;
         if ((a.sh_coeffs * 3) % 4 == 0 && (K * 3) % 4 == 0) {
             float4* p4 = reinterpret_cast<float4*>(psh);
 #pragma unroll
@@ -886,6 +1007,10 @@ cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Hea
     return cudaGetLastError();
 }
 
+// Rows that ShRows can hold: whole 16-byte chunks (16-byte aligned, as the argument checks ask), and none
+// of coefficients above the degree.
+static bool stages_rows(int deg, int sh_coeffs) { return (deg == 1 || deg == 3) && sh_coeffs == (deg + 1) * (deg + 1); }
+
 cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, cudaEvent_t projected) {
     if (a.n == 0) return projected ? cudaEventRecord(projected, st) : cudaSuccess;
     const int threads = 256, blocks = (a.n + threads - 1) / threads;
@@ -904,20 +1029,31 @@ cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, 
     return cudaGetLastError();
 }
 
+template <int DEG, bool STAGED>
+static void launch_bwd(const PreBwdArgs& a, cudaStream_t st) {
+    const int threads = 128, blocks = (a.n + threads - 1) / threads;
+    const size_t bytes = STAGED ? (size_t)threads * ShRows<DEG>::kPitch * sizeof(float4) : 0;
+    if (a.n_views == 1)
+        k_preprocess_bwd<DEG, true, STAGED><<<blocks, threads, bytes, st>>>(a);
+    else
+        k_preprocess_bwd<DEG, false, STAGED><<<blocks, threads, bytes, st>>>(a);
+}
+
 cudaError_t launch_preprocess_bwd(const PreBwdArgs& a, int sh_degree, cudaStream_t st) {
     if (a.n == 0) return cudaSuccess;
-    int threads = 128, blocks = (a.n + threads - 1) / threads;
-    const bool one = a.n_views == 1;
-    switch (sh_degree) {
-        case 0: one ? k_preprocess_bwd<0, true><<<blocks, threads, 0, st>>>(a)
-                    : k_preprocess_bwd<0, false><<<blocks, threads, 0, st>>>(a); break;
-        case 1: one ? k_preprocess_bwd<1, true><<<blocks, threads, 0, st>>>(a)
-                    : k_preprocess_bwd<1, false><<<blocks, threads, 0, st>>>(a); break;
-        case 2: one ? k_preprocess_bwd<2, true><<<blocks, threads, 0, st>>>(a)
-                    : k_preprocess_bwd<2, false><<<blocks, threads, 0, st>>>(a); break;
-        default: one ? k_preprocess_bwd<3, true><<<blocks, threads, 0, st>>>(a)
-                     : k_preprocess_bwd<3, false><<<blocks, threads, 0, st>>>(a); break;
-    }
+    const bool whole = stages_rows(sh_degree, a.sh_coeffs);
+    if (sh_degree == 3 && whole)
+        launch_bwd<3, true>(a, st);
+    else if (sh_degree == 3)
+        launch_bwd<3, false>(a, st);
+    else if (sh_degree == 2)
+        launch_bwd<2, false>(a, st);
+    else if (sh_degree == 1 && whole)
+        launch_bwd<1, true>(a, st);
+    else if (sh_degree == 1)
+        launch_bwd<1, false>(a, st);
+    else
+        launch_bwd<0, false>(a, st);
     return cudaGetLastError();
 }
 
