@@ -134,6 +134,14 @@ odgs_status odgs_loss_l1_dssim(const float *image, const float *target, int widt
                                const odgs_loss_params *p, float *grad, float *loss, void *scratch,
                                size_t scratch_bytes, void *stream);
 
+/* The (weighted) L1 term of n_views images in one pass: the sum over the views of what odgs_loss_l1_dssim
+ * gives with lambda = 0 (p->lambda and p->wrap_u are not read), and every view's gradient. images, targets,
+ * widths, heights, grads: host arrays of n_views entries (grads or its entries may be NULL). scratch:
+ * odgs_loss_scratch_size bytes of any size of image, 16-byte aligned. */
+odgs_status odgs_loss_l1(const float *const *images, const float *const *targets, const int *widths,
+                         const int *heights, int n_views, const odgs_loss_params *p, float *const *grads,
+                         float *loss, void *scratch, size_t scratch_bytes, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -27,7 +27,7 @@ EXPORTED = ("odgs_create", "odgs_destroy", "odgs_workspace_size", "odgs_pair_buf
             "odgs_render_fwd_static", "odgs_measure_peaks", "odgs_last_launch_count", "odgs_status_string",
             "odgs_densify_select", "odgs_densify_scratch_size", "odgs_densify_apply", "odgs_adam_step",
             "odgs_loss_scratch_size", "odgs_loss_l1_dssim", "odgs_set_wait_limit", "odgs_debug_lists",
-            "odgs_debug_screen_grads", "odgs_wait_pairs")
+            "odgs_debug_screen_grads", "odgs_wait_pairs", "odgs_loss_l1")
 
 
 class OdgsError(RuntimeError):
@@ -130,6 +130,8 @@ def load(path: str = LIB_PATH):
     L.odgs_adam_step.argtypes = [C.POINTER(AdamGroup), C.c_int, C.POINTER(AdamParams), vp]
     L.odgs_loss_scratch_size.argtypes = [C.c_int, C.c_int, C.POINTER(sz)]
     L.odgs_loss_l1_dssim.argtypes = [vp, vp, C.c_int, C.c_int, C.POINTER(LossParams), vp, vp, vp, sz, vp]
+    L.odgs_loss_l1.argtypes = [C.POINTER(vp), C.POINTER(vp), C.POINTER(C.c_int), C.POINTER(C.c_int), C.c_int,
+                               C.POINTER(LossParams), C.POINTER(vp), vp, vp, sz, vp]
     L.odgs_densify_apply.argtypes = [C.POINTER(Gaussians), C.c_int, C.c_int, vp, vp, C.POINTER(ParamsOut), C.c_int,
                                      vp, vp, sz, vp]
     L.odgs_set_wait_limit.argtypes = [vp, C.c_uint32]
@@ -144,7 +146,7 @@ def load(path: str = LIB_PATH):
                  "odgs_preprocess_bwd", "odgs_frame_stats", "odgs_get_status", "odgs_render_fwd_static",
                  "odgs_measure_peaks", "odgs_densify_select", "odgs_densify_scratch_size", "odgs_densify_apply",
                  "odgs_adam_step", "odgs_loss_scratch_size", "odgs_loss_l1_dssim", "odgs_set_wait_limit",
-                 "odgs_debug_lists", "odgs_debug_screen_grads", "odgs_wait_pairs"):
+                 "odgs_debug_lists", "odgs_debug_screen_grads", "odgs_wait_pairs", "odgs_loss_l1"):
         getattr(L, name).restype = C.c_int
     _lib = L
     return L

@@ -23,25 +23,36 @@ def _ptr(t):
 def l1_dssim(images, targets, lam: float = 0.2, area_weight: bool = True, wrap_u: bool = True, want_grad: bool = True):
     dev = images[0].device
     lib = L.load()
-    need = 16
-    for im in images:
-        n = C.c_size_t()
-        L.check(lib.odgs_loss_scratch_size(int(im.shape[2]), int(im.shape[1]), C.byref(n)), "odgs_loss_scratch_size")
-        need = max(need, int(n.value))
-    scratch = torch.empty(need, dtype=torch.uint8, device=dev)
-    loss = torch.empty(1, dtype=torch.float32, device=dev)  # the first view writes it, the others add
-    grads = []
-    stream = L.raw_stream(dev)
-    for k, (im, tg) in enumerate(zip(images, targets)):
+    for im, tg in zip(images, targets):
         for t in (im, tg):
             if t.dtype != torch.float32 or not t.is_contiguous() or t.dim() != 3 or t.shape[0] != 3 or t.device != dev:
                 raise ValueError("images and targets must be contiguous float32 [3, H, W] tensors on one device")
         if im.shape != tg.shape:
             raise ValueError("image and target shapes differ")
-        g = torch.empty_like(im) if want_grad else None
+    need = 16
+    for w, h in {(int(im.shape[2]), int(im.shape[1])) for im in images}:
+        n = C.c_size_t()
+        L.check(lib.odgs_loss_scratch_size(w, h, C.byref(n)), "odgs_loss_scratch_size")
+        need = max(need, int(n.value))
+    if lam == 0.0:
+        need = min(need, 1 << 16)  # no maps
+    scratch = torch.empty(need, dtype=torch.uint8, device=dev)
+    loss = torch.empty(1, dtype=torch.float32, device=dev)  # the first view writes it, the others add
+    pairs = list(zip(images, targets))
+    grads = [torch.empty_like(im) if want_grad else None for im, _ in pairs]
+    stream = L.raw_stream(dev)
+    if lam == 0.0 and pairs:  # L1 alone: all views in one pass
+        nv = len(pairs)
+        arr, dims = C.c_void_p * nv, C.c_int * nv
+        prm = L.LossParams(0.0, int(bool(area_weight)), int(bool(wrap_u)), 0)
+        L.check(lib.odgs_loss_l1(arr(*[im.data_ptr() for im, _ in pairs]), arr(*[tg.data_ptr() for _, tg in pairs]),
+                                 dims(*[im.shape[2] for im, _ in pairs]), dims(*[im.shape[1] for im, _ in pairs]), nv,
+                                 C.byref(prm), arr(*[g.data_ptr() for g in grads]) if want_grad else None, _ptr(loss),
+                                 _ptr(scratch), C.c_size_t(scratch.numel()), stream), "odgs_loss_l1")
+        return loss[0], grads
+    for k, (im, tg) in enumerate(pairs):
         prm = L.LossParams(float(lam), int(bool(area_weight)), int(bool(wrap_u)), int(k > 0))
-        L.check(lib.odgs_loss_l1_dssim(_ptr(im), _ptr(tg), int(im.shape[2]), int(im.shape[1]), C.byref(prm), _ptr(g),
-                                       _ptr(loss), _ptr(scratch), C.c_size_t(scratch.numel()), stream),
+        L.check(lib.odgs_loss_l1_dssim(_ptr(im), _ptr(tg), int(im.shape[2]), int(im.shape[1]), C.byref(prm),
+                                       _ptr(grads[k]), _ptr(loss), _ptr(scratch), C.c_size_t(scratch.numel()), stream),
                 "odgs_loss_l1_dssim")
-        grads.append(g)
     return loss[0], grads
