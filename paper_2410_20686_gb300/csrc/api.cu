@@ -18,7 +18,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
     size_t hdr, views, trig, rec_a, rec_b, rec_c, rect, rect2, dkey0, dkey1, dval0, dval1, block_sums, ranges, T_final,
-        n_last, acc, sort_hist, sort_ctr, sort_lb, big, cover, cut, kcount, dbucket, total;
+        n_last, acc, sort_hist, sort_ctr, sort_lb, big, srect, cover, cut, kcount, dbucket, total;
     bool truncate;  // the lists are truncated at saturated tiles (the tables below are present)
 };
 
@@ -66,6 +66,7 @@ Layout make_layout(size_t items, const Geometry& g, bool truncate) {
     L.sort_ctr = take(kCtrBytes + sizeof(uint32_t) * radix_lookback_words(items) * kDepthLbRegions);
     L.sort_lb = L.sort_ctr + kCtrBytes;
     L.big = take(sizeof(uint2) * items);
+    L.srect = take(sizeof(uint4) * items);
     const size_t tt = truncate ? (size_t)g.total_tiles : 0;
     L.cover = take(sizeof(uint32_t) * (size_t)kCutBuckets * (truncate ? tt + 1 : 0));
     L.cut = take(tt);
@@ -492,6 +493,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     b.sorted_idx = dv[rb];
     b.rect = reinterpret_cast<const uint4*>(w + c->L.rect);
     b.rect2 = reinterpret_cast<const uint4*>(w + c->L.rect2);
+    b.srect = reinterpret_cast<uint4*>(w + c->L.srect);
     b.rec_a = reinterpret_cast<const float4*>(w + c->L.rec_a);
     b.rec_b = reinterpret_cast<const float4*>(w + c->L.rec_b);
     b.tile_w = c->s.tile_w;

@@ -1,19 +1,18 @@
 // Tile binning of the depth-sorted items (sm_103a):
-//   k_count_blocks  per block of 512 depth-sorted items: number of (tile, item) pairs
+//   k_count_blocks  per block of 512 depth-sorted items: number of (tile, item) pairs; the items'
+//                   footprint words in depth order
 //   k_scan_blocks   exclusive scan of the block totals (one CTA) + capacity check
-//   k_emit          each item writes one (tile id, item) pair per tile its footprint meets, in
-//                   depth order, at its exclusive-scan offset, and counts the tile sort's digits;
-//                   items with more than 32 pairs are queued for k_emit_big; pairs beyond the
-//                   capacity are dropped (status bit kStCapacity set by k_scan_blocks)
+//   k_emit          the items' (tile id, item) pairs, one per tile a footprint meets, in depth order at
+//                   the exclusive-scan offsets, a warp's items together; counts the tile sort's digits;
+//                   items with more than 32 tiles or 6 row bands are queued for k_emit_big; pairs beyond
+//                   the capacity are dropped (status bit kStCapacity set by k_scan_blocks)
 //   k_emit_big      the queued items, one warp each
 //   k_tile_ranges   [start, end) of every tile's run in the tile-sorted pair list
 // An item's rect is (ty0 | bands << 16, number of tiles, spans of bands 0 and 1), rect2 the spans
 // of bands 2..5; the columns of further bands are recomputed from its records by band_columns
-// (odgs_common.cuh), exactly as the preprocess counted them. A big item's pairs over its stored
-// bands are one flat range that the warp writes 32 at a time; pole-stretched Gaussians can cover
-// hundreds of tiles. With truncated lists (saturation.cu) an item writes only the pairs of the
-// tiles that keep its depth bucket, compacted in its tile order; the scan uses the kept counts,
-// and items keep the thread or warp emission that their whole footprint would take.
+// (odgs_common.cuh), exactly as the preprocess counted them. With truncated lists (saturation.cu) an
+// item writes only the pairs of the tiles that keep its depth bucket, compacted in its tile order; the
+// scan uses the kept counts.
 #include "odgs_common.cuh"
 #include "odgs_internal.h"
 
@@ -22,8 +21,6 @@ namespace odgs {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 2;
 constexpr int kScanTile = kScanThreads * kScanItems;
-
-__device__ __forceinline__ uint32_t rect_tiles(uint4 r) { return r.y; }
 
 __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v, unsigned long long* s) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -74,6 +71,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
             idx = a.sorted_idx[k];
             // idx >= n_items only after a depth sort that gave up (status already set)
             if (idx < a.n_items) rc = a.rect[idx];
+            a.srect[k] = rc;
         }
         if (!a.G) {
             c += rc.y;
@@ -217,143 +215,81 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
     }
 }
 
-// Counts the tile-sort digits of the keys key0 .. key0 + cnt - 1 (a contiguous run) in the block's
-// shared histogram. Lanes [lane0, lane0 + nlanes) share the low digit (distinct bins, one atomic
-// per key); the first lane adds the higher digits one constant-digit segment at a time, so a row
-// of consecutive tiles costs one atomic per higher digit instead of one per key.
-// Higher digits (passes 1 and up) of the run of consecutive keys key0 .. key0 + cnt - 1.
-__device__ __forceinline__ void count_high(uint32_t key0, int cnt, uint32_t (*s_hist)[256], int passes) {
-    if (cnt <= 0) return;
-    const uint32_t end = key0 + (uint32_t)cnt;
-    for (int p = 1; p < passes; ++p) {
-        const int sh = 8 * p;
-        uint32_t k = key0;
-        while (k < end) {
-            const uint32_t seg_end = min(end, ((k >> sh) + 1u) << sh);
-            atomicAdd(&s_hist[p][(k >> sh) & 0xFFu], seg_end - k);
-            k = seg_end;
+// ------------------------------------------------------------------ emission
+//
+// A warp writes its pairs as one sequence: the tiles of its items' row bands (runs of columns), listed
+// in shared memory, are taken 32 at a time, a lane each, so that the writes are coalesced and every
+// lane has a tile whatever the items' sizes. Pairs of tiles that do not keep the item's depth bucket
+// are compacted away by a ballot; the kept ones follow one another in the items' order. The kernels wait
+// on memory: the footprint words come in depth order from the count, which gathers them anyway, and the
+// lists are 8 bytes a run, so that six CTAs fit on an SM. Measured (k_emit + k_emit_big, us) against a
+// thread per small item that gathered its word: 3M Gaussians, 8 views of 4096 x 2048, emitted twice
+// 2157 + 1397 -> 1126 + 1160; 500K, 16 views 240 + 26 -> 174 + 18; 1M, six views 105 + 19 -> 82 + 16; 1M, one
+// view 35 + 36 -> 26 + 40; 100K, one view 25 + 16 -> 13 + 14. The words' copy adds 2 to 27 us to the count.
+constexpr int kStoredBands = 6;   // row bands whose spans the preprocess stored
+constexpr uint32_t kSmallTiles = 32;  // items of more tiles or bands take a warp of their own (k_emit_big)
+constexpr int kRuns = 32 * kStoredBands;  // runs a warp lists
+
+// A run: x = global id of its tile row's first tile, y = first column | lane of its item << 11 | index of
+// its first tile in the warp's sequence << 16 (below 2^16: 32 rows of at most 2048 tiles).
+__device__ __forceinline__ uint2 make_run(uint32_t row, uint32_t col, int item, uint32_t first) {
+    return make_uint2(row, col | ((uint32_t)item << 11) | (first << 16));
+}
+// Its item: x = item, y = position of a kept pair less its rank among the warp's kept pairs, z = depth bucket
+// the tiles have to keep (as int; -1: all do), w = tiles per row of its view.
+
+// Writes the pairs of the warp's nr listed runs (tot tiles), `kept` pairs of its sequence having been
+// written before; returns their number after it. Counts the tile-sort digits. Pairs at or beyond the
+// capacity are neither written nor counted.
+__device__ __forceinline__ uint32_t emit_runs(const EmitArgs& a, const uint2* run, const uint4* items, int nr, int tot,
+                                              uint32_t kept, int lane, uint32_t (*s_hist)[256]) {
+    const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
+    int rs = 0;  // run that holds the window's first tile
+    for (int g0 = 0; g0 < tot; g0 += 32) {
+        // the runs starting inside the window, as a bit mask: a lane's run is rs plus the starts at or
+        // before it
+        const int nx = rs + 1 + lane;
+        const int p = nx < nr ? (int)(run[nx].y >> 16) : 0x7fffffff;  // p > g0
+        const unsigned starts = __reduce_or_sync(full, p < g0 + 32 ? (1u << (p - g0)) : 0u);
+        const int r = rs + __popc(starts & ((2u << lane) - 1u));
+        rs += __popc(__ballot_sync(full, p <= g0 + 32));
+        const int g = g0 + lane;
+        bool write = g < tot;
+        uint32_t key = 0u;
+        uint4 it = make_uint4(0u, 0u, 0u, 0u);
+        if (write) {
+            const uint2 R = run[r];
+            it = items[(R.y >> 11) & 31u];
+            uint32_t tx = (R.y & 2047u) + ((uint32_t)g - (R.y >> 16));
+            if (tx >= it.w) tx -= it.w;
+            key = R.x + tx;
+            write = (int)it.z < 0 || (int)__ldg(a.cut + key) >= (int)it.z;
+        }
+        const unsigned km = __ballot_sync(full, write);
+        const uint32_t o = it.y + kept + (uint32_t)__popc(km & lt);
+        kept += (uint32_t)__popc(km);
+        if (write && o < (uint32_t)a.capacity) {
+            a.keys[o] = key;
+            a.vals[o] = it.x;
+            for (int q = 0; q < a.key_passes; ++q) atomicAdd(&s_hist[q][(key >> (8 * q)) & 0xFFu], 1u);
         }
     }
+    return kept;
 }
 
-__device__ __forceinline__ void count_run(uint32_t key0, int cnt, uint32_t (*s_hist)[256], int passes, int lane0,
-                                          int nlanes) {
-    if (cnt <= 0) return;
-    for (int k = lane0; k < cnt; k += nlanes) atomicAdd(&s_hist[0][(key0 + (uint32_t)k) & 0xFFu], 1u);
-    if (lane0 != 0) return;
-    const uint32_t end = key0 + (uint32_t)cnt;
-    for (int p = 1; p < passes; ++p) {
-        const int sh = 8 * p;
-        uint32_t k = key0;
-        while (k < end) {
-            const uint32_t seg_end = min(end, ((k >> sh) + 1u) << sh);
-            atomicAdd(&s_hist[p][(k >> sh) & 0xFFu], seg_end - k);
-            k = seg_end;
-        }
-    }
-}
-
-// Writes the pairs of one row band: columns start .. start + cnt - 1 (mod tiles_x), lanes
-// [lane0, lane0 + nlanes) sharing the work, and counts their tile-sort digits. Pairs at or
-// beyond the capacity are neither written nor counted.
-__device__ __forceinline__ void write_band(uint32_t row, int start, int cnt, int tiles_x, uint32_t idx,
-                                           unsigned long long off, unsigned long long capacity, int lane0,
-                                           int nlanes, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                           uint32_t (*s_hist)[256], int passes) {
-    if (off >= capacity) return;
-    if ((unsigned long long)cnt > capacity - off) cnt = (int)(capacity - off);
-    for (int k = lane0; k < cnt; k += nlanes) {
-        const unsigned long long o = off + (unsigned long long)k;
-        int tx = start + k;
-        if (tx >= tiles_x) tx -= tiles_x;
-        keys[o] = row + (uint32_t)tx;
-        vals[o] = idx;
-    }
-    // digit counts of the (at most two, seam-wrapped) runs of consecutive keys
-    const int first = min(cnt, tiles_x - start);
-    count_run(row + (uint32_t)start, first, s_hist, passes, lane0, nlanes);
-    count_run(row, cnt - first, s_hist, passes, lane0, nlanes);
-}
-
-// Spans of the item's first kStoredBands row bands, as the preprocess stored them.
-constexpr int kStoredBands = 6;
-__device__ __forceinline__ void stored_spans(uint32_t idx, uint4 rc, const EmitArgs& a, uint32_t spans[kStoredBands]) {
-    spans[0] = rc.z;
-    spans[1] = rc.w;
-    if ((rc.x >> 16) > 2u) {
-        const uint4 r2 = a.rect2[idx];
-        spans[2] = r2.x; spans[3] = r2.y; spans[4] = r2.z; spans[5] = r2.w;
-    } else {
-        spans[2] = spans[3] = spans[4] = spans[5] = 0u;
-    }
-}
-
-// Writes the pairs of one row band that keep bucket bk (cut[tile] >= bk), compacted from offset
-// off by one thread, and counts their digits; returns the offset after them.
-__device__ __forceinline__ unsigned long long write_band_kept(uint32_t row, int start, int cnt, int tiles_x,
-                                                              uint32_t idx, int bk, unsigned long long off,
-                                                              const EmitArgs& a, uint32_t (*s_hist)[256]) {
-    for (int k = 0; k < cnt; ++k) {
-        int tx = start + k;
-        if (tx >= tiles_x) tx -= tiles_x;
-        const uint32_t key = row + (uint32_t)tx;
-        if ((int)__ldg(a.cut + key) < bk) continue;
-        if (off < a.capacity) {
-            a.keys[off] = key;
-            a.vals[off] = idx;
-            for (int p = 0; p < a.key_passes; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 0xFFu], 1u);
-        }
-        ++off;
-    }
-    return off;
-}
-
-// Emits all pairs of one item from offset off, by one thread. The spans of the item's first
-// kStoredBands row bands were stored by the preprocess; further bands are recomputed (same
-// functions). bk >= 0: only the pairs of tiles that keep depth bucket bk.
-__device__ __forceinline__ void emit_item_thread(uint32_t idx, uint4 rc, unsigned long long off, const EmitArgs& a,
-                                                 uint32_t (*s_hist)[256], int bk) {
-    const ViewDev& V = a.views[idx / (uint32_t)a.n_per_view];
-    const int ty0 = (int)(rc.x & 0xFFFFu), nb = (int)(rc.x >> 16);
-    const int th = a.tile_h;
-    uint32_t spans[kStoredBands];
-    stored_spans(idx, rc, a, spans);
+__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
 #pragma unroll
-    for (int b = 0; b < kStoredBands; ++b) {  // constant indices: the spans stay in registers
-        if (b >= nb) break;
-        const uint32_t row = (uint32_t)V.tile_base + (uint32_t)(ty0 + b) * (uint32_t)V.tiles_x;
-        const int cnt = (int)(spans[b] >> 16);
-        if (bk >= 0) {
-            off = write_band_kept(row, (int)(spans[b] & 0xFFFFu), cnt, V.tiles_x, idx, bk, off, a, s_hist);
-            continue;
-        }
-        write_band(row, (int)(spans[b] & 0xFFFFu), cnt, V.tiles_x, idx, off, a.capacity, 0, 1, a.keys, a.vals,
-                   s_hist, a.key_passes);
-        off += (unsigned long long)cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
     }
-    if (nb <= kStoredBands) return;
-    Footprint fp = make_footprint(a.rec_a[idx], a.rec_b[idx]);
-    int jlo, jhi;
-    footprint_rows(fp, V.H, jlo, jhi);
-    for (int ty = ty0 + kStoredBands; ty < ty0 + nb; ++ty) {
-        int start, cnt;
-        band_columns(fp, max(jlo, ty * th), min(jhi, ty * th + th - 1), V.W, a.tile_w, V.tiles_x, V.model == 0, start,
-                         cnt);
-        const uint32_t row = (uint32_t)V.tile_base + (uint32_t)ty * (uint32_t)V.tiles_x;
-        if (bk >= 0) {
-            off = write_band_kept(row, start, cnt, V.tiles_x, idx, bk, off, a, s_hist);
-            continue;
-        }
-        write_band(row, start, cnt, V.tiles_x, idx, off, a.capacity, 0, 1, a.keys, a.vals, s_hist, a.key_passes);
-        off += (unsigned long long)cnt;
-    }
+    return v;
 }
 
-// The kept pairs of one item (tiles that keep depth bucket bk), by a whole warp: lanes compute the
-// spans of 32 row bands at a time, then the warp takes band after band 32 columns per step and
-// writes the kept ones compacted (ballot order = column order).
-__device__ __forceinline__ void emit_item_warp_kept(uint32_t idx, uint4 rc, unsigned long long off, int bk,
-                                                    const EmitArgs& a, int lane, uint32_t (*s_hist)[256]) {
+// The pairs of one item from position off, by a whole warp: lanes list the spans of 32 row bands at a
+// time (the stored ones, further ones recomputed as the preprocess counted them).
+__device__ __forceinline__ void emit_item_warp(uint32_t idx, uint4 rc, uint32_t off, int bucket, const EmitArgs& a, int lane,
+                                               uint2* run, uint4* items, uint32_t (*s_hist)[256]) {
     const unsigned full = 0xffffffffu;
     const ViewDev& V = a.views[idx / (uint32_t)a.n_per_view];
     const int th = a.tile_h, ty0 = (int)(rc.x & 0xFFFFu), nb = (int)(rc.x >> 16);
@@ -364,7 +300,8 @@ __device__ __forceinline__ void emit_item_warp_kept(uint32_t idx, uint4 rc, unsi
         fp = make_footprint(a.rec_a[idx], a.rec_b[idx]);
         footprint_rows(fp, V.H, jlo, jhi);
     }
-    const unsigned lt = (1u << lane) - 1u;
+    if (lane == 0) items[0] = make_uint4(idx, off, (uint32_t)bucket, (uint32_t)V.tiles_x);
+    uint32_t kept = 0u;
     for (int gb = 0; gb < nb; gb += 32) {
         const int b = gb + lane;
         int start = 0, cnt = 0;
@@ -379,121 +316,14 @@ __device__ __forceinline__ void emit_item_warp_kept(uint32_t idx, uint4 rc, unsi
                              start, cnt);
             }
         }
-        unsigned nz = __ballot_sync(full, cnt > 0);
-        while (nz) {
-            const int l = __ffs(nz) - 1;
-            nz &= nz - 1u;
-            const int c = __shfl_sync(full, cnt, l), s0 = __shfl_sync(full, start, l);
-            const uint32_t row = (uint32_t)V.tile_base + (uint32_t)(ty0 + gb + l) * (uint32_t)V.tiles_x;
-            for (int k0 = 0; k0 < c; k0 += 32) {
-                const int k = k0 + lane;
-                uint32_t key = 0u;
-                bool kept = false;
-                if (k < c) {
-                    int tx = s0 + k;
-                    if (tx >= V.tiles_x) tx -= V.tiles_x;
-                    key = row + (uint32_t)tx;
-                    kept = (int)__ldg(a.cut + key) >= bk;
-                }
-                const unsigned km = __ballot_sync(full, kept);
-                if (kept) {
-                    const unsigned long long o = off + (unsigned long long)__popc(km & lt);
-                    if (o < a.capacity) {
-                        a.keys[o] = key;
-                        a.vals[o] = idx;
-                        for (int p = 0; p < a.key_passes; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 0xFFu], 1u);
-                    }
-                }
-                off += (unsigned long long)__popc(km);
-            }
-        }
-    }
-}
-
-// Emits all pairs of one item from offset off, by a whole warp: lanes compute the spans of 32
-// row bands at a time, then the warp writes band after band, 32 columns per step.
-__device__ __forceinline__ void emit_item_warp(uint32_t idx, unsigned long long off, const EmitArgs& a, int lane,
-                                               uint32_t (*s_hist)[256]) {
-    const ViewDev& V = a.views[idx / (uint32_t)a.n_per_view];
-    const uint4 rc = a.rect[idx];
-    const int th = a.tile_h;
-    if ((rc.x >> 16) <= (uint32_t)kStoredBands) {  // spans stored by the preprocess
-        const int ty0 = (int)(rc.x & 0xFFFFu), nb = (int)(rc.x >> 16);
-        uint32_t spans[kStoredBands];
-        stored_spans(idx, rc, a, spans);
-        // the item's pairs as one range: pair t lies in the band b with cum[b] <= t < cum[b + 1]
-        int cum[kStoredBands + 1];
-        cum[0] = 0;
-#pragma unroll
-        for (int b = 0; b < kStoredBands; ++b) cum[b + 1] = cum[b] + (b < nb ? (int)(spans[b] >> 16) : 0);
-        if (off >= a.capacity) return;  // pairs beyond the capacity are neither written nor counted
-        const int avail = (int)min((unsigned long long)cum[kStoredBands], a.capacity - off);
-        const int tiles_x = V.tiles_x;
-        for (int t = lane; t < avail; t += 32) {
-            int b = 0;
-#pragma unroll
-            for (int q = 1; q < kStoredBands; ++q) b += t >= cum[q] ? 1 : 0;
-            uint32_t sp = spans[0];
-            int c0 = 0;
-#pragma unroll
-            for (int q = 1; q < kStoredBands; ++q) {  // selects: the arrays stay in registers
-                sp = b == q ? spans[q] : sp;
-                c0 = b == q ? cum[q] : c0;
-            }
-            int col = (int)(sp & 0xFFFFu) + (t - c0);
-            if (col >= tiles_x) col -= tiles_x;
-            const uint32_t key = (uint32_t)V.tile_base + (uint32_t)(ty0 + b) * (uint32_t)tiles_x + (uint32_t)col;
-            a.keys[off + (unsigned long long)t] = key;
-            a.vals[off + (unsigned long long)t] = idx;
-            atomicAdd(&s_hist[0][key & 0xFFu], 1u);
-        }
-        if (a.key_passes > 1 && lane < nb) {  // higher digits: lane b counts the runs of band b
-            uint32_t sp = spans[0];
-            int c0 = 0;
-#pragma unroll
-            for (int q = 1; q < kStoredBands; ++q) {
-                sp = lane == q ? spans[q] : sp;
-                c0 = lane == q ? cum[q] : c0;
-            }
-            const int c = min(max(avail - c0, 0), (int)(sp >> 16));
-            const int start = (int)(sp & 0xFFFFu);
-            const uint32_t row = (uint32_t)V.tile_base + (uint32_t)(ty0 + lane) * (uint32_t)tiles_x;
-            const int first = min(c, tiles_x - start);
-            count_high(row + (uint32_t)start, first, s_hist, a.key_passes);
-            count_high(row, c - first, s_hist, a.key_passes);
-        }
-        return;
-    }
-    Footprint fp = make_footprint(a.rec_a[idx], a.rec_b[idx]);
-    int jlo, jhi;
-    footprint_rows(fp, V.H, jlo, jhi);
-    if (jlo > jhi) return;
-    const int ty0 = jlo / th, ty1 = jhi / th;
-    for (int gq = ty0; gq <= ty1; gq += 32) {
-        const int ty = gq + lane;
-        int start = 0, cnt = 0;
-        if (ty <= ty1)
-            band_columns(fp, max(jlo, ty * th), min(jhi, ty * th + th - 1), V.W, a.tile_w, V.tiles_x, V.model == 0, start,
-                         cnt);
-        int incl = cnt;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const int excl = incl - cnt;
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        unsigned nz = __ballot_sync(0xffffffffu, cnt > 0);
-        while (nz) {
-            const int l = __ffs(nz) - 1;
-            nz &= nz - 1u;
-            const int c = __shfl_sync(0xffffffffu, cnt, l);
-            const int s0 = __shfl_sync(0xffffffffu, start, l);
-            const int e0 = __shfl_sync(0xffffffffu, excl, l);
-            const uint32_t row = (uint32_t)V.tile_base + (uint32_t)(gq + l) * (uint32_t)V.tiles_x;
-            write_band(row, s0, c, V.tiles_x, idx, off + (unsigned long long)e0, a.capacity, lane, 32, a.keys, a.vals,
-                       s_hist, a.key_passes);
-        }
-        off += (unsigned long long)total;
+        const uint32_t incl = warp_incl_scan((uint32_t)cnt, lane);
+        const unsigned nz = __ballot_sync(full, cnt > 0);
+        if (cnt > 0)
+            run[__popc(nz & ((1u << lane) - 1u))] = make_run((uint32_t)V.tile_base + (uint32_t)(ty0 + b) * (uint32_t)V.tiles_x,
+                                                             (uint32_t)start, 0, incl - (uint32_t)cnt);
+        __syncwarp();
+        kept = emit_runs(a, run, items, __popc(nz), (int)__shfl_sync(full, incl, 31), kept, lane, s_hist);
+        __syncwarp();  // the next bands overwrite the list
     }
 }
 
@@ -509,6 +339,9 @@ __global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
     __shared__ unsigned long long s_warp[kScanThreads / 32];
     __shared__ unsigned long long s_carry;
     __shared__ uint32_t s_hist[4][256];
+    __shared__ uint2 s_run[kScanThreads / 32][kRuns];
+    __shared__ uint4 s_item[kScanThreads / 32][32];
+    const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t base = blockIdx.x * kScanTile;
     for (int i = tid; i < 4 * 256; i += kScanThreads) s_hist[i >> 8][i & 255] = 0u;
@@ -522,17 +355,18 @@ __global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
     for (int round = 0; round < kScanItems; ++round) {
         const uint32_t k = base + (uint32_t)(round * kScanThreads + tid);
         const uint32_t idx = k < a.n_items ? a.sorted_idx[k] : 0u;
-        // an index past the end (only after a depth sort that gave up) emits nothing, as in
-        // k_count_blocks, so that the offsets of the two kernels agree
-        const uint4 rc = (k < a.n_items && idx < a.n_items) ? a.rect[idx] : make_uint4(0u, 0u, 0u, 0u);
-        // kept pairs (the scan) and the item's whole footprint (thread or warp emission)
+        // as k_count_blocks read it (no tiles for an index past the end, after a depth sort that gave up)
+        const uint4 rc = k < a.n_items ? a.srect[k] : make_uint4(0u, 0u, 0u, 0u);
+        // kept pairs (the scan) and the item's whole footprint (warp or shared emission)
         const uint32_t kw = (a.kcount && k < a.n_items) ? a.kcount[k] : rc.y;
         const uint32_t cnt = a.kcount ? (kw & 0x3FFFFFFu) : rc.y;
         const int bk = (a.kcount && cnt < rc.y) ? (int)(kw >> 26) : -1;
+        const int nb = (int)(rc.x >> 16);
+        const bool one = cnt > 0u && rc.y <= kSmallTiles && nb <= kStoredBands;
         // block-wide exclusive scan of the counts of this round (items in depth order)
         unsigned long long x = cnt;
         for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            unsigned long long y = __shfl_up_sync(full, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) s_warp[w] = x;
@@ -545,18 +379,48 @@ __global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
         }
         __syncthreads();
         if (tid == 0) s_carry += tot;
-        // small items: one lane each
-        if (cnt > 0u && rc.y <= 32u) emit_item_thread(idx, rc, off, a, s_hist, bk);
+        // positions past the capacity (below 2^30) are never written: clamped to 32 bits
+        const uint32_t off32 = (uint32_t)min(off, 1ull << 31);
+        // small items: the warp's, as one sequence
+        uint4 r2 = make_uint4(0u, 0u, 0u, 0u);
+        if (one && nb > 2) r2 = a.rect2[idx];
+        const uint32_t sp[kStoredBands] = {rc.z, rc.w, r2.x, r2.y, r2.z, r2.w};
+        uint32_t nz = 0u;
+        if (one) {
+#pragma unroll
+            for (int b = 0; b < kStoredBands; ++b) nz += (b < nb && (sp[b] >> 16) != 0u) ? 1u : 0u;
+        }
+        const uint32_t packed = one ? (nz << 16) | rc.y : 0u;  // runs (at most 192) and tiles (1024)
+        const uint32_t incl = warp_incl_scan(packed, lane);
+        const uint32_t last = __shfl_sync(full, incl, 31);
+        const uint32_t kincl = warp_incl_scan(one ? cnt : 0u, lane);
+        if (one) {
+            const ViewDev& V = a.views[idx / (uint32_t)a.n_per_view];
+            const uint32_t tiles_x = (uint32_t)V.tiles_x;
+            const uint32_t row = (uint32_t)V.tile_base + (rc.x & 0xFFFFu) * tiles_x;
+            uint32_t r = (incl - packed) >> 16, first = (incl - packed) & 0xFFFFu;
+            s_item[w][lane] = make_uint4(idx, off32 - (kincl - cnt), (uint32_t)bk, tiles_x);
+#pragma unroll
+            for (int b = 0; b < kStoredBands; ++b) {
+                if (b < nb && (sp[b] >> 16) != 0u) {
+                    s_run[w][r++] = make_run(row + (uint32_t)b * tiles_x, sp[b] & 0xFFFFu, lane, first);
+                    first += sp[b] >> 16;
+                }
+            }
+        }
+        __syncwarp();
+        emit_runs(a, s_run[w], s_item[w], (int)(last >> 16), (int)(last & 0xFFFFu), 0u, lane, s_hist);
+        __syncwarp();  // the next round overwrites the lists
         // large items: queued for k_emit_big (whole warps, dynamically scheduled). Depth order
         // clusters the nearest, largest Gaussians into the first blocks, so serving them here
         // would leave a few warps writing most of the pairs.
-        const bool big = cnt > 0u && rc.y > 32u;
-        const unsigned bigm = __ballot_sync(0xffffffffu, big);
+        const bool big = cnt > 0u && !one;
+        const unsigned bigm = __ballot_sync(full, big);
         if (bigm) {  // one queue reservation per warp
             uint32_t base_slot = 0u;
             if (lane == __ffs(bigm) - 1) base_slot = atomicAdd(&a.hdr->n_big, (uint32_t)__popc(bigm));
-            base_slot = __shfl_sync(0xffffffffu, base_slot, __ffs(bigm) - 1);
-            if (big) a.big[base_slot + __popc(bigm & ((1u << lane) - 1u))] = make_uint2(k, (uint32_t)off);
+            base_slot = __shfl_sync(full, base_slot, __ffs(bigm) - 1);
+            if (big) a.big[base_slot + __popc(bigm & ((1u << lane) - 1u))] = make_uint2(k, off32);
         }
     }
     flush_digits(s_hist, a.key_hist, a.key_passes);
@@ -564,24 +428,25 @@ __global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
 
 __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
     __shared__ uint32_t s_hist[4][256];
+    __shared__ uint2 s_run[8][32];
+    __shared__ uint4 s_item[8][1];
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) s_hist[i >> 8][i & 255] = 0u;
     __syncthreads();
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t n_big = a.hdr->n_big;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     // static round-robin over the queue: no shared counter to contend on
     for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_big; i += nwarps) {
         const uint2 e = a.big[i];
         const uint32_t idx = a.sorted_idx[e.x];
+        const uint4 rc = a.srect[e.x];
+        int bucket = -1;
         if (a.kcount) {
-            const uint4 rc = a.rect[idx];
             const uint32_t kw = a.kcount[e.x];
-            if ((kw & 0x3FFFFFFu) < rc.y) {
-                emit_item_warp_kept(idx, rc, (unsigned long long)e.y, (int)(kw >> 26), a, lane, s_hist);
-                continue;
-            }
+            if ((kw & 0x3FFFFFFu) < rc.y) bucket = (int)(kw >> 26);
         }
-        emit_item_warp(idx, (unsigned long long)e.y, a, lane, s_hist);
+        emit_item_warp(idx, rc, e.y, bucket, a, lane, s_run[w], s_item[w], s_hist);
+        __syncwarp();
     }
     flush_digits(s_hist, a.key_hist, a.key_passes);
 }
@@ -646,7 +511,7 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
     if (nb == 0 && (e = cudaMemsetAsync(a.key_hist, 0, sizeof(uint32_t) * 4 * 256, st)) != cudaSuccess) return e;
     if (nb > 0) {
         EmitArgs ea{};
-        ea.sorted_idx = a.sorted_idx; ea.rect = a.rect; ea.rect2 = a.rect2; ea.rec_a = a.rec_a; ea.rec_b = a.rec_b; ea.views = a.views;
+        ea.sorted_idx = a.sorted_idx; ea.srect = a.srect; ea.rect2 = a.rect2; ea.rec_a = a.rec_a; ea.rec_b = a.rec_b; ea.views = a.views;
         ea.n_per_view = a.n_per_view; ea.n_items = a.n_items; ea.tile_w = a.tile_w; ea.tile_h = a.tile_h;
         ea.block_offsets = a.block_sums; ea.capacity = a.capacity; ea.keys = a.keys; ea.vals = a.vals;
         ea.big = a.big; ea.hdr = a.hdr;

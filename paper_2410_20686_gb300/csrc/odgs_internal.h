@@ -90,6 +90,7 @@ struct BinArgs {
     const uint32_t* sorted_idx;
     const uint4* rect;
     const uint4* rect2;
+    uint4* srect;  // rect in depth order (written by k_count_blocks, which gathers it)
     const float4 *rec_a, *rec_b;
     int tile_w, tile_h;
     const ViewDev* views;
@@ -122,7 +123,7 @@ struct BinArgs {
 
 struct EmitArgs {
     const uint32_t* sorted_idx;
-    const uint4* rect;
+    const uint4* srect;
     const uint4* rect2;
     const float4 *rec_a, *rec_b;
     const ViewDev* views;

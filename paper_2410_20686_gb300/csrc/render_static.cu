@@ -113,11 +113,12 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
     uint32_t* p_hist = reinterpret_cast<uint32_t*>(take(4 * 4 * 256));
     uint32_t* p_ctr = reinterpret_cast<uint32_t*>(take(4 * 4));
     uint2* big = reinterpret_cast<uint2*>(take(sizeof(uint2) * n));
+    uint4* srect = reinterpret_cast<uint4*>(take(sizeof(uint4) * n));
     if (o >= kStaticBytes) return ODGS_ERR_WORKSPACE;
     // the rest holds the pairs: two key and two value buffers plus the sort look-back words
     const size_t rem = kStaticBytes - o;
     auto pair_bytes = [](size_t c) { return 4 * up256(4 * c) + up256(4 * radix_lookback_words(c)); };
-    size_t cap = rem / 17;  // at least 16.25 bytes per pair
+    size_t cap = rem / 16;  // 16.5 bytes per pair
     while (cap > 0 && pair_bytes(cap) > rem) cap -= (cap < 4096 ? cap : 4096);
     uint32_t* pk[2] = {reinterpret_cast<uint32_t*>(take(4 * cap)), reinterpret_cast<uint32_t*>(take(4 * cap))};
     uint32_t* pv[2] = {reinterpret_cast<uint32_t*>(take(4 * cap)), reinterpret_cast<uint32_t*>(take(4 * cap))};
@@ -147,7 +148,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
                           &launches, kDefaultWaitLimit) != cudaSuccess)
         return ODGS_ERR_CUDA;
     BinArgs b{};
-    b.sorted_idx = dv[rb]; b.rect = rect; b.rect2 = rect2; b.views = vd; b.n_per_view = g->n > 0 ? g->n : 1;
+    b.sorted_idx = dv[rb]; b.rect = rect; b.rect2 = rect2; b.srect = srect; b.views = vd; b.n_per_view = g->n > 0 ? g->n : 1;
     b.rec_a = rec_a; b.rec_b = rec_b; b.tile_w = st.tile_w; b.tile_h = st.tile_h;
     b.n_items = (uint32_t)n; b.block_sums = block_sums; b.hdr = hdr; b.capacity = cap;
     b.keys = pk[0]; b.vals = pv[0];
