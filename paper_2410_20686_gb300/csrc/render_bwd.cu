@@ -26,7 +26,8 @@
 // exponents formed before the pixels' tests, against a row test of every entry by every warp and the
 // reduction of nine values: 1M Gaussians, one 2048 x 1024 view 696 -> 517 us; 500K Gaussians, 16 views
 // 4369 -> 3265 us; 3M Gaussians, 8 views of 4096 x 2048 11438 -> 8920 us. The walk alone: 585, 3660 and
-// 9920 us; with a mask per pixel slot instead of per warp 597, 3632 and 10865 us.
+// 9920 us; with a mask per pixel slot instead of per warp 597, 3632 and 10865 us. Without a flag set by
+// every blending slot: 508, 3210 and 8700 us.
 #include "odgs_common.cuh"
 #include "odgs_internal.h"
 
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
                     // dL/drgb; the conic, opacity and mean terms are linear in these and in dy times them,
                     // so the warp reduces them and the CTA pass after the batch forms the terms
                     float S0 = 0.f, S1 = 0.f, S2 = 0.f, V0 = 0.f, V1 = 0.f, V2 = 0.f;
-                    bool contrib = false;
+                    float wlast = 0.f;  // weight of the last pixel that blends the entry
                     const float4 P = s_e[j].pos;
                     const float4 K = s_e[j].con;
                     const float4 c = s_e[j].col;
@@ -253,13 +254,13 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
 #pragma unroll
                     for (int k = 0; k < PPT; ++k) {
                         if (e >= nl[k] || !(pk[k] >= kLog2AlphaMin)) continue;
-                        const float t = tk[k], p = pk[k];
-                        contrib = true;
-                        const float ar = alpha_exp2(p);
+                        const float t = tk[k];
+                        const float ar = alpha_exp2(pk[k]);
                         const float alpha = fminf(kAlphaMax, ar);
                         const float inv = rcp_approx(__fsub_rn(1.f, alpha));
                         const float Tj = T[k] * inv;
                         const float w = alpha * Tj;
+                        wlast = w;
                         const float cg = c.x * g0[k] + c.y * g1[k] + c.z * g2[k];
                         V0 = fmaf(w, g0[k], V0);
                         V1 = fmaf(w, g1[k], V1);
@@ -275,8 +276,7 @@ __global__ void __launch_bounds__(256) k_render_bwd(BwdArgs a) {
                             S2 = fmaf(dpt, t, S2);
                         }
                     }
-                    const unsigned lanes = __ballot_sync(0xffffffffu, contrib);
-                    if (lanes == 0u) continue;
+                    if (!__any_sync(0xffffffffu, wlast > 0.f)) continue;  // no pixel blended the entry
                     got |= bit;
                     float* red = s_red + ((size_t)j * nwarps + warp) * 9;
                     // sum dp, sum dp t, sum dp t^2, sum dp t dy, sum dp dy, sum dp dy^2, dL/drgb
