@@ -230,7 +230,7 @@ __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int stride
 template <int DEG>
 struct ShRows {
     static constexpr int K = (DEG + 1) * (DEG + 1);
-    static constexpr int kChunks = 3 * K / 4;      // 3 (degree 1) or 12 (degree 3)
+    static constexpr int kChunks = (3 * K + 3) / 4;  // 3 (degree 1) or 12 (degree 3)
     static constexpr int kPitch = kChunks | 1;
 };
 template <int DEG>
@@ -271,7 +271,11 @@ __device__ __forceinline__ void sh_row_colour(const float4* row, const float Y[1
 constexpr int kThreadBands = 4;
 static_assert(kThreadBands <= 6, "the per-thread loop stores the spans of six bands (rect, rect2)");
 
-__global__ void __launch_bounds__(256, 3) k_preprocess_geom(PreArgs a) {
+// Bound by instruction issue and the latency of its arithmetic: CTAs of 128 threads at 72 registers keep 28
+// warps on an SM where 256 threads at 80 kept 24 (1M Gaussians, one view 63.5 -> 57.8 us; 3M, eight views
+// in four groups 1387 -> 1280; 500K, 16 views 328 -> 318).
+constexpr int kGeomThreads = 128;
+__global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) {
     const int g0 = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     unsigned long long local_pairs = 0ull;
@@ -478,8 +482,8 @@ __global__ void __launch_bounds__(256, 3) k_preprocess_geom(PreArgs a) {
         local_pairs += __shfl_xor_sync(0xffffffffu, local_pairs, off);
         local_visible += __shfl_xor_sync(0xffffffffu, local_visible, off);
     }
-    __shared__ unsigned long long s_sum[8];
-    __shared__ uint32_t s_vis[8];
+    __shared__ unsigned long long s_sum[kGeomThreads / 32];
+    __shared__ uint32_t s_vis[kGeomThreads / 32];
     if ((threadIdx.x & 31) == 0) {
         s_sum[threadIdx.x >> 5] = local_pairs;
         s_vis[threadIdx.x >> 5] = local_visible;
@@ -1014,7 +1018,7 @@ static bool stages_rows(int deg, int sh_coeffs) { return (deg == 1 || deg == 3) 
 cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, cudaEvent_t projected) {
     if (a.n == 0) return projected ? cudaEventRecord(projected, st) : cudaSuccess;
     const int threads = 256, blocks = (a.n + threads - 1) / threads;
-    k_preprocess_geom<<<blocks, threads, 0, st>>>(a);
+    k_preprocess_geom<<<(a.n + kGeomThreads - 1) / kGeomThreads, kGeomThreads, 0, st>>>(a);
     if (projected) {
         const cudaError_t e = cudaEventRecord(projected, st);
         if (e != cudaSuccess) return e;
