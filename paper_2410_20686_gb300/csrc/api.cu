@@ -27,6 +27,15 @@ struct PairLayout {
 };
 
 
+// Frames with perspective views and enough items for the partition's three launches to pay: their views
+// cull the Gaussians outside their field, ERP views next to none.
+bool partitions(const ViewTable& tab, size_t items) {
+    if (items < (1u << 17)) return false;
+    for (int v = 0; v < tab.n_views; ++v)
+        if (tab.v[v].model == 1) return true;
+    return false;
+}
+
 // Truncated lists unless the caller asks for the whole lists or the frame has too many tiles.
 bool truncates(const odgs_settings& s, const Geometry& g) { return !s.full_lists && (uint32_t)g.total_tiles <= kCutMaxTiles; }
 
@@ -61,7 +70,7 @@ Layout make_layout(size_t items, const Geometry& g, bool truncate) {
     L.T_final = take(sizeof(float) * (size_t)g.total_pixels);
     L.n_last = take(sizeof(uint32_t) * (size_t)g.total_pixels);
     L.acc = take(3 * sizeof(float4) * items);
-    L.sort_hist = take(sizeof(uint32_t) * 4 * 256);
+    L.sort_hist = take(sizeof(uint32_t) * 2 * 4 * 256);  // of all items, of the visible ones
     // the tile counters kCtrBytes before the look-back regions: one memset clears both
     L.sort_ctr = take(kCtrBytes + sizeof(uint32_t) * radix_lookback_words(items) * kDepthLbRegions);
     L.sort_lb = L.sort_ctr + kCtrBytes;
@@ -219,6 +228,7 @@ struct odgs_ctx {
     // the pairs of the current preprocess, once odgs_query_pairs has read them back
     bool pairs_known = false;
     size_t pairs = 0;
+    bool partition = false;  // visible items first, and only they are depth-sorted (partitions())
     bool whole_lists = false;  // what the last binning that was no rebuild did
     // a second stream on which the binning computes the cuts while the depth sort runs (forked
     // from and joined back to the caller's stream by events)
@@ -360,6 +370,7 @@ odgs_status odgs_preprocess(odgs_ctx* c, const odgs_gaussians* g, const odgs_vie
     c->ws_bytes = ws_bytes;
     c->stage = 0;
     c->launches = 0;
+    c->partition = partitions(tab, geo.n_items);
     c->cut_ready = false;
     c->pairs_known = false;
     c->bwd_batch = std::min(st.batch, 64);
@@ -479,10 +490,29 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     uint32_t* dv[2] = {reinterpret_cast<uint32_t*>(w + c->L.dval0), reinterpret_cast<uint32_t*>(w + c->L.dval1)};
     int rb = c->depth_buf;
     if (!rebuild) {
-        if (launch_radix_sort(dk, dv, &hdr->n_items, c->geo.n_items, 32, reinterpret_cast<uint32_t*>(w + c->L.sort_hist),
+        // The partition leaves the keys by item as they are (another odgs_bin_sort of this frame starts from
+        // them too), so the passes alternate between the second buffer and the emission's queue.
+        uint32_t* sk[2] = {dk[0], dk[1]};
+        uint32_t* sv[2] = {dv[0], dv[1]};
+        const uint32_t* n_sort = &hdr->n_items;
+        uint32_t* hist = reinterpret_cast<uint32_t*>(w + c->L.sort_hist);
+        if (c->partition) {
+            if (launch_partition(dk[0], (uint32_t)c->geo.n_items, reinterpret_cast<unsigned long long*>(w + c->L.block_sums),
+                                 hdr, hist, hist + 4 * 256, dk[1], dv[1], st, &c->launches) != cudaSuccess)
+                return ODGS_ERR_CUDA;
+            sk[0] = dk[1];
+            sv[0] = dv[1];
+            sk[1] = reinterpret_cast<uint32_t*>(w + c->L.big);
+            sv[1] = sk[1] + c->geo.n_items;
+            n_sort = &hdr->n_visible_sort;
+            hist += 4 * 256;
+        }
+        if (launch_radix_sort(sk, sv, n_sort, c->geo.n_items, 32, hist,
                               reinterpret_cast<uint32_t*>(w + c->L.sort_ctr), reinterpret_cast<uint32_t*>(w + c->L.sort_lb),
-                              &hdr->status, c->num_sms, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions, /*cleared=*/true) != cudaSuccess)
+                              &hdr->status, c->num_sms, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions,
+                              /*cleared=*/true) != cudaSuccess)
             return ODGS_ERR_CUDA;
+        if (c->partition) rb = 1;  // four passes end where they began
         c->depth_buf = rb;
     }
     // 2. emit (tile, item) pairs in depth order
@@ -521,6 +551,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         b.kcount = reinterpret_cast<uint32_t*>(w + c->L.kcount);
     }
     b.emit_only = rebuild;
+    b.visible_first = c->partition;
     if (!rebuild && c->geo.n_items > 0) {  // the pair count clears the ranges
         b.ranges_zero = reinterpret_cast<uint2*>(w + c->L.ranges);
         b.n_ranges = (uint32_t)c->geo.total_tiles;

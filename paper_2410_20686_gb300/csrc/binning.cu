@@ -62,12 +62,18 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
     if (a.ranges_zero)
         for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < a.n_ranges; t += gridDim.x * blockDim.x)
             a.ranges_zero[t] = make_uint2(0u, 0u);
+    // culled items end the depth order
+    const uint32_t n_vis = a.visible_first ? (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible) : a.n_items;
+    if (base >= n_vis) {
+        if (threadIdx.x == 0) a.block_sums[blockIdx.x] = 0ull;
+        return;
+    }
     unsigned long long c = 0ull;
     for (int i = threadIdx.x; i < kScanTile; i += kScanThreads) {
         const uint32_t k = base + i;
         uint4 rc = make_uint4(0u, 0u, 0u, 0u);
         uint32_t idx = 0u;
-        if (k < a.n_items) {
+        if (k < n_vis) {
             idx = a.sorted_idx[k];
             // idx >= n_items only after a depth sort that gave up (status already set)
             if (idx < a.n_items) rc = a.rect[idx];
@@ -78,7 +84,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
             continue;
         }
         const int nb = (int)(rc.x >> 16), ty0 = (int)(rc.x & 0xFFFFu);
-        const int bk = k < a.n_items ? depth_bucket(a.sorted_keys[k], a.base) : 0;
+        const int bk = k < n_vis ? depth_bucket(a.sorted_keys[k], a.base) : 0;
         const uint32_t* G = a.G + (size_t)bk * (a.total_tiles + 1u);
         // every tile of the frame keeps this bucket (the items in front of the first cut, among
         // them the near, large ones with many bands): the whole footprint
@@ -104,7 +110,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
             if (many) a.big[slot + __popc(m & ((1u << lane) - 1u))] = make_uint2(k, 0u);
         }
         if (many) continue;  // k_count_big writes its word and adds its pairs to the block's sum
-        if (k < a.n_items) a.kcount[k] = kept | ((uint32_t)bk << 26);
+        if (k < n_vis) a.kcount[k] = kept | ((uint32_t)bk << 26);
         c += kept;
     }
     c = block_sum_u64(c, s);
@@ -154,11 +160,8 @@ __global__ void __launch_bounds__(256) k_count_big(BinArgs a) {
     }
 }
 
-__global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __restrict__ block_sums, int nblocks,
-                                                      Header* hdr, unsigned long long capacity,
-                                                      uint32_t* __restrict__ key_hist) {
-    // the tile sort's digit counts, which the emission adds up, start from 0
-    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) key_hist[i] = 0u;
+// Exclusive scan of nblocks totals in place by one CTA of 1024 threads; returns their sum to every thread.
+__device__ __forceinline__ unsigned long long scan_totals(unsigned long long* __restrict__ block_sums, int nblocks) {
     // eight consecutive totals per thread and step: a frame of 8M items has 15.6K of them, which took
     // 34 us with one per thread and 15 us so
     constexpr int kEach = 8;
@@ -204,8 +207,16 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
         if (threadIdx.x == 0) s_carry += s_warp[31];
         __syncthreads();
     }
+    return s_carry;
+}
+
+__global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __restrict__ block_sums, int nblocks,
+                                                      Header* hdr, unsigned long long capacity,
+                                                      uint32_t* __restrict__ key_hist) {
+    // the tile sort's digit counts, which the emission adds up, start from 0
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) key_hist[i] = 0u;
+    const unsigned long long total = scan_totals(block_sums, nblocks);
     if (threadIdx.x == 0) {
-        unsigned long long total = s_carry;
         unsigned long long used = total < capacity ? total : capacity;
         hdr->pairs_emitted = used;
         hdr->n_pairs_sort = (uint32_t)used;
@@ -351,14 +362,16 @@ __global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
     for (int r = 0; r < 2; ++r)
         for (size_t i = (size_t)blockIdx.x * kScanThreads + tid; i < a.clear_quads[r]; i += (size_t)gridDim.x * kScanThreads)
             a.clear[r][i] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t n_vis = a.visible_first ? (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible) : a.n_items;
+    if (base >= n_vis) return;
     __syncthreads();
     for (int round = 0; round < kScanItems; ++round) {
         const uint32_t k = base + (uint32_t)(round * kScanThreads + tid);
-        const uint32_t idx = k < a.n_items ? a.sorted_idx[k] : 0u;
+        const uint32_t idx = k < n_vis ? a.sorted_idx[k] : 0u;
         // as k_count_blocks read it (no tiles for an index past the end, after a depth sort that gave up)
-        const uint4 rc = k < a.n_items ? a.srect[k] : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 rc = k < n_vis ? a.srect[k] : make_uint4(0u, 0u, 0u, 0u);
         // kept pairs (the scan) and the item's whole footprint (warp or shared emission)
-        const uint32_t kw = (a.kcount && k < a.n_items) ? a.kcount[k] : rc.y;
+        const uint32_t kw = (a.kcount && k < n_vis) ? a.kcount[k] : rc.y;
         const uint32_t cnt = a.kcount ? (kw & 0x3FFFFFFu) : rc.y;
         const int bk = (a.kcount && cnt < rc.y) ? (int)(kw >> 26) : -1;
         const int nb = (int)(rc.x >> 16);
@@ -451,6 +464,96 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
     flush_digits(s_hist, a.key_hist, a.key_passes);
 }
 
+// ------------------------------------------------------------------ visible items first
+//
+// Perspective frames cull most (view, Gaussian) items (a cube map's face sees a sixth of the scene), and
+// every pass of the depth sort would carry them. The items are partitioned first, stably: the
+// visible ones, which alone are sorted, then the culled ones in item order, as the whole sort would leave
+// them. 1M Gaussians on six faces (1.1M of 6M items visible): depth sort 204 -> 63 us with 27 us of partition,
+// pair count 81 -> 33, emission 80 -> 27; the step 2080 -> 1848 us.
+constexpr int kPartThreads = 256, kPartItems = 8, kPartTile = kPartThreads * kPartItems;
+
+__global__ void __launch_bounds__(kPartThreads) k_visible_count(const uint32_t* __restrict__ keys, uint32_t n,
+                                                                unsigned long long* __restrict__ block_sums) {
+    __shared__ int s_count[kPartThreads / 32];
+    const uint32_t base = blockIdx.x * (uint32_t)kPartTile;
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < kPartItems; ++i) {
+        const uint32_t k = base + (uint32_t)(i * kPartThreads) + threadIdx.x;
+        c += __popc(__ballot_sync(0xffffffffu, k < n && keys[k] != 0xFFFFFFFFu));
+    }
+    if ((threadIdx.x & 31) == 0) s_count[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < kPartThreads / 32; ++w) t += s_count[w];
+        block_sums[blockIdx.x] = (unsigned long long)t;
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_visible_scan(unsigned long long* __restrict__ block_sums, int nblocks, uint32_t n,
+                                                       Header* hdr, const uint32_t* __restrict__ hist,
+                                                       uint32_t* __restrict__ ohist) {
+    const uint32_t total = (uint32_t)scan_totals(block_sums, nblocks);
+    if (threadIdx.x == 0) hdr->n_visible_sort = total;
+    // a culled item's key is all ones: it counted once in the last digit of every pass
+    ohist[threadIdx.x] = hist[threadIdx.x] - ((threadIdx.x & 255u) == 255u ? n - total : 0u);
+}
+
+__global__ void __launch_bounds__(kPartThreads) k_partition(const uint32_t* __restrict__ keys, uint32_t n,
+                                                            const unsigned long long* __restrict__ block_sums,
+                                                            const Header* __restrict__ hdr, uint32_t* __restrict__ okeys,
+                                                            uint32_t* __restrict__ ovals) {
+    __shared__ uint32_t s_count[kPartItems][kPartThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t base = blockIdx.x * (uint32_t)kPartTile;
+    uint32_t key[kPartItems];
+    unsigned m[kPartItems];
+#pragma unroll
+    for (int i = 0; i < kPartItems; ++i) {
+        const uint32_t k = base + (uint32_t)(i * kPartThreads) + threadIdx.x;
+        key[i] = k < n ? keys[k] : 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (int i = 0; i < kPartItems; ++i) {
+        m[i] = __ballot_sync(0xffffffffu, key[i] != 0xFFFFFFFFu);
+        if (lane == 0) s_count[i][w] = (uint32_t)__popc(m[i]);
+    }
+    __syncthreads();
+    uint32_t vis = (uint32_t)block_sums[blockIdx.x];  // visible items before the warp's items of round i
+    const uint32_t n_vis = hdr->n_visible_sort;
+#pragma unroll
+    for (int i = 0; i < kPartItems; ++i) {
+        uint32_t before = vis;
+#pragma unroll
+        for (int q = 0; q < kPartThreads / 32; ++q) {
+            const uint32_t c = s_count[i][q];
+            before += q < w ? c : 0u;
+            vis += c;
+        }
+        const uint32_t k = base + (uint32_t)(i * kPartThreads) + threadIdx.x;
+        const uint32_t rank = before + (uint32_t)__popc(m[i] & ((1u << lane) - 1u));
+        if (k < n) {
+            const uint32_t o = key[i] != 0xFFFFFFFFu ? rank : n_vis + (k - rank);
+            okeys[o] = key[i];
+            ovals[o] = k;
+        }
+    }
+}
+
+cudaError_t launch_partition(const uint32_t* keys, uint32_t n, unsigned long long* block_sums, Header* hdr,
+                             const uint32_t* hist, uint32_t* ohist, uint32_t* okeys, uint32_t* ovals, cudaStream_t st,
+                             int* launches) {
+    const int blocks = (int)((n + kPartTile - 1) / kPartTile);
+    if (blocks == 0) return cudaSuccess;
+    k_visible_count<<<blocks, kPartThreads, 0, st>>>(keys, n, block_sums);
+    k_visible_scan<<<1, 1024, 0, st>>>(block_sums, blocks, n, hdr, hist, ohist);
+    k_partition<<<blocks, kPartThreads, 0, st>>>(keys, n, block_sums, hdr, okeys, ovals);
+    *launches += 3;
+    return cudaGetLastError();
+}
+
 // [start, end) of every tile's run. A thread takes 4 consecutive keys (one 16-byte load when the
 // array is 16-byte aligned) plus the keys on either side.
 __global__ void __launch_bounds__(256) k_tile_ranges(const uint32_t* __restrict__ keys, const Header* __restrict__ hdr,
@@ -515,6 +618,7 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         ea.n_per_view = a.n_per_view; ea.n_items = a.n_items; ea.tile_w = a.tile_w; ea.tile_h = a.tile_h;
         ea.block_offsets = a.block_sums; ea.capacity = a.capacity; ea.keys = a.keys; ea.vals = a.vals;
         ea.big = a.big; ea.hdr = a.hdr;
+        ea.visible_first = a.visible_first;
         ea.key_hist = a.key_hist; ea.key_passes = a.key_passes;
         ea.kcount = a.G ? a.kcount : nullptr;
         for (int r = 0; r < 2; ++r) { ea.clear[r] = a.clear[r]; ea.clear_quads[r] = a.clear_quads[r]; }

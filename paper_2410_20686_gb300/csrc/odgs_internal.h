@@ -96,6 +96,7 @@ struct BinArgs {
     const ViewDev* views;
     int n_per_view;
     uint32_t n_items;
+    bool visible_first;  // the items past hdr->visible are culled: not read
     unsigned long long* block_sums;
     Header* hdr;
     unsigned long long capacity;
@@ -129,6 +130,7 @@ struct EmitArgs {
     const ViewDev* views;
     int n_per_view;
     uint32_t n_items;
+    bool visible_first;
     int tile_w, tile_h;
     const unsigned long long* block_offsets;
     unsigned long long capacity;
@@ -210,6 +212,13 @@ constexpr size_t kCtrBytes = 256;
 inline size_t sort_scratch_quads(size_t max_items, int lb_regions) {
     return (kCtrBytes + sizeof(uint32_t) * radix_lookback_words(max_items) * (size_t)lb_regions) / sizeof(uint4);
 }
+
+// Visible items (their keys, and their indices) to the front, culled ones behind, both in item order;
+// their number in hdr->n_visible_sort, and the digit counts hist of all keys without the culled ones' in
+// ohist. block_sums: scan_blocks_for(n) totals.
+cudaError_t launch_partition(const uint32_t* keys, uint32_t n, unsigned long long* block_sums, Header* hdr,
+                             const uint32_t* hist, uint32_t* ohist, uint32_t* okeys, uint32_t* ovals, cudaStream_t st,
+                             int* launches);
 
 int scan_blocks_for(uint32_t n_items);
 cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches);

@@ -964,38 +964,40 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) pq[i] += gq[i];
         a.g_opacity[g] += gop;
-        if (STAGED) return;
+        if constexpr (!STAGED) {
 #pragma unroll
-        for (int k = 0; k < K; ++k)
+            for (int k = 0; k < K; ++k)
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) psh[3 * k + ch] += ONE ? msh[ch] * ysh[k] : gsh[ONE ? 0 : k][ch];
+                for (int ch = 0; ch < 3; ++ch) psh[3 * k + ch] += ONE ? msh[ch] * ysh[k] : gsh[ONE ? 0 : k][ch];
+        }
     } else {
 #pragma unroll
         for (int i = 0; i < 3; ++i) { pm[i] = gm[i]; ps[i] = gs[i]; }
         reinterpret_cast<float4*>(pq)[0] = make_float4(gq[0], gq[1], gq[2], gq[3]);
         a.g_opacity[g] = gop;
-        if (STAGED) return;
-        if ((a.sh_coeffs * 3) % 4 == 0 && (K * 3) % 4 == 0) {
-            float4* p4 = reinterpret_cast<float4*>(psh);
+        if constexpr (!STAGED) {
+            if ((a.sh_coeffs * 3) % 4 == 0 && (K * 3) % 4 == 0) {
+                float4* p4 = reinterpret_cast<float4*>(psh);
 #pragma unroll
-            for (int i = 0; i < K * 3 / 4; ++i) {
-                const int e = 4 * i;
-                float q[4];
+                for (int i = 0; i < K * 3 / 4; ++i) {
+                    const int e = 4 * i;
+                    float q[4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int kk = (e + r) / 3, ch = (e + r) % 3;
-                    q[r] = ONE ? msh[ch] * ysh[kk] : gsh[ONE ? 0 : kk][ch];
+                    for (int r = 0; r < 4; ++r) {
+                        const int kk = (e + r) / 3, ch = (e + r) % 3;
+                        q[r] = ONE ? msh[ch] * ysh[kk] : gsh[ONE ? 0 : kk][ch];
+                    }
+                    p4[i] = make_float4(q[0], q[1], q[2], q[3]);
                 }
-                p4[i] = make_float4(q[0], q[1], q[2], q[3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch) psh[3 * k + ch] = ONE ? msh[ch] * ysh[k] : gsh[ONE ? 0 : k][ch];
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) psh[3 * k + ch] = ONE ? msh[ch] * ysh[k] : gsh[ONE ? 0 : k][ch];
+            for (int k = K; k < a.sh_coeffs; ++k)
+                for (int ch = 0; ch < 3; ++ch) psh[3 * k + ch] = 0.f;
         }
-        for (int k = K; k < a.sh_coeffs; ++k)
-            for (int ch = 0; ch < 3; ++ch) psh[3 * k + ch] = 0.f;
     }
 }
 
