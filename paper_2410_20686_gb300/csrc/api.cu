@@ -715,6 +715,7 @@ odgs_status odgs_preprocess_bwd(odgs_ctx* c, const odgs_grads* grads, void* stre
     b.views = reinterpret_cast<const ViewDev*>(w + c->L.views);
     b.dilation = c->s.cov_dilation;
     b.acc = reinterpret_cast<const float4*>(w + c->L.acc);
+    if (c->partition) b.keys = reinterpret_cast<const uint32_t*>(w + c->L.dkey0);
     b.g_means = grads->means; b.g_scales = grads->scales; b.g_quats = grads->quats;
     b.g_opacity = grads->opacity; b.g_sh = grads->sh;
     b.accumulate = c->s.grad_accumulate;

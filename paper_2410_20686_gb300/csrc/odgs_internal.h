@@ -78,6 +78,7 @@ struct PreBwdArgs {
     const ViewDev* views;
     float dilation;
     const float4* acc;
+    const uint32_t* keys;            // depth keys by item (all ones: culled) where most items are culled, or null
     float *g_means, *g_scales, *g_quats, *g_opacity, *g_sh;
     int accumulate;
     int raw;                         // gradients w.r.t. log-scales and opacity logits

@@ -566,7 +566,11 @@ __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
 // kernel of several views spills 228 bytes, and with three CTAs takes 312, 218 and 1639 us below). Measured
 // (us), unstaged and staged: 1M Gaussians, one view 111 -> 83 (75 at the copy bandwidth); 500K, 16 views
 // 357 -> 319; 1M, six views 240 -> 229; 3M, eight views in four groups 1580 -> 1452.
-template <int DEG, bool ONE, bool STAGED>
+// KEYED: frames that cull most of their items (those that partition them) read the depth keys first, and each
+// lane then goes through the views that do not cull its Gaussian: an accumulator is 12 times a key, and a warp
+// makes as many steps as its busiest lane has views. 1M Gaussians, six perspective views 229 -> 146 us; where
+// nearly every item is visible the masks only cost (500K, 16 ERP views 319 -> 335 us).
+template <int DEG, bool ONE, bool STAGED, bool KEYED>
 __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
     constexpr int K = (DEG + 1) * (DEG + 1);
     using R = ShRows<DEG>;
@@ -613,18 +617,33 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
         st_count = a.d_count[g];
     }
     const uint32_t st_count0 = st_count;
+    unsigned long long seen = 0ull;  // KEYED: bit v set where view v does not cull the Gaussian
+    if (KEYED)
+        for (int v = 0; v < a.n_views; ++v)
+            seen |= (unsigned long long)(__ldg(a.keys + (size_t)v * a.n + g) != 0xFFFFFFFFu) << v;
+    auto after = [&](int v) {  // the view to take after v
+        if (!KEYED) return v + 1;
+        const unsigned long long m = v < kMaxViews - 1 ? seen >> (v + 1) : 0ull;
+        return m ? v + __ffsll((long long)m) : a.n_views;
+    };
     // the next view's accumulators load while this view's are used: most items of a frame of many
     // views have none, and their views would be one load's latency each
-    float4 n0 = a.acc[3 * (size_t)g], n1 = a.acc[3 * (size_t)g + 1], n2 = a.acc[3 * (size_t)g + 2];
+    const int first = after(-1);
+    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0;
+    if (!KEYED || first < a.n_views) {
+        const float4* at = a.acc + 3 * ((size_t)first * a.n + g);
+        n0 = at[0]; n1 = at[1]; n2 = at[2];
+    }
     if (STAGED && ONE)
         sh_rows_fetch<DEG>(rows, a.sh, gt - lane,
                            __ballot_sync(0xffffffffu, act && (n1.z != 0.f || n1.w != 0.f || n2.x != 0.f)), lane);
-    for (int v = 0; v < a.n_views; ++v) {
+    for (int v = first, nx; v < a.n_views; v = nx) {
         const size_t item = (size_t)v * a.n + g;
         const float4 g0 = n0, g1 = n1, g2 = n2;
-        if (!ONE && v + 1 < a.n_views) {
-            const float4* nx = a.acc + 3 * (item + (size_t)a.n);
-            n0 = nx[0]; n1 = nx[1]; n2 = nx[2];
+        nx = after(v);
+        if (!ONE && nx < a.n_views) {
+            const float4* at = a.acc + 3 * ((size_t)nx * a.n + g);
+            n0 = at[0]; n1 = at[1]; n2 = at[2];
         }
         if (a.d_count && a.rect[item].y > 0u) {
             // visible in view v: ERP-mean gradient in [-1, 1] image units, and 1 - cos(theta)
@@ -855,13 +874,13 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
     if (!ONE && any) {
         float shc[STAGED ? 1 : 16][3];
         if (!STAGED) load_sh<DEG>(a.sh, a.sh_coeffs, g, reinterpret_cast<float(*)[3]>(shc));
-        n1 = a.acc[3 * (size_t)g + 1], n2 = a.acc[3 * (size_t)g + 2];
-        for (int v = 0; v < a.n_views; ++v) {
-            const size_t item = (size_t)v * a.n + g;
+        n1 = a.acc[3 * ((size_t)first * a.n + g) + 1], n2 = a.acc[3 * ((size_t)first * a.n + g) + 2];
+        for (int v = first, nx; v < a.n_views; v = nx) {
             const float4 g1 = n1, g2 = n2;
-            if (v + 1 < a.n_views) {
-                const float4* nx = a.acc + 3 * (item + (size_t)a.n);
-                n1 = nx[1]; n2 = nx[2];
+            nx = after(v);
+            if (nx < a.n_views) {
+                const float4* at = a.acc + 3 * ((size_t)nx * a.n + g);
+                n1 = at[1]; n2 = at[2];
             }
             if (g1.z == 0.f && g1.w == 0.f && g2.x == 0.f) continue;
             const ViewDev& V = a.views[v];
@@ -1040,9 +1059,11 @@ static void launch_bwd(const PreBwdArgs& a, cudaStream_t st) {
     const int threads = 128, blocks = (a.n + threads - 1) / threads;
     const size_t bytes = STAGED ? (size_t)threads * ShRows<DEG>::kPitch * sizeof(float4) : 0;
     if (a.n_views == 1)
-        k_preprocess_bwd<DEG, true, STAGED><<<blocks, threads, bytes, st>>>(a);
+        k_preprocess_bwd<DEG, true, STAGED, false><<<blocks, threads, bytes, st>>>(a);
+    else if (a.keys)
+        k_preprocess_bwd<DEG, false, STAGED, true><<<blocks, threads, bytes, st>>>(a);
     else
-        k_preprocess_bwd<DEG, false, STAGED><<<blocks, threads, bytes, st>>>(a);
+        k_preprocess_bwd<DEG, false, STAGED, false><<<blocks, threads, bytes, st>>>(a);
 }
 
 cudaError_t launch_preprocess_bwd(const PreBwdArgs& a, int sh_degree, cudaStream_t st) {
