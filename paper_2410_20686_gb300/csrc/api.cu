@@ -324,6 +324,7 @@ static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
     a.dval = reinterpret_cast<uint32_t*>(w + c->L.dval0);
     a.dhist = dhist;
     a.num_sms = c->num_sms;
+    a.culls = c->partition;
     if (c->L.truncate) {
         a.dbucket = w + c->L.dbucket;
         uint32_t rn;

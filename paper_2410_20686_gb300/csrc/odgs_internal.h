@@ -69,6 +69,7 @@ struct PreArgs {
     uint8_t* dbucket;  // per item its depth bucket (saturation.cu), or null
     uint32_t cut_base;  // depth_bucket's origin
     int num_sms;
+    bool culls;  // most items are culled (frames that partition them)
     Header* hdr;
 };
 

@@ -275,6 +275,33 @@ static_assert(kThreadBands <= 6, "the per-thread loop stores the spans of six ba
 // warps on an SM where 256 threads at 80 kept 24 (1M Gaussians, one view 63.5 -> 57.8 us; 3M, eight views
 // in four groups 1387 -> 1280; 500K, 16 views 328 -> 318).
 constexpr int kGeomThreads = 128;
+
+// Whether a pinhole view surely culls a centre (false where it may lie inside the limits). t = R mu + t and
+// the products below are off by at most a few units in the last place of the sums of their terms'
+// magnitudes; the margin is 40 times that, so a centre that the projection would keep never misses.
+__device__ __forceinline__ bool misses_pinhole(const ViewDev& V, float m0, float m1, float m2, float tz) {
+    float t[2], mag[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float p0 = V.R[3 * i] * m0, p1 = V.R[3 * i + 1] * m1, p2 = V.R[3 * i + 2] * m2;
+        if (i < 2) t[i] = p0 + p1 + p2 + V.t[i];
+        mag[i] = fabsf(p0) + fabsf(p1) + fabsf(p2) + fabsf(V.t[i]);
+    }
+    const float W = (float)V.W, H = (float)V.H;
+    const float mx = 1e-5f * (fabsf(V.fx) * mag[0] + (fabsf(V.cx) + 1.3f * W) * mag[2]);
+    const float my = 1e-5f * (fabsf(V.fy) * mag[1] + (fabsf(V.cy) + 1.3f * H) * mag[2]);
+    const float x = V.fx * t[0], y = V.fy * t[1];
+    return tz > 0.f && (x + (V.cx - 1.3f * W) * tz > mx || -x - (V.cx + 0.3f * W) * tz > mx ||
+                        y + (V.cy - 1.3f * H) * tz > my || -y - (V.cy + 0.3f * H) * tz > my);
+}
+
+// CULLS: frames that partition their items (perspective views, which cull most of them). A cheap test of all
+// views first, then each lane goes through the views that may see its Gaussian, so that a warp makes as many
+// steps as its busiest lane has such views and not one for each view that some lane needs. Culled items get
+// no records and no value for the sort: with no tiles they emit no pair, and the partition forms the order's
+// items itself. 1M Gaussians, six perspective views 216 -> 132 us (193 with the culled records written); ERP
+// views cull next to nothing, and their frames keep the plain loop.
+template <bool CULLS>
 __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) {
     const int g0 = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -313,13 +340,32 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
         const float Qalpha = (255.f * o > 1.f) ? 2.f * logf(255.f * o) : -1.f;  // Mahalanobis^2 at alpha = 1/255
         const float Qb = Qalpha * (1.f + 1e-4f) + 1e-4f;
 
-        for (int v = 0; v < a.n_views; ++v) {
+        unsigned long long todo = 0ull;  // CULLS: the views that may see the Gaussian
+        if (CULLS) {
+            for (int v = 0; v < a.n_views; ++v) {
+                const ViewDev& V = a.views[v];
+                const float r = depth_key(V, m0, m1, m2);
+                if (act && finite_in && (r > a.st.r_near) && (r < a.st.r_far) && (Qalpha > 0.f) &&
+                    !(V.model == 1 && misses_pinhole(V, m0, m1, m2, r))) {
+                    todo |= 1ull << v;
+                } else if (act) {
+                    const size_t item = (size_t)v * a.n + g;
+                    a.rect[item] = make_uint4(0u, 0u, 0u, 0u);
+                    a.dkey[item] = 0xFFFFFFFFu;
+                    if (a.dbucket) a.dbucket[item] = (uint8_t)depth_bucket(0xFFFFFFFFu, a.cut_base);
+                }
+            }
+        }
+        for (int step = 0; CULLS ? __any_sync(0xffffffffu, todo != 0ull) : step < a.n_views; ++step) {
+            const bool on = CULLS ? todo != 0ull : act;
+            const int v = !CULLS ? step : (on ? __ffsll((long long)todo) - 1 : 0);
+            if (CULLS) todo &= todo - 1ull;
             const ViewDev& V = a.views[v];
             const size_t item = (size_t)v * a.n + g;
             uint4 rect = make_uint4(0u, 0u, 0u, 0u);
             uint32_t key = 0xFFFFFFFFu;
             const float r = depth_key(V, m0, m1, m2);
-            bool ok = act && finite_in && (r > a.st.r_near) && (r < a.st.r_far) && (Qalpha > 0.f);
+            bool ok = on && finite_in && (r > a.st.r_near) && (r < a.st.r_far) && (Qalpha > 0.f);
             // camera-space mean in float-float: t = W mu + t_wc
             ff t[3];
 #pragma unroll
@@ -427,14 +473,15 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
                 f.ystar = __shfl_sync(0xffffffffu, fp.ystar, src);
                 const int wjlo = __shfl_sync(0xffffffffu, jlo, src), wjhi = __shfl_sync(0xffffffffu, jhi, src);
                 const int wty0 = __shfl_sync(0xffffffffu, ty0, src), wnb = __shfl_sync(0xffffffffu, nb, src);
+                const ViewDev& U = a.views[CULLS ? __shfl_sync(0xffffffffu, v, src) : v];
                 uint32_t tot = 0u, w0 = 0u, w1 = 0u, w2 = 0u, w3 = 0u, w4 = 0u, w5 = 0u;
                 for (int b0 = 0; b0 < wnb; b0 += 32) {
                     const int b = b0 + lane;
                     int st0 = 0, cnt = 0;
                     if (b < wnb) {
                         const int ty = wty0 + b;
-                        band_columns(f, max(wjlo, ty * th), min(wjhi, ty * th + th - 1), V.W, a.st.tile_w,
-                                     V.tiles_x, V.model == 0, st0, cnt);
+                        band_columns(f, max(wjlo, ty * th), min(wjhi, ty * th + th - 1), U.W, a.st.tile_w,
+                                     U.tiles_x, U.model == 0, st0, cnt);
                     }
                     uint32_t c = (uint32_t)cnt;
 #pragma unroll
@@ -461,8 +508,8 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
                 a.rec_a[item] = ra;
                 a.rec_b[item] = rb;
             }
-            if (act) {
-                if (key == 0xFFFFFFFFu) {
+            if (on) {
+                if (!CULLS && key == 0xFFFFFFFFu) {
                     // culled: finite records that never pass the alpha test (opacity 0), so that an
                     // index that reaches the blend only through a sort that gave up reads no stale
                     // memory (the colour kernel writes rec_c of the visible items only)
@@ -473,7 +520,7 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
                 a.rect[item] = rect;
                 a.dkey[item] = key;
                 if (a.dbucket) a.dbucket[item] = (uint8_t)depth_bucket(key, a.cut_base);
-                a.dval[item] = (uint32_t)item;
+                if (!CULLS) a.dval[item] = (uint32_t)item;
             }
         }
     }
@@ -507,8 +554,9 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
 // CTA per 256 Gaussians those atomics, all to the same addresses, cost as much as the coefficients'
 // fetch. Three CTAs per SM (80 registers); measured (us) with a CTA per 256 Gaussians and so: 1M
 // Gaussians, one view 57 -> 50 (35 at the copy bandwidth); 1M, six views 107 -> 74; 500K, 16 views
-// 103 -> 77; 3M, 2 views 167 -> 136. Coefficient rows staged through shared memory: 48, 73, 84, 132.
-template <int DEG>
+// 103 -> 77; 3M, 2 views 167 -> 136. CULLS: a lane goes through its own views, as in the projection (1M, six
+// views 76 -> 63). Coefficient rows staged through shared memory: 48, 73, 84, 132.
+template <int DEG, bool CULLS>
 __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
     constexpr int K = (DEG + 1) * (DEG + 1);
     // digit histograms of the depth keys for the depth sort (all items, culled ones included),
@@ -518,9 +566,11 @@ __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
     __syncthreads();
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.n; g += gridDim.x * blockDim.x) {
         bool seen = false;  // in some view
+        unsigned long long views = 0ull;
         for (int v = 0; v < a.n_views; ++v) {
             const uint32_t key = a.dkey[(size_t)v * a.n + g];
             seen |= key != 0xFFFFFFFFu;
+            if (CULLS) views |= (unsigned long long)(key != 0xFFFFFFFFu) << v;
 #pragma unroll
             for (int p = 0; p < 4; ++p) atomicAdd(&s_dh[p][(key >> (8 * p)) & 0xFFu], 1u);
         }
@@ -528,9 +578,11 @@ __global__ void __launch_bounds__(256) k_preprocess_color(PreArgs a) {
         const float m0 = __ldg(a.means + 3 * g), m1 = __ldg(a.means + 3 * g + 1), m2 = __ldg(a.means + 3 * g + 2);
         float shc[16][3];
         load_sh<DEG>(a.sh, a.sh_coeffs, g, shc);
-        for (int v = 0; v < a.n_views; ++v) {
+        for (int step = 0; CULLS ? views != 0ull : step < a.n_views; ++step) {
+            const int v = CULLS ? __ffsll((long long)views) - 1 : step;
+            if (CULLS) views &= views - 1ull;
             const size_t item = (size_t)v * a.n + g;
-            if (a.dkey[item] == 0xFFFFFFFFu) continue;  // culled in this view
+            if (!CULLS && a.dkey[item] == 0xFFFFFFFFu) continue;  // culled in this view
             const ViewDev& V = a.views[v];
             const float dx = m0 - V.cam[0], dy = m1 - V.cam[1], dz = m2 - V.cam[2];
             const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
@@ -1036,21 +1088,35 @@ cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Hea
 // of coefficients above the degree.
 static bool stages_rows(int deg, int sh_coeffs) { return (deg == 1 || deg == 3) && sh_coeffs == (deg + 1) * (deg + 1); }
 
+template <int DEG>
+static void launch_color(const PreArgs& a, int grid, cudaStream_t st) {
+    if (a.culls)
+        k_preprocess_color<DEG, true><<<grid, 256, 0, st>>>(a);
+    else
+        k_preprocess_color<DEG, false><<<grid, 256, 0, st>>>(a);
+}
+
 cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, cudaEvent_t projected) {
     if (a.n == 0) return projected ? cudaEventRecord(projected, st) : cudaSuccess;
     const int threads = 256, blocks = (a.n + threads - 1) / threads;
-    k_preprocess_geom<<<(a.n + kGeomThreads - 1) / kGeomThreads, kGeomThreads, 0, st>>>(a);
+    const int geom_blocks = (a.n + kGeomThreads - 1) / kGeomThreads;
+    if (a.culls)
+        k_preprocess_geom<true><<<geom_blocks, kGeomThreads, 0, st>>>(a);
+    else
+        k_preprocess_geom<false><<<geom_blocks, kGeomThreads, 0, st>>>(a);
     if (projected) {
         const cudaError_t e = cudaEventRecord(projected, st);
         if (e != cudaSuccess) return e;
     }
     const int grid = min(blocks, 3 * a.num_sms);
-    switch (sh_degree) {
-        case 0: k_preprocess_color<0><<<grid, threads, 0, st>>>(a); break;
-        case 1: k_preprocess_color<1><<<grid, threads, 0, st>>>(a); break;
-        case 2: k_preprocess_color<2><<<grid, threads, 0, st>>>(a); break;
-        default: k_preprocess_color<3><<<grid, threads, 0, st>>>(a); break;
-    }
+    if (sh_degree == 0)
+        launch_color<0>(a, grid, st);
+    else if (sh_degree == 1)
+        launch_color<1>(a, grid, st);
+    else if (sh_degree == 2)
+        launch_color<2>(a, grid, st);
+    else
+        launch_color<3>(a, grid, st);
     return cudaGetLastError();
 }
 
