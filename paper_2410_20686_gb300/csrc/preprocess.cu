@@ -297,10 +297,11 @@ __device__ __forceinline__ bool misses_pinhole(const ViewDev& V, float m0, float
 
 // CULLS: frames that partition their items (perspective views, which cull most of them). A cheap test of all
 // views first, then each lane goes through the views that may see its Gaussian, so that a warp makes as many
-// steps as its busiest lane has such views and not one for each view that some lane needs. Culled items get
-// no records and no value for the sort: with no tiles they emit no pair, and the partition forms the order's
-// items itself. 1M Gaussians, six perspective views 216 -> 132 us (193 with the culled records written); ERP
-// views cull next to nothing, and their frames keep the plain loop.
+// steps as its busiest lane has such views and not one for each view that some lane needs. A culled item gets
+// an opacity of 0, so that the blend passes it over whatever the rest of its record holds (an index of one
+// reaches the blend only through a sort that gave up), and no value for the sort: the partition forms the
+// order's items itself. 1M Gaussians, six perspective views 216 -> 138 us (193 with all of the culled records
+// written); ERP views cull next to nothing, and their frames keep the plain loop.
 template <bool CULLS>
 __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) {
     const int g0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -350,6 +351,7 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
                     todo |= 1ull << v;
                 } else if (act) {
                     const size_t item = (size_t)v * a.n + g;
+                    a.rec_a[item] = make_float4(0.f, 0.f, 0.f, 0.f);
                     a.rect[item] = make_uint4(0u, 0u, 0u, 0u);
                     a.dkey[item] = 0xFFFFFFFFu;
                     if (a.dbucket) a.dbucket[item] = (uint8_t)depth_bucket(0xFFFFFFFFu, a.cut_base);
@@ -509,11 +511,11 @@ __global__ void __launch_bounds__(kGeomThreads, 7) k_preprocess_geom(PreArgs a) 
                 a.rec_b[item] = rb;
             }
             if (on) {
+                if (key == 0xFFFFFFFFu) a.rec_a[item] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (!CULLS && key == 0xFFFFFFFFu) {
                     // culled: finite records that never pass the alpha test (opacity 0), so that an
                     // index that reaches the blend only through a sort that gave up reads no stale
                     // memory (the colour kernel writes rec_c of the visible items only)
-                    a.rec_a[item] = make_float4(0.f, 0.f, 0.f, 0.f);
                     a.rec_b[item] = make_float4(1.f, 0.f, 1.f, 0.f);
                     a.rec_c[item] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }

@@ -54,3 +54,29 @@ def test_frame_matches_single_views(kind, shift):
         s1 = one.stats()
         visible, pairs = visible + s1["visible"], pairs + s1["pairs"]
     assert (st["visible"], st["pairs"]) == (visible, pairs)
+
+
+def test_sort_that_gives_up_reads_no_stale_record():
+    """A frame whose sorts give up at once (a wait limit of 0), on a workspace of NaN bytes and a pair buffer
+    that lists items which this frame culls: flagged, with finite images and gradients, then exact again."""
+    import torch
+    from paper_2410_20686_gb300 import _lib as L
+    from paper_2410_20686_gb300.rasterizer import Rasterizer, RenderSettings
+    sc = S.random_scene(30_000, 96, 96, seed=5, sh_degree=1, radius=(0.3, 5.0), log_scale=(-3.5, 0.6))
+    p, rs, views = to_torch(sc), RenderSettings(sh_degree=1), S.cubemap_views(96, (0.1, 0.0, -0.2))
+    turned = [views[k] for k in (1, 0, 3, 2, 5, 4)]
+    r = Rasterizer()
+    r.reserve_pairs(4 << 20)
+    r.forward(*p, turned, rs)
+    torch.cuda.synchronize()
+    r.ws.fill_(255)
+    r.set_wait_limit(0)
+    imgs, _ = r.forward(*p, views, rs)
+    g = r.backward([torch.ones_like(i) for i in imgs])
+    torch.cuda.synchronize()
+    assert r.status() & L.DEV_TIMEOUT
+    assert all(torch.isfinite(i).all() for i in imgs) and all(torch.isfinite(t).all() for t in g.values())
+    r.set_wait_limit(1 << 22)
+    imgs, _ = r.forward(*p, views, rs)
+    ref, _ = Rasterizer().forward(*p, views, rs)
+    assert r.status() == 0 and all(torch.equal(a, b) for a, b in zip(imgs, ref))
