@@ -6,7 +6,7 @@
 //                   the exclusive-scan offsets, a warp's items together; counts the tile sort's digits;
 //                   items with more than 32 tiles or 6 row bands are queued for k_emit_big; pairs beyond
 //                   the capacity are dropped (status bit kStCapacity set by k_scan_blocks)
-//   k_emit_big      the queued items, one warp each
+//   k_emit_big      the queued items, one warp each, or several for those of many tiles
 //   k_tile_ranges   [start, end) of every tile's run in the tile-sorted pair list
 // An item's rect is (ty0 | bands << 16, number of tiles, spans of bands 0 and 1), rect2 the spans
 // of bands 2..5; the columns of further bands are recomputed from its records by band_columns
@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
         hdr->pairs_emitted = used;
         hdr->n_pairs_sort = (uint32_t)used;
         hdr->n_big = 0u;
+        hdr->n_huge = 0u;
         hdr->n_count_big = 0u;
         if (total > capacity) atomicOr(&hdr->status, kStCapacity);
     }
@@ -239,6 +240,12 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
 // view 35 + 36 -> 26 + 40; 100K, one view 25 + 16 -> 13 + 14. The words' copy adds 2 to 27 us to the count.
 constexpr int kStoredBands = 6;   // row bands whose spans the preprocess stored
 constexpr uint32_t kSmallTiles = 32;  // items of more tiles or bands take a warp of their own (k_emit_big)
+// Items of at least kHugeTiles tiles take kHugeParts warps, each a range of their row bands. With a warp per
+// item the SMs idled two thirds of k_emit_big's time for the last ones, pole-stretched Gaussians of thousands of
+// tiles: 1M Gaussians, one view 41 -> 16 us; 100K 14 -> 8; 3M, eight views emitted twice 1170 -> 865 (with the
+// line at 256 tiles 20, 6 and 930 us, at 1024 19, 10 and 885; in four or sixteen parts 17, 8, 874 and 18, 8, 903).
+constexpr uint32_t kHugeTiles = 512;
+constexpr uint32_t kHugeParts = 8;
 constexpr int kRuns = 32 * kStoredBands;  // runs a warp lists
 
 // A run: x = global id of its tile row's first tile, y = first column | lane of its item << 11 | index of
@@ -297,10 +304,11 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
     return v;
 }
 
-// The pairs of one item from position off, by a whole warp: lanes list the spans of 32 row bands at a
-// time (the stored ones, further ones recomputed as the preprocess counted them).
+// The pairs of one item whose first is at position off, by a whole warp: lanes list the spans of 32 row bands
+// at a time (the stored ones, further ones recomputed as the preprocess counted them). part of parts: a range
+// of its bands, whose pairs follow the kept pairs of the bands before, as the counts counted them.
 __device__ __forceinline__ void emit_item_warp(uint32_t idx, uint4 rc, uint32_t off, int bucket, const EmitArgs& a, int lane,
-                                               uint2* run, uint4* items, uint32_t (*s_hist)[256]) {
+                                               uint2* run, uint4* items, uint32_t (*s_hist)[256], int part, int parts) {
     const unsigned full = 0xffffffffu;
     const ViewDev& V = a.views[idx / (uint32_t)a.n_per_view];
     const int th = a.tile_h, ty0 = (int)(rc.x & 0xFFFFu), nb = (int)(rc.x >> 16);
@@ -311,22 +319,32 @@ __device__ __forceinline__ void emit_item_warp(uint32_t idx, uint4 rc, uint32_t 
         fp = make_footprint(a.rec_a[idx], a.rec_b[idx]);
         footprint_rows(fp, V.H, jlo, jhi);
     }
+    auto span = [&](int b, int& start, int& cnt) {
+        if (b < kStoredBands) {
+            const uint32_t sp = b == 0 ? rc.z : (b == 1 ? rc.w : (b == 2 ? r2.x : (b == 3 ? r2.y : (b == 4 ? r2.z : r2.w))));
+            start = (int)(sp & 0xFFFFu);
+            cnt = (int)(sp >> 16);
+        } else {
+            const int ty = ty0 + b;
+            band_columns(fp, max(jlo, ty * th), min(jhi, ty * th + th - 1), V.W, a.tile_w, V.tiles_x, V.model == 0, start, cnt);
+        }
+    };
     if (lane == 0) items[0] = make_uint4(idx, off, (uint32_t)bucket, (uint32_t)V.tiles_x);
+    const int first = nb * part / parts, end = nb * (part + 1) / parts;
     uint32_t kept = 0u;
-    for (int gb = 0; gb < nb; gb += 32) {
+    for (int b = lane; b < first; b += 32) {
+        int start = 0, cnt = 0;
+        span(b, start, cnt);
+        const uint32_t row = (uint32_t)V.tile_base + (uint32_t)(ty0 + b) * (uint32_t)V.tiles_x;
+        if (cnt > 0)
+            kept += bucket < 0 ? (uint32_t)cnt
+                               : kept_in_run(a.G + (size_t)bucket * (a.total_tiles + 1u), row, start, cnt, V.tiles_x);
+    }
+    if (first > 0) kept = __reduce_add_sync(full, kept);
+    for (int gb = first; gb < end; gb += 32) {
         const int b = gb + lane;
         int start = 0, cnt = 0;
-        if (b < nb) {
-            if (b < kStoredBands) {
-                const uint32_t sp = b == 0 ? rc.z : (b == 1 ? rc.w : (b == 2 ? r2.x : (b == 3 ? r2.y : (b == 4 ? r2.z : r2.w))));
-                start = (int)(sp & 0xFFFFu);
-                cnt = (int)(sp >> 16);
-            } else {
-                const int ty = ty0 + b;
-                band_columns(fp, max(jlo, ty * th), min(jhi, ty * th + th - 1), V.W, a.tile_w, V.tiles_x, V.model == 0,
-                             start, cnt);
-            }
-        }
+        if (b < end) span(b, start, cnt);
         const uint32_t incl = warp_incl_scan((uint32_t)cnt, lane);
         const unsigned nz = __ballot_sync(full, cnt > 0);
         if (cnt > 0)
@@ -346,7 +364,8 @@ __device__ __forceinline__ void flush_digits(uint32_t (*s_hist)[256], uint32_t* 
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
+// 32 registers: at the 40 that the two queues make of it, 3M Gaussians, eight views take 1145 us instead of 1073.
+__global__ void __launch_bounds__(kScanThreads, 8) k_emit(EmitArgs a) {
     __shared__ unsigned long long s_warp[kScanThreads / 32];
     __shared__ unsigned long long s_carry;
     __shared__ uint32_t s_hist[4][256];
@@ -427,13 +446,20 @@ __global__ void __launch_bounds__(kScanThreads) k_emit(EmitArgs a) {
         // large items: queued for k_emit_big (whole warps, dynamically scheduled). Depth order
         // clusters the nearest, largest Gaussians into the first blocks, so serving them here
         // would leave a few warps writing most of the pairs.
-        const bool big = cnt > 0u && !one;
-        const unsigned bigm = __ballot_sync(full, big);
-        if (bigm) {  // one queue reservation per warp
+        // The queue's end holds, backwards, those of them that take several warps.
+        const bool big = cnt > 0u && !one, huge = big && rc.y >= kHugeTiles;
+        const unsigned bigm = __ballot_sync(full, big && !huge), hugem = __ballot_sync(full, huge);
+        if (bigm | hugem) {  // one reservation per warp and queue
             uint32_t base_slot = 0u;
-            if (lane == __ffs(bigm) - 1) base_slot = atomicAdd(&a.hdr->n_big, (uint32_t)__popc(bigm));
-            base_slot = __shfl_sync(full, base_slot, __ffs(bigm) - 1);
-            if (big) a.big[base_slot + __popc(bigm & ((1u << lane) - 1u))] = make_uint2(k, off32);
+            if (bigm && lane == __ffs(bigm) - 1) base_slot = atomicAdd(&a.hdr->n_big, (uint32_t)__popc(bigm));
+            if (hugem && lane == __ffs(hugem) - 1) base_slot = atomicAdd(&a.hdr->n_huge, (uint32_t)__popc(hugem));
+            const uint32_t sb = __shfl_sync(full, base_slot, bigm ? __ffs(bigm) - 1 : 0);
+            const uint32_t sh = __shfl_sync(full, base_slot, hugem ? __ffs(hugem) - 1 : 0);
+            const unsigned lt = (1u << lane) - 1u;
+            if (huge)
+                a.big[a.n_items - 1u - sh - __popc(hugem & lt)] = make_uint2(k, off32);
+            else if (big)
+                a.big[sb + __popc(bigm & lt)] = make_uint2(k, off32);
         }
     }
     flush_digits(s_hist, a.key_hist, a.key_passes);
@@ -446,11 +472,12 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) s_hist[i >> 8][i & 255] = 0u;
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t n_big = a.hdr->n_big;
+    const uint32_t n_parts = a.hdr->n_huge * kHugeParts, n_all = n_parts + a.hdr->n_big;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    // static round-robin over the queue: no shared counter to contend on
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_big; i += nwarps) {
-        const uint2 e = a.big[i];
+    // static round-robin over the parts of the huge items, then the others: no shared counter to contend on
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_all; i += nwarps) {
+        const bool huge = i < n_parts;
+        const uint2 e = a.big[huge ? a.n_items - 1u - i / kHugeParts : i - n_parts];
         const uint32_t idx = a.sorted_idx[e.x];
         const uint4 rc = a.srect[e.x];
         int bucket = -1;
@@ -458,7 +485,8 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
             const uint32_t kw = a.kcount[e.x];
             if ((kw & 0x3FFFFFFu) < rc.y) bucket = (int)(kw >> 26);
         }
-        emit_item_warp(idx, rc, e.y, bucket, a, lane, s_run[w], s_item[w], s_hist);
+        emit_item_warp(idx, rc, e.y, bucket, a, lane, s_run[w], s_item[w], s_hist, huge ? (int)(i % kHugeParts) : 0,
+                       huge ? (int)kHugeParts : 1);
         __syncwarp();
     }
     flush_digits(s_hist, a.key_hist, a.key_passes);
@@ -594,7 +622,7 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
     cudaError_t e;
     const int nb = scan_blocks_for(a.n_items);
     if (a.emit_only) {
-        if ((e = cudaMemsetAsync(&a.hdr->n_big, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(&a.hdr->n_big, 0, 2 * sizeof(uint32_t), st)) != cudaSuccess) return e;
     } else if (nb > 0) {
         // the kept-count queue counter is 0: cleared by the preprocess's setup and by every scan
         k_count_blocks<<<nb, kScanThreads, 0, st>>>(a);
@@ -623,6 +651,8 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         ea.kcount = a.G ? a.kcount : nullptr;
         for (int r = 0; r < 2; ++r) { ea.clear[r] = a.clear[r]; ea.clear_quads[r] = a.clear_quads[r]; }
         ea.cut = a.cut;
+        ea.G = a.G;
+        ea.total_tiles = (uint32_t)a.total_tiles;
         // zeroed by the scan, except when the scan does not run
         if (a.emit_only && (e = cudaMemsetAsync(a.key_hist, 0, sizeof(uint32_t) * 4 * 256, st)) != cudaSuccess) return e;
         k_emit<<<nb, kScanThreads, 0, st>>>(ea);

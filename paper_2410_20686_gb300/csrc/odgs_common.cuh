@@ -86,9 +86,10 @@ struct Header {
     uint32_t n_items;                 // views * n
     uint32_t n_pairs_sort;            // 32-bit copy of pairs_emitted for the sort kernels
     uint32_t n_big;                   // items queued for the warp-wide emission
+    uint32_t n_huge;                  // items queued for several warps each (cleared together with n_big)
     uint32_t n_count_big;             // items queued for the warp-wide kept-pair count
     uint32_t n_visible_sort;          // visible items, of a depth order partitioned before its sort
-    uint32_t pad[2];
+    uint32_t pad;
 };
 
 struct Settings {

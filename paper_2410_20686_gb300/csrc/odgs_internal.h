@@ -143,6 +143,8 @@ struct EmitArgs {
     int key_passes;
     const uint32_t* kcount;  // by depth-order position, or null
     const uint8_t* cut;
+    const uint32_t* G;  // prefix counts of the tiles that keep a bucket, with kcount
+    uint32_t total_tiles;
     uint4* clear[2];
     size_t clear_quads[2];
 };
