@@ -211,8 +211,8 @@ def stage_rooflines(kern, stats, n, sh_degree, tiles, pair_passes, hbm_gbs, alu_
 # bench reports null until it is captured again.
 PROFILED_TRAFFIC = {"kernel": "k_render_bwd", "sources": ("render_bwd.cu", "odgs_common.cuh"),
                     "structs": ("odgs_internal.h", "BwdArgs"),
-                    "sha256": "79548bc8d827a32d6196073bbce0fad16e61150ec889680e230c810e30ee5cfe",
-                    "bytes": 171006208}
+                    "sha256": "ef5d6d0b5e3b148400fb487bcad6eb004c50b9aba346c8a9bb4e4d2b3aba10a4",
+                    "bytes": 169329152}
 
 
 def kernel_sources_digest(spec=PROFILED_TRAFFIC):

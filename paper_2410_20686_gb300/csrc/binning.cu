@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
 // every pass of the depth sort would carry them. The items are partitioned first, stably: the
 // visible ones, which alone are sorted, then the culled ones in item order, as the whole sort would leave
 // them. 1M Gaussians on six faces (1.1M of 6M items visible): depth sort 204 -> 63 us with 27 us of partition,
-// pair count 81 -> 33, emission 80 -> 27; the step 2080 -> 1848 us.
+// pair count 81 -> 33, emission 80 -> 27; the step 2080 -> 1837 us.
 constexpr int kPartThreads = 256, kPartItems = 8, kPartTile = kPartThreads * kPartItems;
 
 __global__ void __launch_bounds__(kPartThreads) k_visible_count(const uint32_t* __restrict__ keys, uint32_t n,

@@ -22,7 +22,7 @@ namespace odgs {
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItemsMax = 16;  // 4096 keys per CTA for sorts of at least kLargeSort keys, else 2048
-constexpr size_t kLargeSort = 1u << 20;  // 1M items by depth: 78 us with 2048-key tiles, 82 with 4096
+constexpr size_t kLargeSort = 1u << 20;  // 1M items by depth, one look-back word at a time: 78 us with 2048-key tiles, 82 with 4096
 constexpr int kRadix = 256;
 constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagPrefix = 2u << 30;
