@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kScanThreads, 8) k_emit(EmitArgs a) {
         __syncwarp();
         emit_runs(a, s_run[w], s_item[w], (int)(last >> 16), (int)(last & 0xFFFFu), 0u, lane, s_hist);
         __syncwarp();  // the next round overwrites the lists
-        // large items: queued for k_emit_big (whole warps, dynamically scheduled). Depth order
+        // large items: queued for k_emit_big (whole warps, round robin). Depth order
         // clusters the nearest, largest Gaussians into the first blocks, so serving them here
         // would leave a few warps writing most of the pairs.
         // The queue's end holds, backwards, those of them that take several warps.
