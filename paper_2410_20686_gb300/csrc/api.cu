@@ -220,16 +220,13 @@ struct odgs_ctx {
     int launches = 0;
     int bwd_batch = 64;
     uint32_t wait_limit = kDefaultWaitLimit;
-    int depth_buf = 0, pair_buf = 0;  // which buffer of each double-buffered sort holds its result
-    // the cut per tile and the kept counts per item of the current preprocess are in the
-    // workspace (they are computed from the depth keys by item, which the depth sort overwrites,
-    // so a second odgs_bin_sort or a rebuild of the lists reuses them)
+    int depth_buf = 0, pair_buf = 0;  // which buffer holds the depth-sorted keys, the tile-sorted pairs
+    // the cut per tile of the current preprocess is in the workspace: a second odgs_bin_sort reuses it
     bool cut_ready = false;
     // the pairs of the current preprocess, once odgs_query_pairs has read them back
     bool pairs_known = false;
     size_t pairs = 0;
     bool partition = false;  // visible items first, and only they are depth-sorted (partitions())
-    bool whole_lists = false;  // what the last binning that was no rebuild did
     // a second stream on which the binning computes the cuts while the depth sort runs (forked
     // from and joined back to the caller's stream by events)
     cudaStream_t side = nullptr;
@@ -302,7 +299,7 @@ static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
     float4* trig = reinterpret_cast<float4*>(w + c->L.trig);
     uint32_t* dhist = reinterpret_cast<uint32_t*>(w + c->L.sort_hist);
     if (launch_setup(c->tab, vd, trig, hdr, c->geo.total_trig, dhist, reinterpret_cast<uint4*>(w + c->L.sort_ctr),
-                     sort_scratch_quads(c->geo.n_items, kDepthLbRegions), st) != cudaSuccess)
+                     sort_scratch_quads(c->geo.n_items, kDepthLbRegions), c->partition, st) != cudaSuccess)
         return ODGS_ERR_CUDA;
     c->launches += 1;
     PreArgs a{};
@@ -458,10 +455,11 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     // saves nothing, and the cuts are five launches and four event calls of a frame that is bound by
     // its launches (1K Gaussians at 256 x 128, one view: 151 -> 134 us with this and the sorts'
     // scratch cleared by kernels instead of memsets).
+    // A rebuild emits what the count that ran last counted (Header::kept_pairs).
     constexpr size_t kFewPairs = 32768;
-    if (!rebuild) c->whole_lists = !c->L.truncate || (c->pairs_known && c->pairs <= std::min(c->pb_cap, kFewPairs));
-    const bool truncate = !c->whole_lists;
-    // 0. which tiles saturate, and from which depth on (before the depth sort reorders the keys)
+    const bool few = c->pairs_known && c->pairs <= std::min(c->pb_cap, kFewPairs);
+    const bool truncate = c->L.truncate && !few && !rebuild;
+    // 0. which tiles saturate, and from which depth on
     if (truncate && !c->cut_ready) {
         SatArgs sa{};
         sa.rect = reinterpret_cast<const uint4*>(w + c->L.rect);
@@ -489,22 +487,21 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     // 1. depth sort of all (view, Gaussian) items (digit histograms counted by the preprocess)
     uint32_t* dk[2] = {reinterpret_cast<uint32_t*>(w + c->L.dkey0), reinterpret_cast<uint32_t*>(w + c->L.dkey1)};
     uint32_t* dv[2] = {reinterpret_cast<uint32_t*>(w + c->L.dval0), reinterpret_cast<uint32_t*>(w + c->L.dval1)};
-    int rb = c->depth_buf;
     if (!rebuild) {
+        int rb = 0;
         // The partition leaves the keys by item as they are (another odgs_bin_sort of this frame starts from
-        // them too), so the passes alternate between the second buffer and the emission's queue.
+        // them too), so its keys alternate between the second buffer and the emission's queue. The four passes
+        // end where they began: the items in dval0 whichever way they came, as a rebuild reads them.
         uint32_t* sk[2] = {dk[0], dk[1]};
         uint32_t* sv[2] = {dv[0], dv[1]};
         const uint32_t* n_sort = &hdr->n_items;
         uint32_t* hist = reinterpret_cast<uint32_t*>(w + c->L.sort_hist);
         if (c->partition) {
             if (launch_partition(dk[0], (uint32_t)c->geo.n_items, reinterpret_cast<unsigned long long*>(w + c->L.block_sums),
-                                 hdr, hist, hist + 4 * 256, dk[1], dv[1], st, &c->launches) != cudaSuccess)
+                                 hdr, hist, hist + 4 * 256, dk[1], dv[0], st, &c->launches) != cudaSuccess)
                 return ODGS_ERR_CUDA;
             sk[0] = dk[1];
-            sv[0] = dv[1];
             sk[1] = reinterpret_cast<uint32_t*>(w + c->L.big);
-            sv[1] = sk[1] + c->geo.n_items;
             n_sort = &hdr->n_visible_sort;
             hist += 4 * 256;
         }
@@ -513,15 +510,14 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
                               &hdr->status, c->num_sms, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions,
                               /*cleared=*/true) != cudaSuccess)
             return ODGS_ERR_CUDA;
-        if (c->partition) rb = 1;  // four passes end where they began
-        c->depth_buf = rb;
+        c->depth_buf = c->partition ? 1 : 0;
     }
     // 2. emit (tile, item) pairs in depth order
     uint8_t* p = c->pb;
     uint32_t* pk[2] = {reinterpret_cast<uint32_t*>(p + c->P.keys0), reinterpret_cast<uint32_t*>(p + c->P.keys1)};
     uint32_t* pv[2] = {reinterpret_cast<uint32_t*>(p + c->P.vals0), reinterpret_cast<uint32_t*>(p + c->P.vals1)};
     BinArgs b{};
-    b.sorted_idx = dv[rb];
+    b.sorted_idx = dv[0];
     b.rect = reinterpret_cast<const uint4*>(w + c->L.rect);
     b.rect2 = reinterpret_cast<const uint4*>(w + c->L.rect2);
     b.srect = reinterpret_cast<uint4*>(w + c->L.srect);
@@ -541,10 +537,11 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     b.num_sms = c->num_sms;
     b.key_hist = reinterpret_cast<uint32_t*>(p + c->P.hist);
     b.key_passes = radix_passes(c->geo.key_bits);
-    if (truncate && c->geo.n_items > 0) {
+    if (c->L.truncate && c->geo.n_items > 0) {
+        b.truncate = truncate;
         b.cut = w + c->L.cut;
         b.G = reinterpret_cast<const uint32_t*>(w + c->L.cover);
-        b.sorted_keys = dk[rb];
+        b.sorted_keys = dk[c->depth_buf];
         uint32_t rn;
         std::memcpy(&rn, &c->s.r_near, sizeof(rn));
         b.base = rn >> kCutShift;
@@ -552,7 +549,6 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         b.kcount = reinterpret_cast<uint32_t*>(w + c->L.kcount);
     }
     b.emit_only = rebuild;
-    b.visible_first = c->partition;
     if (!rebuild && c->geo.n_items > 0) {  // the pair count clears the ranges
         b.ranges_zero = reinterpret_cast<uint2*>(w + c->L.ranges);
         b.n_ranges = (uint32_t)c->geo.total_tiles;
@@ -717,6 +713,7 @@ odgs_status odgs_preprocess_bwd(odgs_ctx* c, const odgs_grads* grads, void* stre
     b.dilation = c->s.cov_dilation;
     b.acc = reinterpret_cast<const float4*>(w + c->L.acc);
     if (c->partition) b.keys = reinterpret_cast<const uint32_t*>(w + c->L.dkey0);
+    b.hdr = reinterpret_cast<const Header*>(w + c->L.hdr);
     b.g_means = grads->means; b.g_scales = grads->scales; b.g_quats = grads->quats;
     b.g_opacity = grads->opacity; b.g_sh = grads->sh;
     b.accumulate = c->s.grad_accumulate;
@@ -775,7 +772,7 @@ odgs_status odgs_debug_lists(odgs_ctx* c, uint32_t* depth_keys, uint32_t* depth_
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint8_t* w = c->ws;
     const uint8_t* p = c->pb;
-    const size_t dk = c->depth_buf ? c->L.dkey1 : c->L.dkey0, dv = c->depth_buf ? c->L.dval1 : c->L.dval0;
+    const size_t dk = c->depth_buf ? c->L.dkey1 : c->L.dkey0, dv = c->L.dval0;
     const size_t pk = c->pair_buf ? c->P.keys1 : c->P.keys0, pv = c->pair_buf ? c->P.vals1 : c->P.vals0;
     struct Copy {
         void* dst;

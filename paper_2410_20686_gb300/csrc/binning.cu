@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
         for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < a.n_ranges; t += gridDim.x * blockDim.x)
             a.ranges_zero[t] = make_uint2(0u, 0u);
     // culled items end the depth order
-    const uint32_t n_vis = a.visible_first ? (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible) : a.n_items;
+    const uint32_t n_vis = (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible);
     if (base >= n_vis) {
         if (threadIdx.x == 0) a.block_sums[blockIdx.x] = 0ull;
         return;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
             if (idx < a.n_items) rc = a.rect[idx];
             a.srect[k] = rc;
         }
-        if (!a.G) {
+        if (!a.truncate) {
             c += rc.y;
             continue;
         }
@@ -212,7 +212,7 @@ __device__ __forceinline__ unsigned long long scan_totals(unsigned long long* __
 
 __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __restrict__ block_sums, int nblocks,
                                                       Header* hdr, unsigned long long capacity,
-                                                      uint32_t* __restrict__ key_hist) {
+                                                      uint32_t* __restrict__ key_hist, bool truncate) {
     // the tile sort's digit counts, which the emission adds up, start from 0
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) key_hist[i] = 0u;
     const unsigned long long total = scan_totals(block_sums, nblocks);
@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
         hdr->n_big = 0u;
         hdr->n_huge = 0u;
         hdr->n_count_big = 0u;
+        hdr->kept_pairs = truncate ? 1u : 0u;
         if (total > capacity) atomicOr(&hdr->status, kStCapacity);
     }
 }
@@ -381,8 +382,9 @@ __global__ void __launch_bounds__(kScanThreads, 8) k_emit(EmitArgs a) {
     for (int r = 0; r < 2; ++r)
         for (size_t i = (size_t)blockIdx.x * kScanThreads + tid; i < a.clear_quads[r]; i += (size_t)gridDim.x * kScanThreads)
             a.clear[r][i] = make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t n_vis = a.visible_first ? (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible) : a.n_items;
+    const uint32_t n_vis = (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible);
     if (base >= n_vis) return;
+    const uint32_t* kcount = a.kcount && a.hdr->kept_pairs ? a.kcount : nullptr;
     __syncthreads();
     for (int round = 0; round < kScanItems; ++round) {
         const uint32_t k = base + (uint32_t)(round * kScanThreads + tid);
@@ -390,9 +392,9 @@ __global__ void __launch_bounds__(kScanThreads, 8) k_emit(EmitArgs a) {
         // as k_count_blocks read it (no tiles for an index past the end, after a depth sort that gave up)
         const uint4 rc = k < n_vis ? a.srect[k] : make_uint4(0u, 0u, 0u, 0u);
         // kept pairs (the scan) and the item's whole footprint (warp or shared emission)
-        const uint32_t kw = (a.kcount && k < n_vis) ? a.kcount[k] : rc.y;
-        const uint32_t cnt = a.kcount ? (kw & 0x3FFFFFFu) : rc.y;
-        const int bk = (a.kcount && cnt < rc.y) ? (int)(kw >> 26) : -1;
+        const uint32_t kw = (kcount && k < n_vis) ? kcount[k] : rc.y;
+        const uint32_t cnt = kcount ? (kw & 0x3FFFFFFu) : rc.y;
+        const int bk = (kcount && cnt < rc.y) ? (int)(kw >> 26) : -1;
         const int nb = (int)(rc.x >> 16);
         const bool one = cnt > 0u && rc.y <= kSmallTiles && nb <= kStoredBands;
         // block-wide exclusive scan of the counts of this round (items in depth order)
@@ -474,6 +476,7 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t n_parts = a.hdr->n_huge * kHugeParts, n_all = n_parts + a.hdr->n_big;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const bool kept = a.kcount && a.hdr->kept_pairs;
     // static round-robin over the parts of the huge items, then the others: no shared counter to contend on
     for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_all; i += nwarps) {
         const bool huge = i < n_parts;
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
         const uint32_t idx = a.sorted_idx[e.x];
         const uint4 rc = a.srect[e.x];
         int bucket = -1;
-        if (a.kcount) {
+        if (kept) {
             const uint32_t kw = a.kcount[e.x];
             if ((kw & 0x3FFFFFFu) < rc.y) bucket = (int)(kw >> 26);
         }
@@ -628,14 +631,14 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         k_count_blocks<<<nb, kScanThreads, 0, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *launches += 1;
-        if (a.G) {
+        if (a.truncate) {
             k_count_big<<<a.num_sms * 8, 256, 0, st>>>(a);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             *launches += 1;
         }
     }
     if (!a.emit_only) {
-        k_scan_blocks<<<1, 1024, 0, st>>>(a.block_sums, nb, a.hdr, a.capacity, a.key_hist);
+        k_scan_blocks<<<1, 1024, 0, st>>>(a.block_sums, nb, a.hdr, a.capacity, a.key_hist, a.truncate);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *launches += 1;
     }
@@ -646,9 +649,8 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         ea.n_per_view = a.n_per_view; ea.n_items = a.n_items; ea.tile_w = a.tile_w; ea.tile_h = a.tile_h;
         ea.block_offsets = a.block_sums; ea.capacity = a.capacity; ea.keys = a.keys; ea.vals = a.vals;
         ea.big = a.big; ea.hdr = a.hdr;
-        ea.visible_first = a.visible_first;
         ea.key_hist = a.key_hist; ea.key_passes = a.key_passes;
-        ea.kcount = a.G ? a.kcount : nullptr;
+        ea.kcount = a.kcount;
         for (int r = 0; r < 2; ++r) { ea.clear[r] = a.clear[r]; ea.clear_quads[r] = a.clear_quads[r]; }
         ea.cut = a.cut;
         ea.G = a.G;

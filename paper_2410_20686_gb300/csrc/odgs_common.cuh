@@ -89,6 +89,10 @@ struct Header {
     uint32_t n_huge;                  // items queued for several warps each (cleared together with n_big)
     uint32_t n_count_big;             // items queued for the warp-wide kept-pair count
     uint32_t n_visible_sort;          // visible items, of a depth order partitioned before its sort
+    // how the passes that ran last left the workspace, for later ones: the host's own record is of the calls
+    // it made, which a replayed graph does not make again
+    uint32_t kept_pairs;              // 1: the block offsets count the kept pairs, 0: whole footprints
+    uint32_t partitioned;             // 1: the depth keys by item stay as the projection wrote them
     uint32_t pad;
 };
 

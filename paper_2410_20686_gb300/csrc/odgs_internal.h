@@ -79,7 +79,8 @@ struct PreBwdArgs {
     const ViewDev* views;
     float dilation;
     const float4* acc;
-    const uint32_t* keys;            // depth keys by item (all ones: culled) where most items are culled, or null
+    const uint32_t* keys;            // depth keys where most items are culled (all ones: culled), or null
+    const Header* hdr;               // says whether they still lie by item
     float *g_means, *g_scales, *g_quats, *g_opacity, *g_sh;
     int accumulate;
     int raw;                         // gradients w.r.t. log-scales and opacity logits
@@ -98,7 +99,6 @@ struct BinArgs {
     const ViewDev* views;
     int n_per_view;
     uint32_t n_items;
-    bool visible_first;  // the items past hdr->visible are culled: not read
     unsigned long long* block_sums;
     Header* hdr;
     unsigned long long capacity;
@@ -107,9 +107,9 @@ struct BinArgs {
     int num_sms;
     uint32_t* key_hist;  // [passes][256] digit histograms of the emitted tile ids (zeroed here)
     int key_passes;
-    // truncated lists (saturation.cu), or null: per tile the last depth bucket it keeps and per
-    // bucket the prefix counts over the tiles of cut >= bucket; the depth-sorted keys (buckets);
-    // per depth-order position the kept pairs | bucket << 26 (written by k_count_blocks)
+    // frames that may have truncated lists (saturation.cu), or null: per tile the last depth bucket it
+    // keeps and per bucket the prefix counts over the tiles of cut >= bucket; the depth-sorted keys
+    // (buckets); per depth-order position the kept pairs | bucket << 26 (written by k_count_blocks)
     const uint8_t* cut;
     const uint32_t* G;
     const uint32_t* sorted_keys;
@@ -117,6 +117,7 @@ struct BinArgs {
     uint32_t n_ranges;
     uint32_t base, total_tiles;
     uint32_t* kcount;
+    bool truncate;  // count the kept pairs (an emission follows what the last count did)
     // the pair counts, their scan and the kept-pair words of this depth order are in place from an
     // earlier binning of the same frame: emit only (a rebuild of the lists for the backward pass)
     bool emit_only;
@@ -132,7 +133,6 @@ struct EmitArgs {
     const ViewDev* views;
     int n_per_view;
     uint32_t n_items;
-    bool visible_first;
     int tile_w, tile_h;
     const unsigned long long* block_offsets;
     unsigned long long capacity;
@@ -141,7 +141,7 @@ struct EmitArgs {
     Header* hdr;
     uint32_t* key_hist;
     int key_passes;
-    const uint32_t* kcount;  // by depth-order position, or null
+    const uint32_t* kcount;  // by depth-order position, read if the last count was of kept pairs; or null
     const uint8_t* cut;
     const uint32_t* G;  // prefix counts of the tiles that keep a bucket, with kcount
     uint32_t total_tiles;
@@ -196,7 +196,7 @@ struct BwdArgs {
 };
 
 cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Header* hdr, int total_trig,
-                         uint32_t* dhist, uint4* clear, size_t clear_quads, cudaStream_t st);
+                         uint32_t* dhist, uint4* clear, size_t clear_quads, bool partition, cudaStream_t st);
 // projected: recorded once the projection (records, pairs, keys) is done, before the colours; or null
 cudaError_t launch_preprocess(const PreArgs& a, int sh_degree, cudaStream_t st, cudaEvent_t projected = nullptr);
 cudaError_t launch_preprocess_bwd(const PreBwdArgs& a, int sh_degree, cudaStream_t st);

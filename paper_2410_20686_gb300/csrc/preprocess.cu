@@ -16,7 +16,7 @@ namespace odgs {
 // ------------------------------------------------------------------ setup
 
 __global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr, int total_trig, uint32_t* dhist,
-                        uint4* clear, size_t clear_quads) {
+                        uint4* clear, size_t clear_quads, bool partition) {
     int gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid < tab.n_views) views[gid] = tab.v[gid];
     // the depth sort's digit histograms, counted by k_preprocess_geom
@@ -38,6 +38,7 @@ __global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr
         hdr->work_bwd = 0u;
         hdr->n_big = 0u;
         hdr->n_huge = 0u;
+        hdr->partitioned = partition ? 1u : 0u;
         hdr->n_count_big = 0u;  // the binning's queue counters (each binning leaves them at 0)
     }
     for (int e = gid; e < total_trig; e += gridDim.x * blockDim.x) {
@@ -673,9 +674,11 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
     }
     const uint32_t st_count0 = st_count;
     unsigned long long seen = 0ull;  // KEYED: bit v set where view v does not cull the Gaussian
-    if (KEYED)
+    if (KEYED) {
+        const bool by_item = a.hdr->partitioned != 0u;
         for (int v = 0; v < a.n_views; ++v)
-            seen |= (unsigned long long)(__ldg(a.keys + (size_t)v * a.n + g) != 0xFFFFFFFFu) << v;
+            seen |= (unsigned long long)(!by_item || __ldg(a.keys + (size_t)v * a.n + g) != 0xFFFFFFFFu) << v;
+    }
     auto after = [&](int v) {  // the view to take after v
         if (!KEYED) return v + 1;
         const unsigned long long m = v < kMaxViews - 1 ? seen >> (v + 1) : 0ull;
@@ -1078,12 +1081,12 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
 // ------------------------------------------------------------------ launchers
 
 cudaError_t launch_setup(const ViewTable& tab, ViewDev* views, float4* trig, Header* hdr, int total_trig,
-                         uint32_t* dhist, uint4* clear, size_t clear_quads, cudaStream_t st) {
+                         uint32_t* dhist, uint4* clear, size_t clear_quads, bool partition, cudaStream_t st) {
     int threads = 256;
     int blocks = (max(total_trig, tab.n_views) + threads - 1) / threads;
     blocks = max(blocks, (int)min(clear_quads / (4 * (size_t)threads), (size_t)1024));
     blocks = max(1, min(blocks, 1024));
-    k_setup<<<blocks, threads, 0, st>>>(tab, views, trig, hdr, total_trig, dhist, clear, clear_quads);
+    k_setup<<<blocks, threads, 0, st>>>(tab, views, trig, hdr, total_trig, dhist, clear, clear_quads, partition);
     return cudaGetLastError();
 }
 

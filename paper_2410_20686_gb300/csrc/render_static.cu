@@ -127,7 +127,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
 
     // ---- the forward path (same kernels as the workspace entry points)
     int launches = 0;
-    if (launch_setup(tab, vd, trig, hdr, geo.total_trig, d_hist, nullptr, 0, strm) != cudaSuccess) return ODGS_ERR_CUDA;
+    if (launch_setup(tab, vd, trig, hdr, geo.total_trig, d_hist, nullptr, 0, false, strm) != cudaSuccess) return ODGS_ERR_CUDA;
     PreArgs a{};
     a.means = g->means; a.scales = g->scales; a.quats = g->quats; a.opacity = g->opacity; a.sh = g->sh;
     a.n = g->n; a.n_views = 1; a.sh_coeffs = st.sh_coeffs;
