@@ -508,7 +508,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         if (launch_radix_sort(sk, sv, n_sort, c->geo.n_items, 32, hist,
                               reinterpret_cast<uint32_t*>(w + c->L.sort_ctr), reinterpret_cast<uint32_t*>(w + c->L.sort_lb),
                               &hdr->status, c->num_sms, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions,
-                              /*cleared=*/true) != cudaSuccess)
+                              /*cleared=*/true, c->partition ? nullptr : &hdr->by_item) != cudaSuccess)
             return ODGS_ERR_CUDA;
         c->depth_buf = c->partition ? 1 : 0;
     }
@@ -549,6 +549,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         b.kcount = reinterpret_cast<uint32_t*>(w + c->L.kcount);
     }
     b.emit_only = rebuild;
+    b.partition = c->partition;
     if (!rebuild && c->geo.n_items > 0) {  // the pair count clears the ranges
         b.ranges_zero = reinterpret_cast<uint2*>(w + c->L.ranges);
         b.n_ranges = (uint32_t)c->geo.total_tiles;

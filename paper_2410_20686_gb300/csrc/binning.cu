@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
         for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < a.n_ranges; t += gridDim.x * blockDim.x)
             a.ranges_zero[t] = make_uint2(0u, 0u);
     // culled items end the depth order
-    const uint32_t n_vis = (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible);
+    const uint32_t n_vis = a.partition ? (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible) : a.n_items;
     if (base >= n_vis) {
         if (threadIdx.x == 0) a.block_sums[blockIdx.x] = 0ull;
         return;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_blocks(BinArgs a) {
             if (idx < a.n_items) rc = a.rect[idx];
             a.srect[k] = rc;
         }
-        if (!a.truncate) {
+        if (!a.G) {
             c += rc.y;
             continue;
         }
@@ -212,7 +212,7 @@ __device__ __forceinline__ unsigned long long scan_totals(unsigned long long* __
 
 __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __restrict__ block_sums, int nblocks,
                                                       Header* hdr, unsigned long long capacity,
-                                                      uint32_t* __restrict__ key_hist, bool truncate) {
+                                                      uint32_t* __restrict__ key_hist, bool truncate, bool partition) {
     // the tile sort's digit counts, which the emission adds up, start from 0
     for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) key_hist[i] = 0u;
     const unsigned long long total = scan_totals(block_sums, nblocks);
@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
         hdr->n_huge = 0u;
         hdr->n_count_big = 0u;
         hdr->kept_pairs = truncate ? 1u : 0u;
+        hdr->by_item = partition ? 1u : 0u;
         if (total > capacity) atomicOr(&hdr->status, kStCapacity);
     }
 }
@@ -382,9 +383,10 @@ __global__ void __launch_bounds__(kScanThreads, 8) k_emit(EmitArgs a) {
     for (int r = 0; r < 2; ++r)
         for (size_t i = (size_t)blockIdx.x * kScanThreads + tid; i < a.clear_quads[r]; i += (size_t)gridDim.x * kScanThreads)
             a.clear[r][i] = make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t n_vis = (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible);
+    // (culled items end both depth orders, so a rebuild need not know which it was)
+    const uint32_t n_vis = a.visible_first ? (uint32_t)min((unsigned long long)a.n_items, a.hdr->visible) : a.n_items;
     if (base >= n_vis) return;
-    const uint32_t* kcount = a.kcount && a.hdr->kept_pairs ? a.kcount : nullptr;
+    const uint32_t* kcount = a.rebuild && !a.hdr->kept_pairs ? nullptr : a.kcount;
     __syncthreads();
     for (int round = 0; round < kScanItems; ++round) {
         const uint32_t k = base + (uint32_t)(round * kScanThreads + tid);
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(256, 4) k_emit_big(EmitArgs a) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t n_parts = a.hdr->n_huge * kHugeParts, n_all = n_parts + a.hdr->n_big;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const bool kept = a.kcount && a.hdr->kept_pairs;
+    const bool kept = a.kcount && !(a.rebuild && !a.hdr->kept_pairs);
     // static round-robin over the parts of the huge items, then the others: no shared counter to contend on
     for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_all; i += nwarps) {
         const bool huge = i < n_parts;
@@ -628,7 +630,9 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         if ((e = cudaMemsetAsync(&a.hdr->n_big, 0, 2 * sizeof(uint32_t), st)) != cudaSuccess) return e;
     } else if (nb > 0) {
         // the kept-count queue counter is 0: cleared by the preprocess's setup and by every scan
-        k_count_blocks<<<nb, kScanThreads, 0, st>>>(a);
+        BinArgs ca = a;
+        if (!a.truncate) ca.G = nullptr;  // whole footprints
+        k_count_blocks<<<nb, kScanThreads, 0, st>>>(ca);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *launches += 1;
         if (a.truncate) {
@@ -638,7 +642,7 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         }
     }
     if (!a.emit_only) {
-        k_scan_blocks<<<1, 1024, 0, st>>>(a.block_sums, nb, a.hdr, a.capacity, a.key_hist, a.truncate);
+        k_scan_blocks<<<1, 1024, 0, st>>>(a.block_sums, nb, a.hdr, a.capacity, a.key_hist, a.truncate, a.partition);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *launches += 1;
     }
@@ -650,7 +654,9 @@ cudaError_t launch_binning(const BinArgs& a, cudaStream_t st, int* launches) {
         ea.block_offsets = a.block_sums; ea.capacity = a.capacity; ea.keys = a.keys; ea.vals = a.vals;
         ea.big = a.big; ea.hdr = a.hdr;
         ea.key_hist = a.key_hist; ea.key_passes = a.key_passes;
-        ea.kcount = a.kcount;
+        ea.kcount = a.truncate || a.emit_only ? a.kcount : nullptr;
+        ea.rebuild = a.emit_only;
+        ea.visible_first = a.partition || a.emit_only;
         for (int r = 0; r < 2; ++r) { ea.clear[r] = a.clear[r]; ea.clear_quads[r] = a.clear_quads[r]; }
         ea.cut = a.cut;
         ea.G = a.G;

@@ -92,7 +92,7 @@ struct Header {
     // how the passes that ran last left the workspace, for later ones: the host's own record is of the calls
     // it made, which a replayed graph does not make again
     uint32_t kept_pairs;              // 1: the block offsets count the kept pairs, 0: whole footprints
-    uint32_t partitioned;             // 1: the depth keys by item stay as the projection wrote them
+    uint32_t by_item;                 // 1: the depth keys lie by item (an item's index goes without saying)
     uint32_t pad;
 };
 

@@ -117,9 +117,11 @@ struct BinArgs {
     uint32_t n_ranges;
     uint32_t base, total_tiles;
     uint32_t* kcount;
-    bool truncate;  // count the kept pairs (an emission follows what the last count did)
+    bool truncate;   // count the kept pairs
+    bool partition;  // the items past hdr->visible are culled: not read
     // the pair counts, their scan and the kept-pair words of this depth order are in place from an
-    // earlier binning of the same frame: emit only (a rebuild of the lists for the backward pass)
+    // earlier binning of the same frame: emit only (a rebuild of the lists for the backward pass), as the
+    // header says that binning counted, whatever truncate and partition are
     bool emit_only;
     uint4* clear[2];  // cleared by k_emit: the tile sort's scratch, the depth sort's (or null)
     size_t clear_quads[2];
@@ -133,6 +135,8 @@ struct EmitArgs {
     const ViewDev* views;
     int n_per_view;
     uint32_t n_items;
+    bool rebuild;        // kcount counts only if the header says so
+    bool visible_first;  // the items past hdr->visible are culled: not read
     int tile_w, tile_h;
     const unsigned long long* block_offsets;
     unsigned long long capacity;
@@ -141,7 +145,7 @@ struct EmitArgs {
     Header* hdr;
     uint32_t* key_hist;
     int key_passes;
-    const uint32_t* kcount;  // by depth-order position, read if the last count was of kept pairs; or null
+    const uint32_t* kcount;  // by depth-order position, or null
     const uint8_t* cut;
     const uint32_t* G;  // prefix counts of the tiles that keep a bucket, with kcount
     uint32_t total_tiles;
@@ -209,7 +213,8 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
                               uint32_t* hist, uint32_t* tile_ctrs, uint32_t* lookback, uint32_t* status, int num_sms,
                               cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit,
                               int lb_regions = 1,     // look-back regions of radix_lookback_words each
-                              bool cleared = false);  // counters and regions are already 0
+                              bool cleared = false,   // counters and regions are already 0
+                              const uint32_t* implied = nullptr);  // device word: 1 if the values are 0, 1, 2, ...
 // A sort whose four tile counters lie kCtrBytes before its look-back regions (one per pass) clears
 // both at once (sort_scratch_quads 16-byte groups).
 constexpr size_t kCtrBytes = 256;

@@ -38,7 +38,7 @@ __global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr
         hdr->work_bwd = 0u;
         hdr->n_big = 0u;
         hdr->n_huge = 0u;
-        hdr->partitioned = partition ? 1u : 0u;
+        hdr->by_item = partition ? 1u : 0u;
         hdr->n_count_big = 0u;  // the binning's queue counters (each binning leaves them at 0)
     }
     for (int e = gid; e < total_trig; e += gridDim.x * blockDim.x) {
@@ -675,9 +675,10 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
     const uint32_t st_count0 = st_count;
     unsigned long long seen = 0ull;  // KEYED: bit v set where view v does not cull the Gaussian
     if (KEYED) {
-        const bool by_item = a.hdr->partitioned != 0u;
+        const uint32_t by_item = a.hdr->by_item;
         for (int v = 0; v < a.n_views; ++v)
-            seen |= (unsigned long long)(!by_item || __ldg(a.keys + (size_t)v * a.n + g) != 0xFFFFFFFFu) << v;
+            seen |= (unsigned long long)(__ldg(a.keys + (size_t)v * a.n + g) != 0xFFFFFFFFu) << v;
+        if (!by_item) seen = ~0ull >> (64 - a.n_views);
     }
     auto after = [&](int v) {  // the view to take after v
         if (!KEYED) return v + 1;

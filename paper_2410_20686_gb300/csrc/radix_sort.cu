@@ -56,13 +56,15 @@ __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <int kSortItems>
+// IMPLIED: where *implied is 1 the values read are dropped: each is its key's place. (A kernel of its own for the
+// pass that may need it: a choice at run time in every pass cost a frame of 8 views 25.48 -> 25.75 ms.)
+template <int kSortItems, bool IMPLIED>
 __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                                          uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                          const uint32_t* __restrict__ n_ptr, int shift,
                                                          int bits, const uint32_t* __restrict__ hist,
                                                          uint32_t* lookback, uint32_t* tile_ctr, uint32_t* status,
-                                                         uint32_t wait_limit) {
+                                                         uint32_t wait_limit, const uint32_t* implied) {
     extern __shared__ uint2 s_dyn[];
     uint32_t (*s_mask)[kRadix] = reinterpret_cast<uint32_t (*)[kRadix]>(s_dyn);  // [warps] lanes
     uint32_t (*s_cnt)[kRadix] = s_mask + kSortWarps;                             // [warps] counts
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t n = *n_ptr;
+    const bool by_index = IMPLIED && *implied;
     const uint32_t mask = (1u << bits) - 1u;
     const uint32_t lt = (1u << lane) - 1u;
     // global digit offset of this pass (exclusive scan of the global histogram), the same for
@@ -105,6 +108,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
             const bool valid = idx < n;
             key[i] = valid ? kin[idx] : 0u;
             val[i] = valid ? vin[idx] : 0u;
+            if (IMPLIED && by_index) val[i] = idx;
         }
         // stable warp-level ranking: items are ordered by (warp, i, lane).
 #pragma unroll
@@ -219,6 +223,17 @@ constexpr size_t onesweep_smem(int items) {
     return kSortWarps * kRadix * sizeof(uint2) + 2 * sizeof(uint32_t) * (size_t)kSortThreads * items;
 }
 
+using OnesweepKernel = decltype(&k_onesweep<kSortItemsMax, false>);
+static OnesweepKernel onesweep(bool large, bool implied) {
+    if (large) return implied ? k_onesweep<kSortItemsMax, true> : k_onesweep<kSortItemsMax, false>;
+    return implied ? k_onesweep<kSortItemsMax / 2, true> : k_onesweep<kSortItemsMax / 2, false>;
+}
+
+static void set_onesweep_attributes(OnesweepKernel k, int items) {
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)onesweep_smem(items));
+}
+
 int radix_passes(int bits) { return (bits + 7) / 8; }
 
 // Look-back words for the smaller (2048-key) tile, which needs the most.
@@ -230,11 +245,12 @@ size_t radix_lookback_words(size_t max_items) {
 
 // Sorts (k[0], v[0]) by key bits [0, bits); returns the buffer index (0 or 1) that holds the
 // result. hist: the digit counts of all passes, [passes][256], from the kernels that wrote the keys.
-// scratch: tile counters [4] + lookback [radix_lookback_words].
+// scratch: tile counters [4] + lookback [radix_lookback_words]. implied: a device word or null; where it is 1,
+// v[0] is not read and the values are 0, 1, 2, ...
 cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_ptr, size_t max_items, int bits,
                               uint32_t* hist, uint32_t* tile_ctrs, uint32_t* lookback, uint32_t* status, int num_sms,
                               cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit, int lb_regions,
-                              bool cleared) {
+                              bool cleared, const uint32_t* implied) {
     const int passes = radix_passes(bits);
     *result_buf = 0;
     if (passes == 0 || max_items == 0) return cudaSuccess;
@@ -246,16 +262,15 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
     if (!ctr_with_lb && !cleared && (e = cudaMemsetAsync(tile_ctrs, 0, sizeof(uint32_t) * 4, st)) != cudaSuccess) return e;
     static bool carveout_set = false;  // all of the SM's shared memory for the onesweep CTAs
     if (!carveout_set) {
-        cudaFuncSetAttribute(k_onesweep<kSortItemsMax>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(k_onesweep<kSortItemsMax / 2>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(k_onesweep<kSortItemsMax>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)onesweep_smem(kSortItemsMax));
+        set_onesweep_attributes(k_onesweep<kSortItemsMax, false>, kSortItemsMax);
+        set_onesweep_attributes(k_onesweep<kSortItemsMax, true>, kSortItemsMax);
+        set_onesweep_attributes(k_onesweep<kSortItemsMax / 2, false>, kSortItemsMax / 2);
+        set_onesweep_attributes(k_onesweep<kSortItemsMax / 2, true>, kSortItemsMax / 2);
         carveout_set = true;
     }
     const bool large = max_items >= kLargeSort;
     const int per_cta = kSortThreads * (large ? kSortItemsMax : kSortItemsMax / 2);
+    const size_t smem = onesweep_smem(large ? kSortItemsMax : kSortItemsMax / 2);
     const size_t lb_words = radix_lookback_words(max_items);
     const int tiles = (int)((max_items + per_cta - 1) / per_cta);
     // persistent CTAs: as many as fit at once, at most one per tile
@@ -263,10 +278,7 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
     int& res = resident[large ? 1 : 0];
     if (res == 0) {
         int per_sm = 0;
-        if (large)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<kSortItemsMax>, kSortThreads, onesweep_smem(kSortItemsMax));
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<kSortItemsMax / 2>, kSortThreads, onesweep_smem(kSortItemsMax / 2));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, onesweep(large, true), kSortThreads, smem);
         res = max(per_sm, 1);
     }
     const int grid = max(min(tiles, res * num_sms), 1);
@@ -283,14 +295,9 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
         const int pbits = min(8, bits - shift);
         uint32_t* lb = regions ? lookback + (size_t)p * lb_words : lookback;
         if (!regions && (e = cudaMemsetAsync(lb, 0, sizeof(uint32_t) * lb_words, st)) != cudaSuccess) return e;
-        if (large)
-            k_onesweep<kSortItemsMax><<<grid, kSortThreads, onesweep_smem(kSortItemsMax), st>>>(
-                k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits,
-                hist + p * kRadix, lb, tile_ctrs + p, status, wait_limit);
-        else
-            k_onesweep<kSortItemsMax / 2><<<grid, kSortThreads, onesweep_smem(kSortItemsMax / 2), st>>>(
-                k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits,
-                hist + p * kRadix, lb, tile_ctrs + p, status, wait_limit);
+        onesweep(large, implied && p == 0)<<<grid, kSortThreads, smem, st>>>(
+            k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], n_ptr, shift, pbits, hist + p * kRadix, lb, tile_ctrs + p, status,
+            wait_limit, implied);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         *launches += 1;
         cur ^= 1;

@@ -97,3 +97,13 @@ def test_backward_after_a_replay_and_an_eager_frame_of_another_camera(first, reb
     got = r.backward(w)
     assert r.status() == 0 and all(torch.equal(a, b) for a, b in zip(imgs, want_imgs))
     _check_grads(got, want)
+    alone = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(alone):
+        r.preprocess(*p, views, rs)
+    r.forward(*p, other, rs)
+    alone.replay()  # the projection alone: the binning is the host's
+    r.bin_sort()
+    imgs, _ = r.render_fwd(want_T=False)
+    got = r.backward(w)
+    assert r.status() == 0 and all(torch.equal(a, b) for a, b in zip(imgs, want_imgs))
+    _check_grads(got, want)
