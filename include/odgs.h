@@ -116,7 +116,9 @@ typedef struct {
                            pairs are emitted and sorted. Frames of more than 2^19 tiles keep
                            the whole lists, and so do frames whose pairs odgs_query_pairs or
                            odgs_wait_pairs has reported as at most 32768 when they all fit in
-                           the pair buffer. 1: the whole lists (every Gaussian whose footprint
+                           the pair buffer (but not in a captured odgs_bin_sort, nor once an
+                           odgs_preprocess of the context has been captured: a replay may
+                           bring more). 1: the whole lists (every Gaussian whose footprint
                            meets the tile)                                                 */
 } odgs_settings;
 
@@ -171,8 +173,9 @@ odgs_status odgs_query_pairs(odgs_ctx *ctx, size_t *pairs, void *stream);
 
 /* As odgs_query_pairs, but right after odgs_preprocess it waits only for the projection, not for the
  * colours that the stream computes after it, so that the caller can queue odgs_bin_sort while they
- * run. (The first call of a context, calls in later stages and calls after a captured
- * odgs_preprocess synchronize the stream as odgs_query_pairs does.) */
+ * run. (The first call of a context, calls in later stages and all calls once an odgs_preprocess of
+ * the context has been captured in a graph, which may have been replayed since, synchronize the
+ * stream as odgs_query_pairs does.) */
 odgs_status odgs_wait_pairs(odgs_ctx *ctx, size_t *pairs, void *stream);
 
 /* Depth sort, per-tile pair emission and stable tile sort (the "sorting by depth" of Sec.

@@ -227,6 +227,9 @@ struct odgs_ctx {
     bool pairs_known = false;
     size_t pairs = 0;
     bool partition = false;  // visible items first, and only they are depth-sorted (partitions())
+    // a preprocess of this context has been captured: a replay may have run since the calls the host knows
+    // of, so its record of the frame (cuts, pairs, the projection's event) is not relied on
+    bool captured = false;
     // a second stream on which the binning computes the cuts while the depth sort runs (forked
     // from and joined back to the caller's stream by events)
     cudaStream_t side = nullptr;
@@ -292,6 +295,13 @@ odgs_status odgs_pair_buffer_size(size_t cap, size_t* bytes) {
     return ODGS_OK;
 }
 
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the launches that follow report what is wrong with the stream
+    return true;
+}
+
 static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
     uint8_t* w = c->ws;
     Header* hdr = reinterpret_cast<Header*>(w + c->L.hdr);
@@ -329,10 +339,9 @@ static odgs_status run_preprocess(odgs_ctx* c, cudaStream_t st) {
         a.cut_base = rn >> kCutShift;
     }
     a.hdr = hdr;
-    // an event of a capture could not be waited for outside it
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    const bool record = c->ev_pairs && cudaStreamIsCapturing(st, &capture) == cudaSuccess &&
-                        capture == cudaStreamCaptureStatusNone;
+    // an event of a capture could not be waited for outside it, and one from before a replay is past
+    if (capturing(st)) c->captured = true;
+    const bool record = c->ev_pairs && !c->captured;
     if (launch_preprocess(a, c->s.sh_degree, st, record ? c->ev_pairs : nullptr) != cudaSuccess) return ODGS_ERR_CUDA;
     c->pairs_recorded = record;
     if (c->n > 0) c->launches += 2;
@@ -455,12 +464,15 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     // saves nothing, and the cuts are five launches and four event calls of a frame that is bound by
     // its launches (1K Gaussians at 256 x 128, one view: 151 -> 134 us with this and the sorts'
     // scratch cleared by kernels instead of memsets).
-    // A rebuild emits what the count that ran last counted (Header::kept_pairs).
+    // A captured binning may be replayed on frames of any number of pairs; a rebuild emits what the count that
+    // ran last counted (Header::kept_pairs).
     constexpr size_t kFewPairs = 32768;
-    const bool few = c->pairs_known && c->pairs <= std::min(c->pb_cap, kFewPairs);
+    bool few = c->pairs_known && !c->captured && c->pairs <= std::min(c->pb_cap, kFewPairs);
+    bool cut_ready = c->cut_ready && !c->captured;
+    if ((few || cut_ready) && capturing(st)) few = cut_ready = false;
     const bool truncate = c->L.truncate && !few && !rebuild;
     // 0. which tiles saturate, and from which depth on
-    if (truncate && !c->cut_ready) {
+    if (truncate && !cut_ready) {
         SatArgs sa{};
         sa.rect = reinterpret_cast<const uint4*>(w + c->L.rect);
         sa.rec_a = reinterpret_cast<const float4*>(w + c->L.rec_a);

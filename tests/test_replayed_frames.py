@@ -78,6 +78,7 @@ def test_backward_after_a_replay_and_an_eager_frame_of_another_camera(first, reb
     from paper_2410_20686_gb300.rasterizer import Rasterizer, RenderSettings
     n, at = 22_000, (0.1, 0.0, -0.2)
     sc = S.random_scene(n, 64, 64, seed=43, sh_degree=1, radius=(0.1, 5.0), log_scale=(-4.0, 0.5))
+    sc.opacity[::5] = 0.001  # below 1 / 255: culled in every view
     kinds = {"perspective": S.cubemap_views(64, at), "erp": [S.yaw_view(64, 64, at, 0.7 * k) for k in range(6)]}
     views = kinds.pop(first)
     (other,) = kinds.values()
@@ -107,3 +108,64 @@ def test_backward_after_a_replay_and_an_eager_frame_of_another_camera(first, reb
     got = r.backward(w)
     assert r.status() == 0 and all(torch.equal(a, b) for a, b in zip(imgs, want_imgs))
     _check_grads(got, want)
+
+
+def _pairs(r, name):
+    import ctypes as C
+    from paper_2410_20686_gb300 import _lib as L
+    k = C.c_size_t()
+    assert getattr(r.lib, name)(r.ctx, C.byref(k), L.raw_stream(r.device)) == L.ODGS_OK
+    return int(k.value)
+
+
+def test_pair_count_after_a_replay_that_brings_more_pairs():
+    import torch
+    from paper_2410_20686_gb300.rasterizer import Rasterizer, RenderSettings
+    sc = _scene()
+    p, rs = to_torch(sc), RenderSettings(sh_degree=0)
+    scales = p[1].clone()
+    r = Rasterizer(capacity_mode="fixed")
+    r.reserve_pairs(1 << 17)
+    r.forward(*p, sc.views, rs)
+    many = _pairs(r, "odgs_query_pairs")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        r.preprocess(*p, sc.views, rs)
+    for _ in range(2):
+        p[1].copy_(0.05 * scales)
+        r.preprocess(*p, sc.views, rs)
+        few = _pairs(r, "odgs_wait_pairs")  # makes the event, or is the second eager frame
+        p[1].copy_(scales)
+        torch.cuda._sleep(20_000_000)  # the replay is still to come when the count is asked for
+        g.replay()
+        assert _pairs(r, "odgs_wait_pairs") == many > 4 * few
+
+
+def test_binning_captured_after_a_query_takes_any_number_of_pairs():
+    import torch
+    from paper_2410_20686_gb300.rasterizer import Rasterizer, RenderSettings
+    sc = _scene()
+    p, rs = to_torch(sc), RenderSettings(sh_degree=0)
+    ref = Rasterizer(capacity_mode="fixed")
+    ref.reserve_pairs(1 << 17)
+    (want,), _ = ref.forward(*p, sc.views, rs)
+    st = ref.stats()
+    cap = (st["pairs"] + st["pairs_sorted"]) // 2  # the cut lists fit, the whole ones do not
+    assert st["pairs_sorted"] < cap < st["pairs"]
+    r = Rasterizer(capacity_mode="fixed")
+    r.reserve_pairs(cap)
+    scales = p[1].clone()
+    p[1].copy_(0.05 * scales)
+    r.forward(*p, sc.views, rs)
+    assert r.query_pairs() < cap
+    r.preprocess(*p, sc.views, rs)
+    r.query_pairs()  # few pairs, which would fit
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        r.bin_sort()
+        (img,), _ = r.render_fwd(want_T=False)
+    p[1].copy_(scales)
+    r.preprocess(*p, sc.views, rs)
+    g.replay()
+    assert r.status() == 0 and r.stats()["pairs_sorted"] <= cap
+    assert torch.equal(img, want)
