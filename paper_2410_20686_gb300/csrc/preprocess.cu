@@ -897,8 +897,12 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
                     if (e < K * 3) col[e % 3] = fmaf(q[r], Y[e / 3], col[e % 3]);
                 }
             }
+            bool lit[3];  // not clamped; a clamped channel's coefficients, which may be infinite, count for nothing
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) msh[ch] = col[ch] < 0.f ? 0.f : drgb[ch];  // clamped channels
+            for (int ch = 0; ch < 3; ++ch) {
+                lit[ch] = !(col[ch] < 0.f);
+                msh[ch] = lit[ch] ? drgb[ch] : 0.f;
+            }
             if (DEG > 0) {
                 float w[16];
 #pragma unroll
@@ -916,7 +920,7 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
                         const int e = 4 * i + r;
-                        if (e < K * 3) w[e / 3] = fmaf(msh[e % 3], q[r], w[e / 3]);
+                        if (e < K * 3 && lit[e % 3]) w[e / 3] = fmaf(msh[e % 3], q[r], w[e / 3]);
                     }
                 }
                 float gx, gy, gz;
@@ -955,8 +959,12 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
             if (STAGED) {
                 float col[3], mc[3];
                 sh_row_colour<DEG>(row, Y, col);
+                bool lit[3];  // not clamped (as above)
 #pragma unroll
-                for (int ch = 0; ch < 3; ++ch) mc[ch] = col[ch] < 0.f ? 0.f : drgb[ch];  // clamped channels
+                for (int ch = 0; ch < 3; ++ch) {
+                    lit[ch] = !(col[ch] < 0.f);
+                    mc[ch] = lit[ch] ? drgb[ch] : 0.f;
+                }
 #pragma unroll
                 for (int i = 0; i < R::kChunks; ++i) {
                     const float4 q4 = row[i];
@@ -964,7 +972,7 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_bwd(PreBwdArgs a) {
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
                         const int e = 4 * i + r;
-                        wsum[e / 3] = fmaf(mc[e % 3], q[r], wsum[e / 3]);
+                        if (lit[e % 3]) wsum[e / 3] = fmaf(mc[e % 3], q[r], wsum[e / 3]);
                         gsh[ONE ? 0 : e / 3][e % 3] = fmaf(mc[e % 3], Y[e / 3], gsh[ONE ? 0 : e / 3][e % 3]);
                     }
                 }
