@@ -153,8 +153,10 @@ def load(path: str = LIB_PATH):
 
 
 def raw_stream(device) -> C.c_void_p:
-    """The device's current stream as a cudaStream_t."""
+    """The device's current stream as a cudaStream_t. Any other device is refused: its pointers are not the GPU's."""
     import torch
+    if device.type != "cuda":
+        raise ValueError(f"expected tensors on a CUDA device, not {device}")
     k = torch.cuda.current_device() if device.index is None else device.index
     return C.c_void_p(torch._C._cuda_getCurrentRawStream(k))
 
