@@ -16,6 +16,7 @@
 // consumer of the sorted arrays bounds the indices it reads.
 #include "odgs_common.cuh"
 #include "odgs_internal.h"
+#include "per_device.h"
 
 namespace odgs {
 
@@ -229,9 +230,19 @@ static OnesweepKernel onesweep(bool large, bool implied) {
     return implied ? k_onesweep<kSortItemsMax / 2, true> : k_onesweep<kSortItemsMax / 2, false>;
 }
 
-static void set_onesweep_attributes(OnesweepKernel k, int items) {
-    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)onesweep_smem(items));
+// CTAs of the kernels for large or smaller sorts that fit on an SM of the current device, with all of its shared
+// memory for them (with the static arrays the larger tile needs more than the 48 KB of a plain launch); 0 if
+// they cannot be launched there.
+static int resident_ctas(bool large, size_t smem) {
+    int per_sm = 0;
+    for (bool implied : {false, true}) {
+        const OnesweepKernel k = onesweep(large, implied);
+        if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kSortThreads, smem) != cudaSuccess)
+            return 0;
+    }
+    return per_sm;
 }
 
 int radix_passes(int bits) { return (bits + 7) / 8; }
@@ -260,26 +271,19 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
     const bool ctr_with_lb = lb_regions >= passes &&
                              reinterpret_cast<uint8_t*>(lookback) == reinterpret_cast<uint8_t*>(tile_ctrs) + kCtrBytes;
     if (!ctr_with_lb && !cleared && (e = cudaMemsetAsync(tile_ctrs, 0, sizeof(uint32_t) * 4, st)) != cudaSuccess) return e;
-    static bool carveout_set = false;  // all of the SM's shared memory for the onesweep CTAs
-    if (!carveout_set) {
-        set_onesweep_attributes(k_onesweep<kSortItemsMax, false>, kSortItemsMax);
-        set_onesweep_attributes(k_onesweep<kSortItemsMax, true>, kSortItemsMax);
-        set_onesweep_attributes(k_onesweep<kSortItemsMax / 2, false>, kSortItemsMax / 2);
-        set_onesweep_attributes(k_onesweep<kSortItemsMax / 2, true>, kSortItemsMax / 2);
-        carveout_set = true;
-    }
     const bool large = max_items >= kLargeSort;
     const int per_cta = kSortThreads * (large ? kSortItemsMax : kSortItemsMax / 2);
     const size_t smem = onesweep_smem(large ? kSortItemsMax : kSortItemsMax / 2);
     const size_t lb_words = radix_lookback_words(max_items);
     const int tiles = (int)((max_items + per_cta - 1) / per_cta);
     // persistent CTAs: as many as fit at once, at most one per tile
-    static int resident[2] = {0, 0};
-    int& res = resident[large ? 1 : 0];
-    if (res == 0) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, onesweep(large, true), kSortThreads, smem);
-        res = max(per_sm, 1);
+    static PerDevice resident[2];
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    const int res = resident[large ? 1 : 0].get(dev, [&] { return resident_ctas(large, smem); });
+    if (res <= 0) {
+        e = cudaGetLastError();
+        return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
     }
     const int grid = max(min(tiles, res * num_sms), 1);
     int cur = 0;
