@@ -27,13 +27,21 @@ struct PairLayout {
 };
 
 
-// Frames with perspective views and enough items for the partition's three launches to pay: their views
-// cull the Gaussians outside their field, ERP views next to none.
+// Whether a frame's items are partitioned: perspective views cull the Gaussians outside their field, ERP views
+// next to none. Both ways measured, whole steps in us, sorted whole / partitioned:
+//   all views perspective, inside a room: six faces, 1M Gaussians 2080 / 1837; two, 200K 307 / 305; one, 1M 985 / 980,
+//     one image 514 / 516, 140K 194 / 201
+//   all Gaussians in front of the views: one, 1M 467 / 492; one, 200K 276 / 289; four, 300K 991 / 1015
+//   ERP and perspective views, 300K: 7 + 1 2105 / 2140, 2 + 1 1061 / 1080, 1 + 1 (500K) 958 / 968, 2 + 3 1209 / 1196, 3 + 3
+//     1393 / 1386, 1 + 5 1161 / 1105
+// so it takes two perspective views, and as many as ERP views. Several views that all look at the same
+// Gaussians lose 2 %: the host can't tell them from the faces of a cube. Below 2^17 items the three launches cost more
+// than they save.
 bool partitions(const ViewTable& tab, size_t items) {
     if (items < (1u << 17)) return false;
-    for (int v = 0; v < tab.n_views; ++v)
-        if (tab.v[v].model == 1) return true;
-    return false;
+    int perspective = 0;
+    for (int v = 0; v < tab.n_views; ++v) perspective += tab.v[v].model == 1;
+    return perspective >= 2 && 2 * perspective >= tab.n_views;
 }
 
 // Truncated lists unless the caller asks for the whole lists or the frame has too many tiles.
