@@ -574,10 +574,11 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         b.ranges_zero = reinterpret_cast<uint2*>(w + c->L.ranges);
         b.n_ranges = (uint32_t)c->geo.total_tiles;
     }
-    // k_emit clears the tile sort's scratch, and the depth sort's for another odgs_bin_sort of this frame
-    // (the preprocess clears it for the first)
-    const bool emits = c->geo.n_items > 0 && c->pb_cap > 0;
-    if (emits) {
+    // k_emit clears the tile sort's scratch (where it has a look-back region per pass: else the sort clears its one
+    // before every pass), and the depth sort's for another odgs_bin_sort of this frame (the preprocess clears
+    // it for the first)
+    const bool clears = c->geo.n_items > 0 && c->pb_cap > 0 && b.key_passes <= kPairLbRegions;
+    if (clears) {
         b.clear[0] = reinterpret_cast<uint4*>(p + c->P.ctr);
         b.clear_quads[0] = sort_scratch_quads(c->pb_cap, kPairLbRegions);
     }
@@ -591,7 +592,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     int rp = 0;
     if (launch_radix_sort(pk, pv, &hdr->n_pairs_sort, c->pb_cap, c->geo.key_bits, reinterpret_cast<uint32_t*>(p + c->P.hist),
                           reinterpret_cast<uint32_t*>(p + c->P.ctr), reinterpret_cast<uint32_t*>(p + c->P.lb),
-                          &hdr->status, c->num_sms, st, &rp, &c->launches, c->wait_limit, kPairLbRegions, /*cleared=*/emits) != cudaSuccess)
+                          &hdr->status, c->num_sms, st, &rp, &c->launches, c->wait_limit, kPairLbRegions, /*cleared=*/clears) != cudaSuccess)
         return ODGS_ERR_CUDA;
     c->sorted_vals = pv[rp];
     c->pair_buf = rp;
