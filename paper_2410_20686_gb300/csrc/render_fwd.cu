@@ -96,13 +96,16 @@ __global__ void __launch_bounds__(256, PPT <= 2 ? 4 : (PPT == 4 ? 3 : 2)) k_rend
         const int n = (int)(rg.y - rg.x);
 
         float T[PPT], C0[PPT], C1[PPT], C2[PPT];
-        float thr[PPT];  // exponent a blended entry reaches: log2(1/255), +inf once the pixel stopped
+        // exponent a blended entry reaches: log2(1/255), NaN (which none reaches, not even that of an infinite
+        // opacity) once the pixel stopped and below the image
+        const float kNever = __int_as_float(0x7fc00000);
+        float thr[PPT];
         int last[PPT];
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
             T[k] = 1.f; C0[k] = C1[k] = C2[k] = 0.f;
             last[k] = 0;
-            thr[k] = inside ? kLog2AlphaMin : __int_as_float(0x7f800000);
+            thr[k] = inside ? kLog2AlphaMin : kNever;
         }
         for (int b0 = 0; b0 < n; b0 += B) {
             const int cnt = min(B, n - b0);
@@ -159,7 +162,7 @@ __global__ void __launch_bounds__(256, PPT <= 2 ? 4 : (PPT == 4 ? 3 : 2)) k_rend
                         const float alpha = fminf(kAlphaMax, alpha_exp2(pk[k]));
                         const float Tn = __fmul_rn(T[k], __fsub_rn(1.f, alpha));
                         if (Tn < kTMin) {
-                            thr[k] = __int_as_float(0x7f800000);
+                            thr[k] = kNever;
                             evals += (uint32_t)(b0 + j + 1);
                             atomicMax(&s_etile, (uint32_t)(b0 + j + 1));
                             continue;
