@@ -153,12 +153,19 @@ def load(path: str = LIB_PATH):
 
 
 def raw_stream(device) -> C.c_void_p:
-    """The device's current stream as a cudaStream_t. Any other device is refused: its pointers are not the GPU's."""
+    """The (CUDA) device's current stream as a cudaStream_t."""
     import torch
+    k = device.index
+    if k is None:
+        require_cuda(device)
+        k = torch.cuda.current_device()
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(k))
+
+
+def require_cuda(device):
+    """For calls that take tensors as they come: the pointers of any other device are not the GPU's."""
     if device.type != "cuda":
         raise ValueError(f"expected tensors on a CUDA device, not {device}")
-    k = torch.cuda.current_device() if device.index is None else device.index
-    return C.c_void_p(torch._C._cuda_getCurrentRawStream(k))
 
 
 def status_string(st: int) -> str:

@@ -59,6 +59,7 @@ def select(stats: DensifyStats, scales: torch.Tensor, opacity: torch.Tensor,
     params = params or DensifyParams()
     n = stats.grad.numel()
     dev = stats.grad.device
+    L.require_cuda(dev)
     for t in (scales, opacity):
         if t.dtype != torch.float32 or not t.is_contiguous() or t.device != dev:
             raise ValueError("scales and opacity must be contiguous float32 tensors on the statistics' device")
@@ -79,6 +80,7 @@ def apply(means, scales, quats, opacity, sh, action, noise=None, generator=None,
     Synchronizes once to read the count."""
     n = means.shape[0]
     dev = means.device
+    L.require_cuda(dev)
     if noise is None:
         noise = torch.randn((n, 2, 3), device=dev, dtype=torch.float32, generator=generator)
     ins = [means, scales, quats, opacity, sh, noise]

@@ -22,6 +22,7 @@ def _ptr(t):
 
 def l1_dssim(images, targets, lam: float = 0.2, area_weight: bool = True, wrap_u: bool = True, want_grad: bool = True):
     dev = images[0].device
+    L.require_cuda(dev)
     lib = L.load()
     for im, tg in zip(images, targets):
         for t in (im, tg):

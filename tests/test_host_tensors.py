@@ -21,8 +21,13 @@ def _apply():
                    torch.zeros(4, dtype=torch.uint8))
 
 
-@pytest.mark.parametrize("call", [lambda: L.raw_stream(torch.device("cpu")), _loss(0.2), _loss(0.0), _select, _apply],
-                         ids=["stream", "loss", "l1", "select", "apply"])
+def _indexed():
+    x = torch.rand(3, 8, 16, device="cpu:0")
+    return l1_dssim([x], [x])
+
+
+@pytest.mark.parametrize("call", [lambda: L.raw_stream(torch.device("cpu")), _loss(0.2), _loss(0.0), _select, _apply, _indexed],
+                         ids=["stream", "loss", "l1", "select", "apply", "indexed"])
 def test_host_tensors_are_refused(call):
     with pytest.raises(ValueError):
         call()
