@@ -527,7 +527,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
         }
         if (launch_radix_sort(sk, sv, n_sort, c->geo.n_items, 32, hist,
                               reinterpret_cast<uint32_t*>(w + c->L.sort_ctr), reinterpret_cast<uint32_t*>(w + c->L.sort_lb),
-                              &hdr->status, c->num_sms, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions,
+                              &hdr->status, c->num_sms, c->device, st, &rb, &c->launches, c->wait_limit, kDepthLbRegions,
                               /*cleared=*/true, c->partition ? nullptr : &hdr->by_item) != cudaSuccess)
             return ODGS_ERR_CUDA;
         c->depth_buf = c->partition ? 1 : 0;
@@ -592,7 +592,7 @@ static odgs_status run_bin_sort(odgs_ctx* c, cudaStream_t st, bool rebuild = fal
     int rp = 0;
     if (launch_radix_sort(pk, pv, &hdr->n_pairs_sort, c->pb_cap, c->geo.key_bits, reinterpret_cast<uint32_t*>(p + c->P.hist),
                           reinterpret_cast<uint32_t*>(p + c->P.ctr), reinterpret_cast<uint32_t*>(p + c->P.lb),
-                          &hdr->status, c->num_sms, st, &rp, &c->launches, c->wait_limit, kPairLbRegions, /*cleared=*/clears) != cudaSuccess)
+                          &hdr->status, c->num_sms, c->device, st, &rp, &c->launches, c->wait_limit, kPairLbRegions, /*cleared=*/clears) != cudaSuccess)
         return ODGS_ERR_CUDA;
     c->sorted_vals = pv[rp];
     c->pair_buf = rp;

@@ -211,7 +211,7 @@ size_t radix_lookback_words(size_t max_items);
 constexpr uint32_t kDefaultWaitLimit = 1u << 22;
 cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_ptr, size_t max_items, int bits,
                               uint32_t* hist, uint32_t* tile_ctrs, uint32_t* lookback, uint32_t* status, int num_sms,
-                              cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit,
+                              int device, cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit,
                               int lb_regions = 1,     // look-back regions of radix_lookback_words each
                               bool cleared = false,   // counters and regions are already 0
                               const uint32_t* implied = nullptr);  // device word: 1 if the values are 0, 1, 2, ...

@@ -257,10 +257,11 @@ size_t radix_lookback_words(size_t max_items) {
 // Sorts (k[0], v[0]) by key bits [0, bits); returns the buffer index (0 or 1) that holds the
 // result. hist: the digit counts of all passes, [passes][256], from the kernels that wrote the keys.
 // scratch: tile counters [4] + lookback [radix_lookback_words]. implied: a device word or null; where it is 1,
-// v[0] is not read and the values are 0, 1, 2, ...
+// v[0] is not read and the values are 0, 1, 2, ... device: the current one (asked for in every sort, it cost an eager
+// frame 6 us of host time and more).
 cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_ptr, size_t max_items, int bits,
                               uint32_t* hist, uint32_t* tile_ctrs, uint32_t* lookback, uint32_t* status, int num_sms,
-                              cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit, int lb_regions,
+                              int device, cudaStream_t st, int* result_buf, int* launches, uint32_t wait_limit, int lb_regions,
                               bool cleared, const uint32_t* implied) {
     const int passes = radix_passes(bits);
     *result_buf = 0;
@@ -278,9 +279,7 @@ cudaError_t launch_radix_sort(uint32_t* k[2], uint32_t* v[2], const uint32_t* n_
     const int tiles = (int)((max_items + per_cta - 1) / per_cta);
     // persistent CTAs: as many as fit at once, at most one per tile
     static PerDevice resident[2];
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    const int res = resident[large ? 1 : 0].get(dev, [&] { return resident_ctas(large, smem); });
+    const int res = resident[large ? 1 : 0].get(device, [&] { return resident_ctas(large, smem); });
     if (res <= 0) {
         e = cudaGetLastError();
         return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;

@@ -144,7 +144,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
     a.hdr = hdr;
     if (launch_preprocess(a, st.sh_degree, strm) != cudaSuccess) return ODGS_ERR_CUDA;
     int rb = 0;
-    if (launch_radix_sort(dk, dv, &hdr->n_items, n, 32, d_hist, d_ctr, d_lb, &hdr->status, num_sms, strm, &rb,
+    if (launch_radix_sort(dk, dv, &hdr->n_items, n, 32, d_hist, d_ctr, d_lb, &hdr->status, num_sms, dev, strm, &rb,
                           &launches, kDefaultWaitLimit) != cudaSuccess)
         return ODGS_ERR_CUDA;
     BinArgs b{};
@@ -157,7 +157,7 @@ extern "C" odgs_status odgs_render_fwd_static(const odgs_gaussians* g, const odg
     if (launch_binning(b, strm, &launches) != cudaSuccess) return ODGS_ERR_CUDA;
     int rp = 0;
     if (launch_radix_sort(pk, pv, &hdr->n_pairs_sort, cap, key_bits, p_hist, p_ctr, p_lb, &hdr->status, num_sms,
-                          strm, &rp, &launches, kDefaultWaitLimit) != cudaSuccess)
+                          dev, strm, &rp, &launches, kDefaultWaitLimit) != cudaSuccess)
         return ODGS_ERR_CUDA;
     if (launch_tile_ranges(pk[rp], hdr, ranges, tiles, cap, num_sms, strm, &launches) != cudaSuccess)
         return ODGS_ERR_CUDA;
