@@ -44,15 +44,15 @@ class GraphedFrame:
         dev = self.params[0].device
         self.rast = Rasterizer(dev, capacity_mode="query", headroom=headroom)
         self.grads = {k: torch.empty_like(t) for k, t in zip(_GRAD_NAMES, self.params)}
-        # eager run: sizes the workspace and the pair buffer, loads every kernel
+        # eager run: sizes the workspace and the pair buffer
         self._step()
         torch.cuda.synchronize(dev)
         st = self.rast.status()
         if st != 0:
             raise RuntimeError(f"device status {st} during the sizing run")
         self.rast.capacity_mode = "fixed"
-        self.launches = self.rast.launch_count()
-        # warm up on a side stream, then capture
+        # warm up on a side stream (the captured step's kernels: the sizing run of a frame of few pairs keeps whole
+        # lists, so it does not load them all), then capture
         s = torch.cuda.Stream(dev)
         s.wait_stream(torch.cuda.current_stream(dev))
         with torch.cuda.stream(s):
@@ -62,6 +62,7 @@ class GraphedFrame:
         self.graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(self.graph):
             self.loss = self._step()
+        self.launches = self.rast.launch_count()  # of a replay
 
     def _step(self):
         r = self.rast

@@ -169,3 +169,17 @@ def test_binning_captured_after_a_query_takes_any_number_of_pairs():
     g.replay()
     assert r.status() == 0 and r.stats()["pairs_sorted"] <= cap
     assert torch.equal(img, want)
+
+
+def test_launches_of_a_graphed_frame_are_the_replayed_ones():
+    import torch
+    from paper_2410_20686_gb300.graph import GraphedFrame
+    from paper_2410_20686_gb300.rasterizer import Rasterizer, RenderSettings
+    sc = _scene()  # few pairs: the sizing run keeps whole lists, the captured step cuts them
+    p, rs = to_torch(sc), RenderSettings(sh_degree=0)
+    frame = GraphedFrame(p, sc.views, [torch.rand(3, 128, 256, device="cuda")], rs)
+    r = Rasterizer(capacity_mode="fixed")
+    r.reserve_pairs(1 << 17)
+    r.forward(*p, sc.views, rs)
+    r.backward(_upstream(sc.views))
+    assert frame.launches == r.launch_count()
