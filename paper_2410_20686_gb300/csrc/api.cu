@@ -47,8 +47,8 @@ bool partitions(const ViewTable& tab, size_t items) {
 // Truncated lists unless the caller asks for the whole lists or the frame has too many tiles.
 bool truncates(const odgs_settings& s, const Geometry& g) { return !s.full_lists && (uint32_t)g.total_tiles <= kCutMaxTiles; }
 
-// Look-back regions of the two sorts: one per pass, so that one memset clears them (the depth
-// sort's four passes; the tile sort's passes when the tile ids take at most 16 bits).
+// Look-back regions of the two sorts: one per pass, so that they are cleared at once (by k_setup and k_emit: the
+// depth sort's four passes; the tile sort's passes when the tile ids take at most 16 bits).
 constexpr int kDepthLbRegions = 4;
 constexpr int kPairLbRegions = 2;
 
@@ -79,7 +79,7 @@ Layout make_layout(size_t items, const Geometry& g, bool truncate) {
     L.n_last = take(sizeof(uint32_t) * (size_t)g.total_pixels);
     L.acc = take(3 * sizeof(float4) * items);
     L.sort_hist = take(sizeof(uint32_t) * 2 * 4 * 256);  // of all items, of the visible ones
-    // the tile counters kCtrBytes before the look-back regions: one memset clears both
+    // the tile counters kCtrBytes before the look-back regions: cleared together
     L.sort_ctr = take(kCtrBytes + sizeof(uint32_t) * radix_lookback_words(items) * kDepthLbRegions);
     L.sort_lb = L.sort_ctr + kCtrBytes;
     L.big = take(sizeof(uint2) * items);

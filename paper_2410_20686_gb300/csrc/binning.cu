@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(unsigned long long* __rest
 // lane has a tile whatever the items' sizes. Pairs of tiles that do not keep the item's depth bucket
 // are compacted away by a ballot; the kept ones follow one another in the items' order. The kernels wait
 // on memory: the footprint words come in depth order from the count, which gathers them anyway, and the
-// lists are 8 bytes a run, so that six CTAs fit on an SM. Measured (k_emit + k_emit_big, us) against a
+// lists are 8 bytes a run, so that eight CTAs (20.6 KB of shared memory, 32 registers) fit on an SM. Measured (k_emit + k_emit_big, us) against a
 // thread per small item that gathered its word: 3M Gaussians, 8 views of 4096 x 2048, emitted twice
 // 2157 + 1397 -> 1126 + 1160; 500K, 16 views 240 + 26 -> 174 + 18; 1M, six views 105 + 19 -> 82 + 16; 1M, one
 // view 35 + 36 -> 26 + 40; 100K, one view 25 + 16 -> 13 + 14. The words' copy adds 2 to 27 us to the count.

@@ -323,12 +323,6 @@ __device__ __forceinline__ void band_columns(const Footprint& f, int J0, int J1,
     count = n;
 }
 
-// Offset from the Gaussian centre to the pixel centre (fi, fj are the integer pixel indices).
-__device__ __forceinline__ void pixel_offset(float fi, float fj, float fc, float4 pos, float& dx, float& dy) {
-    dx = __fsub_rn(__fsub_rn(fi, fc), pos.z);
-    dy = __fsub_rn(__fsub_rn(fj, pos.y), pos.w);
-}
-
 // 2^p by the hardware's base-2 exponential (PTX ex2.approx.ftz.f32: relative error below 2^-22;
 // the blend evaluates it only for p >= log2(1/255), so no result is subnormal). Forward and
 // backward both use it, so they compute the same alpha.

@@ -19,7 +19,7 @@ __global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr
                         uint4* clear, size_t clear_quads, bool partition) {
     int gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid < tab.n_views) views[gid] = tab.v[gid];
-    // the depth sort's digit histograms, counted by k_preprocess_geom
+    // the depth sort's digit histograms, counted by k_preprocess_color
     for (int i = gid; i < 4 * 256; i += gridDim.x * blockDim.x) dhist[i] = 0u;
     // and its scratch
     for (size_t i = gid; i < clear_quads; i += gridDim.x * blockDim.x) clear[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -39,7 +39,7 @@ __global__ void k_setup(ViewTable tab, ViewDev* views, float4* trig, Header* hdr
         hdr->n_big = 0u;
         hdr->n_huge = 0u;
         hdr->by_item = partition ? 1u : 0u;
-        hdr->n_count_big = 0u;  // the binning's queue counters (each binning leaves them at 0)
+        hdr->n_count_big = 0u;  // (and each scan leaves the binning's queue counters at 0)
     }
     for (int e = gid; e < total_trig; e += gridDim.x * blockDim.x) {
         // locate the view and whether e is a column or a row entry
@@ -198,8 +198,6 @@ __device__ __forceinline__ Cov2 cov2d(const float TM[6], float delta) {
     c.det = det0 + delta * (c.A0 + c.C0) + delta * delta;
     return c;
 }
-
-__device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 template <int DEG>
 __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int stride, int g, float c[16][3]) {

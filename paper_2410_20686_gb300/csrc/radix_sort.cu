@@ -23,7 +23,9 @@ namespace odgs {
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItemsMax = 16;  // 4096 keys per CTA for sorts of at least kLargeSort keys, else 2048
-constexpr size_t kLargeSort = 1u << 20;  // 1M items by depth, one look-back word at a time: 78 us with 2048-key tiles, 82 with 4096
+// Whole steps of 600K, 800K and 1M Gaussians (a depth sort of as many items) with the line here and at 2^19:
+// 923 / 924, 1066 / 1069 and 1142 / 1146 us; 270K in two views 843 / 848
+constexpr size_t kLargeSort = 1u << 20;
 constexpr int kRadix = 256;
 constexpr uint32_t kFlagAgg = 1u << 30;
 constexpr uint32_t kFlagPrefix = 2u << 30;
@@ -215,8 +217,8 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const uint32_t* __
             }
         }
         if ((n + per_cta - 1) / per_cta <= gridDim.x) break;
-        // the next tile's first barrier orders these reads of s_keys, s_vals and s_base before
-        // its writes; s_tile and s_cell are not read here
+        // the next tile's first barrier orders these reads of s_keys, s_vals and s_base before its writes. s_tile,
+        // s_mask and s_cnt, which it writes before that barrier, are last read before the one above
     }
 }
 

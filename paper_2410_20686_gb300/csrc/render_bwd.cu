@@ -1,7 +1,7 @@
 // Backward alpha blending (reverse of Eq. 3) on ERP tiles (sm_103a).
 //
 // Same persistent (view, tile) schedule and layout as the forward kernel: PPT pixels of one row per
-// thread, tile_w / PPT columns apart.
+// thread, as many columns apart as lanes hold a row of the warp's rectangle (four, or all of the tile's row).
 // Each pixel starts from its final transmittance and the index after its last blended Gaussian,
 // and walks its tile list back to front, recovering T_j = T_{j+1} / (1 - alpha_j). Per blended
 // Gaussian it forms

@@ -17,7 +17,7 @@
 // and gamma dy^2 + log2 o) and the shared-memory loads are paid once per thread and entry, not once
 // per pixel; per pixel the exponent is (a t) t + row term with t the offset from the slice centre.
 // A pixel stops before the Gaussian that would take its transmittance below 1e-4; a thread stops
-// when its pixels have; the tile stops when all threads have (__syncthreads_count).
+// when its pixels have; the tile stops when all threads have (__syncthreads_or).
 //
 // Per pixel the result depends only on the pixel, the Gaussians' records and their global
 // order, never on the tile shape, the batch size or PPT: the offset to a Gaussian is formed from
