@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(32) k_ssim_bwd(LossArgs a) {
 // whose 700 MB take 103 us. Up to 8192 CTAs, mostly one per step: a CTA's loads end with its row, so the next row's
 // have to be another CTA's. With as many as are resident (1216), each taking several rows, 16384 x 4096
 // takes 379 us instead of 350 (2432: 365; 4864: 354), 8 views of 4096 x 2048 376 instead of 350 and one 53.8 instead of 51.4.
+// Frames of few or narrow rows take 1216: a CTA per row of six views of 208 x 208 costs it and the reduction 13.7 -> 16.4 us.
 constexpr int kL1Views = 64;
 struct L1View {
     const float* x;
@@ -436,7 +437,8 @@ __global__ void __launch_bounds__(kThreads) k_loss_reduce(const float* __restric
 }
 
 constexpr int kSms = 152;  // GB300
-constexpr int kL1Blocks = 8192;  // at most, of the L1 pass alone
+constexpr int kL1Blocks = 8192, kL1Few = 8 * kSms;  // CTAs of the L1 pass alone
+constexpr int kL1Values = 2048;                     // it is worth one for
 
 // 1 over the sum of an image's pixel weights; the sum over j of sin(pi (j + 1/2) / H) is 1 / sin(pi / (2 H))
 float inv_weight_sum(int W, int H, int area) {
@@ -498,6 +500,7 @@ extern "C" odgs_status odgs_loss_l1(const float* const* images, const float* con
         const bool first = k == 0;
         L1Args a{};
         a.partial = static_cast<float*>(scratch);
+        long long values = 0;
         for (; k < n_views && a.views < kL1Views && (a.views == 0 || heights[k] <= (INT_MAX - a.rows) / 3); ++k) {
             L1View& v = a.v[a.views++];
             v.x = images[k];
@@ -509,8 +512,9 @@ extern "C" odgs_status odgs_loss_l1(const float* const* images, const float* con
             v.inv_wsum = inv_weight_sum(v.W, v.H, v.area);
             v.row0 = a.rows;
             a.rows += 3 * v.H;
+            values += 3ll * v.W * v.H;
         }
-        const int blocks = std::min(a.rows, kL1Blocks);
+        const int blocks = (int)std::min<long long>(a.rows, std::clamp<long long>(values / kL1Values, kL1Few, kL1Blocks));
         k_l1<<<blocks, kThreads, 0, st>>>(a);
         k_loss_reduce<<<1, kThreads, 0, st>>>(a.partial, blocks, loss, (p->accumulate || !first) ? 1 : 0);
     }
