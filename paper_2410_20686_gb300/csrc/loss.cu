@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(kThreads) k_loss_reduce(const float* __restric
 }
 
 constexpr int kSms = 152;  // GB300
-constexpr int kL1Blocks = 8192, kL1Few = 8 * kSms;  // CTAs of the L1 pass alone
+constexpr int kL1Blocks = 8192, kL1Few = 8 * kSms;  // CTAs of the L1 pass alone, as far as the scratch holds their sums
 constexpr int kL1Values = 2048;                     // it is worth one for
 
 // 1 over the sum of an image's pixel weights; the sum over j of sin(pi (j + 1/2) / H) is 1 / sin(pi / (2 H))
@@ -475,7 +475,7 @@ Plan make_plan(int W, int H) {
 size_t maps_bytes(const Plan& p, int H) { return (9 * (size_t)p.pitch * H * sizeof(float) + 15) & ~(size_t)15; }
 size_t scratch_for(int W, int H) {
     const Plan p = make_plan(W, H);
-    return maps_bytes(p, H) + (size_t)std::max(p.warps(), kL1Blocks) * sizeof(float);
+    return maps_bytes(p, H) + (size_t)std::max(p.warps(), kL1Few) * sizeof(float);
 }
 
 }  // namespace
@@ -493,9 +493,10 @@ extern "C" odgs_status odgs_loss_l1(const float* const* images, const float* con
     for (int k = 0; k < n_views; ++k)
         if (!images[k] || !targets[k] || widths[k] < 1 || heights[k] < 1 || heights[k] > INT_MAX / 3)
             return ODGS_ERR_INVALID_ARG;
-    if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 15u) || scratch_bytes < kL1Blocks * sizeof(float))
+    if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 15u) || scratch_bytes < kL1Few * sizeof(float))
         return ODGS_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const int most = (int)std::min<size_t>(kL1Blocks, scratch_bytes / sizeof(float));
     for (int k = 0; k < n_views;) {
         const bool first = k == 0;
         L1Args a{};
@@ -514,7 +515,7 @@ extern "C" odgs_status odgs_loss_l1(const float* const* images, const float* con
             a.rows += 3 * v.H;
             values += 3ll * v.W * v.H;
         }
-        const int blocks = (int)std::min<long long>(a.rows, std::clamp<long long>(values / kL1Values, kL1Few, kL1Blocks));
+        const int blocks = (int)std::min<long long>(a.rows, std::clamp<long long>(values / kL1Values, kL1Few, most));
         k_l1<<<blocks, kThreads, 0, st>>>(a);
         k_loss_reduce<<<1, kThreads, 0, st>>>(a.partial, blocks, loss, (p->accumulate || !first) ? 1 : 0);
     }
